@@ -13,6 +13,7 @@
 
 #include "../../include/rasp.h"
 #include "engine.cuh"
+#include "fuse.cuh"
 #include "internal.h"
 
 using namespace rasp;
@@ -82,7 +83,7 @@ struct BucketPlan {
 struct Layout {
   size_t off_i, off_a, off_steps, off_cap, off_status, off_uhead, off_ylen, off_n, off_memoff;
   size_t off_mem, off_prog, off_progoff, off_progvm, off_tape, off_y, off_ids, off_heads, off_err,
-      off_hist, off_stats, off_dirty, off_pvoff, off_pvids, off_thist, off_ids2, off_rcount, off_topk;
+      off_hist, off_stats, off_dirty, off_pvoff, off_pvids, off_thist, off_ids2, off_rcount, off_topk, off_frec;
   size_t total;
 };
 
@@ -135,7 +136,8 @@ struct rasp_batch {
   uint32_t* d_pvids = nullptr;
   uint32_t num_programs = 0;
   uint32_t max_plen = 0;
-  bool dirty_valid = false;    // codedirty is up to date (only the shared kernel tracks it)
+  bool dirty_valid = false;    // codedirty is up to date for the VMs of the schedules that keep it
+  bool ran_untracked = false;  // since the last pack a schedule ran that does not keep codedirty
   bool code_lazy = false;      // slabs of VMs with codedirty = 0 lack their program words (lazy pack)
   bool tuned_block = false;    // autotuned: the SMEM-staged schedule one step at a time
   bool narrow = false;         // M in 4-byte words (w <= 32)
@@ -227,6 +229,7 @@ Layout make_layout(uint64_t V, uint64_t mem_words, uint32_t ellp, uint32_t sp, u
   L.off_ids2 = take(4 * V);                             // compacted queue between budget rounds
   L.off_rcount = take(4 * kNumBuckets);                 // its length, per launch group
   L.off_topk = take(sizeof(TopCand) * (topk_blocks(V) + 1) * kMaxTopK);  // top-k candidates, result
+  L.off_frec = take(16 * fuse_records(mem_words, V));  // records of the fused entries
   L.total = o;
   return L;
 }
@@ -390,6 +393,29 @@ cudaError_t ensure_prog64(rasp_batch* b, cudaStream_t st) {
   return launch_widen(b->prog32, b->d_prog, b->prog_words, st);
 }
 
+// Whether a launch group keeps codedirty: the shared-program schedule, and
+// the HBM-slab epoch loop when the programs have fused entries.
+bool tracks_code(const rasp_batch* b, const Group& g) {
+  if (g.sched == RASP_SCHED_SHARED) return true;
+  const StepVariant v = variant_of(b);
+  return g.sched == RASP_SCHED_PERSIST_GL && b->S.fops && !v.checked && !v.hist && !v.vote && !v.block;
+}
+
+// Before a run (eagerly, outside any captured graph): where codedirty is not
+// up to date -- another schedule may have written program words, and the plan
+// has changed since -- every VM runs from its memory until the next pack.
+cudaError_t settle_dirty(rasp_batch* b, cudaStream_t st) {
+  bool tracked = false, untracked = false;
+  for (const Group& g : b->groups) (tracks_code(b, g) ? tracked : untracked) = true;
+  cudaError_t e = cudaSuccess;
+  if (tracked && !b->dirty_valid) {
+    e = cudaMemsetAsync(b->S.codedirty, 1, b->V, st);
+    b->dirty_valid = true;
+  }
+  b->ran_untracked = b->ran_untracked || untracked;
+  return e;
+}
+
 // Before anything but the shared-program kernel reads the slabs of a lazily
 // packed batch: the program words of every VM whose slab lacks them.
 cudaError_t materialize(rasp_batch* b, cudaStream_t st) {
@@ -411,6 +437,7 @@ cudaError_t apply_uhead_reset(rasp_batch* b, cudaStream_t st) {
 }
 
 int replan(rasp_batch* b);
+void drop_graphs(rasp_batch* b);
 
 int check_device_error(rasp_batch* b) {
   int err = 0;
@@ -628,6 +655,32 @@ int rasp_load_programs_i32(rasp_batch* b, const int32_t* words, const uint64_t* 
 
 }  // extern "C"
 
+namespace {
+
+// Whether the fused entries may read program words as data: not where the
+// shared-program schedule packs memories without them.
+bool owns_code(const rasp_batch* b) {
+  return !b->shared_programs && (b->cfg.flags & RASP_SCHED_MASK) != RASP_SCHED_SHARED;
+}
+
+// The place of the fused entries (at most 16 bytes per instruction, 8 per
+// program word; as much of the M arena is scratch while they are made, before
+// the pack) in the part of the program area that the programs leave free: behind
+// the 8-byte words, or behind where they would be widened to -- from the start
+// when nothing widens them. NULL where there is no room (programs that fill
+// more than half of the memories), where no kernel would run from them, or
+// where a program has more instructions than an entry can name.
+uint4* place_fused(const rasp_batch* b, uint64_t total, bool keep32) {
+  const StepVariant v = variant_of(b);
+  if (!total || v.checked || v.hist || v.vote || v.block || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
+  const uint64_t lo = keep32 && owns_code(b) ? 0 : 8ull * total;
+  const uint64_t end = keep32 ? 4ull * ((b->mem_words + 1ull) & ~1ull) : 8ull * b->mem_words;
+  if (lo + 8ull * total > end || 8ull * total > (b->narrow ? 4ull : 8ull) * b->mem_words) return nullptr;
+  return reinterpret_cast<uint4*>(reinterpret_cast<char*>(b->d_prog) + lo);
+}
+
+}  // namespace
+
 // Programs given as 8-byte words are copied into the program area; 4-byte
 // words are copied into the M arena (which the pack overwrites anyway) and
 // widened on the device, with sign extension, once the checks have passed.
@@ -692,6 +745,9 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
     cudaStreamSynchronize(st);   // the caller's buffers are read before the call returns
     return bad;
   }
+  const bool same_args = b->shared_programs == (prog_of_vm != nullptr) && b->max_plen == max_plen &&
+                         b->num_programs == (uint32_t)num_programs;
+  const uint4* fops_before = b->S.fops;
   b->shared_programs = prog_of_vm != nullptr;
   b->max_plen = max_plen;
   b->num_programs = (uint32_t)num_programs;
@@ -712,12 +768,30 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
     CK(cudaStreamSynchronize(st));
   }
   CK(cudaStreamSynchronize(st));   // the caller's buffers are read before the call returns
+  // fused entries: their place, and the smallest memory that runs each program
+  const uint32_t* bound = b->S.n;
+  b->S.fops = place_fused(b, total, keep32);
+  b->S.frec = (const uint4*)(b->base + b->L.off_frec);
+  b->S.prog_off = b->d_progoff;
+  b->S.prog_of_vm = b->shared_programs ? b->d_progvm : nullptr;
+  if (b->S.fops && prog_of_vm) {
+    std::vector<uint32_t> least(num_programs, 1u << 31);
+    for (uint32_t v = 0; v < b->V; ++v) least[prog_of_vm[v]] = std::min(least[prog_of_vm[v]], b->h_n[v]);
+    CK(cudaMemcpyAsync(b->d_ids2, least.data(), 4 * num_programs, cudaMemcpyHostToDevice, st));
+    CK(cudaStreamSynchronize(st));
+    bound = b->d_ids2;
+  }
+  if (!same_args || b->S.fops != fops_before) drop_graphs(b);   // captured runs hold the old launch arguments
   // widening, like the pack, is left queued on the stream: it may have to
   // wait for SMs that another batch's run holds, and the host need not
   b->prog32 = keep32 && total ? staged : nullptr;
   b->prog_words = total;
   b->prog64_valid = !b->prog32;
   if (word_size == 4 && total && !keep32) CK(launch_widen(staged, b->d_prog, total, st));
+  if (b->S.fops)
+    CK(launch_fuse(b->d_prog, b->prog32, b->d_progoff, bound, b->num_programs, b->wmask, variant_of(b).classic,
+                   owns_code(b), reinterpret_cast<uint4*>(b->S.mem), const_cast<uint4*>(b->S.fops),
+                   const_cast<uint4*>(b->S.frec), st));
   CK(fill_bytes(b->d_hist, 0, 8 * 10, st));
   b->code_lazy = pack_lazy(b);
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,
@@ -725,6 +799,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   b->uhead_pending = false;        // the pack resets u_0
   b->programs_loaded = true;
   b->dirty_valid = true;
+  b->ran_untracked = false;
   g_err.clear();
   return RASP_OK;
 }
@@ -801,6 +876,7 @@ int rasp_reset(rasp_batch* b) {
                  b->wmask, b->sp, b->code_lazy, b->stream));
   b->uhead_pending = false;
   b->dirty_valid = true;
+  b->ran_untracked = false;
   return RASP_OK;
 }
 
@@ -847,24 +923,15 @@ int enqueue_run(rasp_batch* b, cudaStream_t st, uint64_t max_steps) {
       launches++;
     }
     if (g.sched == RASP_SCHED_SHARED) {
-      if (!b->dirty_valid) {
-        // another schedule ran since c_0 and did not track code writes: every
-        // VM fetches from its own slab until the next reset
-        CK(cudaMemsetAsync(b->S.codedirty, 1, b->V, st));
-        b->dirty_valid = true;
-      }
       CK(ensure_prog64(b, st));
       CK(launch_shared(var, b->S, P, b->d_prog, b->d_progoff, b->d_pvoff, b->d_pvids, b->num_programs,
                        b->max_plen, b->cfg.epoch, st));
     } else if (g.sched == RASP_SCHED_PLAIN) {
-      b->dirty_valid = false;
       CK(launch_plain(var, b->S, P, ids, g.count, st));
     } else if (g.sched == RASP_SCHED_PERSIST) {
-      b->dirty_valid = false;
       Queue Q{ids, g.count, b->d_heads + k, b->d_heads + kNumBuckets + k, 0, nullptr};
       CK(launch_persist(var, b->S, P, Q, g.shape, st));
     } else {
-      b->dirty_valid = false;
       std::vector<uint64_t> budgets;
       const uint64_t limit = std::min(max_steps, b->max_cap);
       const uint64_t lanes = (uint64_t)g.shape.grid * g.shape.warps * 32u;
@@ -914,6 +981,7 @@ int rasp_run(rasp_batch* b, uint64_t max_steps) {
   }
   // 8-byte program words for the kernels that read them, eagerly (outside any captured graph)
   if (b->code_lazy || (b->cfg.flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED) CK(ensure_prog64(b, b->stream));
+  CK(settle_dirty(b, b->stream));
   if (!b->cap_stream) return enqueue_run(b, b->stream, max_steps);
   // CUDA graph: capture the run once per budget on a private stream, replay it on the batch stream
   cudaGraphExec_t exec = nullptr;
@@ -1147,6 +1215,7 @@ void drop_graphs(rasp_batch* b) {
 int replan(rasp_batch* b) {
   plan_buckets(b);
   build_groups(b);
+  if (b->ran_untracked) b->dirty_valid = false;   // VMs may move to a schedule that keeps codedirty
   drop_graphs(b);
   return b->inputs_loaded ? order_ids(b) : RASP_OK;
 }
@@ -1168,7 +1237,7 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
   // mutable state: i, a, steps | status, uhead, ylen | M | y | counters
   const size_t spans[][2] = {{L.off_i, L.off_cap}, {L.off_status, L.off_n}, {L.off_mem, L.off_prog},
                              {L.off_y, L.off_ids}, {L.off_hist, L.off_stats}, {L.off_dirty, L.off_dirty + b->V}};
-  const bool dirty_valid0 = b->dirty_valid, code_lazy0 = b->code_lazy;
+  const bool dirty_valid0 = b->dirty_valid, code_lazy0 = b->code_lazy, untracked0 = b->ran_untracked;
   size_t total = 0;
   for (auto& sp : spans) total += sp[1] - sp[0];
   char* snap = nullptr;
@@ -1224,6 +1293,8 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
       ce = copy_state(false);
       b->dirty_valid = dirty_valid0;
       b->code_lazy = code_lazy0;
+      b->ran_untracked = untracked0;
+      if (ce == cudaSuccess) ce = settle_dirty(b, st);
       if (ce != cudaSuccess) break;
       cudaEventRecord(e0, st);
       r2 = enqueue_run(b, st, max_steps);
@@ -1319,6 +1390,7 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
   const cudaError_t ce2 = copy_state(false);
   b->dirty_valid = dirty_valid0;
   b->code_lazy = code_lazy0;
+  b->ran_untracked = untracked0;
   cudaStreamSynchronize(st);
   cudaFree(snap);
   cudaEventDestroy(e0);

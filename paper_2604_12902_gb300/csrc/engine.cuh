@@ -41,6 +41,10 @@ struct DevState {
   const uint64_t* tape;       // u_1..u_l, stride ellp words per VM
   uint64_t* y;                // y_1..y_s, stride sp words per VM
   uint8_t* codedirty;         // 1 if the VM may have written into its program words (NULL: untracked)
+  const uint4* fops;          // fused entries of the programs (fuse.cuh; NULL: none)
+  const uint4* frec;          // masks of the instructions that have one
+  const uint64_t* prog_off;   // word offset of each program
+  const uint32_t* prog_of_vm; // program of each VM (NULL: program v)
 };
 
 struct Params {

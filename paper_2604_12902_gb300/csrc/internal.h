@@ -21,6 +21,7 @@ struct StepVariant {
   bool block;    // HBM-slab persistent: one predicated block per step instead of the epoch loop;
                  // shared-program schedule: one step at a time per lane instead of the epoch loop
   bool narrow;   // M in 4-byte words (w <= 32): plain and HBM-slab persistent schedules
+  bool fuse;     // HBM-slab epoch loop: the programs have fused entries
 };
 
 // Persistent-kernel launch shape for one bucket of VMs.
@@ -45,6 +46,14 @@ struct PersistShape {
 cudaError_t launch_pack(const DevState& S, const uint64_t* prog, const int32_t* prog32, const uint64_t* prog_off,
                         const uint32_t* prog_of_vm, uint32_t num_vms, uint64_t wmask, uint32_t sp,
                         bool lazy, cudaStream_t stream);
+
+// The fused entries of every program (fuse.cuh), at half the program's word
+// offset in `out`, and their records. bound[p]: the smallest n among the VMs of
+// program p; own: the VMs' memories hold the program words; tmp: scratch of
+// 16 bytes per instruction.
+cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint64_t* prog_off, const uint32_t* bound,
+                        uint32_t num_programs, uint64_t wmask, bool classic, bool own, uint4* tmp, uint4* out,
+                        uint4* recs, cudaStream_t stream);
 
 // Shared-program schedule: one CTA per program (program in shared memory),
 // lanes run the program's VMs pv_ids[pv_off[p] .. pv_off[p+1]) (epoch loop

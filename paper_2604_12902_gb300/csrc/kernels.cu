@@ -19,6 +19,7 @@
 #include <cstdio>
 
 #include "engine.cuh"
+#include "fuse.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -117,6 +118,89 @@ __global__ void __launch_bounds__(256) k_pack(DevState S, const W* __restrict__ 
           w.y = 0ull;
         }
         *reinterpret_cast<ulonglong2*>(dst + k) = w;
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------------ fuse
+// The fused entries of every program (fuse.cuh), one program per lane: the
+// entries reached from instruction 0 are decoded one after the other (an
+// entry names the next ones), kept by instruction in `tmp`, and then written
+// densely with their jumps renumbered. A lane reads only the instructions
+// that runs start at, about 1.1 times each: 1M template programs in 0.3 ms,
+// against 2.6 ms with one instruction per lane (7 of 32 lanes active, every
+// run of every instruction decoded).
+// bound: the smallest memory that runs program p. tmp: 16 bytes per
+// instruction (at half the program's offset).
+template <class W>
+__global__ void __launch_bounds__(128) k_fuse(const W* __restrict__ prog, const uint64_t* __restrict__ prog_off,
+                                              const uint32_t* __restrict__ bound, uint32_t num_programs,
+                                              uint64_t wmask, uint32_t classic, uint32_t own, uint4* tmp,
+                                              uint4* __restrict__ out, uint4* recs) {
+  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < num_programs; p += gridDim.x * blockDim.x) {
+    const uint64_t po = prog_off[p];
+    const uint32_t plen = (uint32_t)(prog_off[p + 1] - po), n = bound[p];
+    const uint32_t ilim = wmask >= (uint64_t)n - 1u ? n : (uint32_t)(wmask + 1ull);
+    const uint32_t mok = min(plen, ilim) >> 1;
+    uint4* t = tmp + (po >> 1);
+    uint4* rec = recs + (po >> 7) + p;
+    const uint32_t nrec = (plen + 127u) / 128u;
+    for (uint32_t k = 0; k < nrec; ++k) rec[k] = make_uint4(k == 0u && mok ? 1u : 0u, 0u, 0u, 0u);
+    uint32_t entries = 0, writes = 0;                    // reached, and of them writes into the program
+    // records in order; a target before the current record starts over from there
+    for (uint32_t k = 0; k < nrec;) {
+      uint32_t back = ~0u;
+      uint4 r = rec[k];
+      uint64_t want = fuse_mask(r), done = ((uint64_t)r.w << 32) | r.z;
+      while (want & ~done) {
+        const uint32_t e = 64u * k + (uint32_t)__ffsll((long long)(want & ~done)) - 1u;
+        done |= 1ull << (e & 63u);
+        const uint4 x = fuse_one(prog + po, e, plen, n, mok, wmask, classic != 0u, own != 0u);
+        t[e] = x;
+        entries += 1u;
+        uint32_t next[2] = {x.w >> 16, x.w & 0xFFFFu};
+        if (!(x.y & FO_COUNT)) {                         // a stall: where its instruction may go on
+          const ulonglong2 oj = fuse_pair(prog + po, 2u * e, wmask);
+          const bool valid = oj.x - 1ull < 7ull;
+          writes += (oj.x == 4ull || oj.x == 6ull) && oj.y < (uint64_t)plen ? 1u : 0u;
+          next[0] = valid && e + 1u < mok ? e + 1u : e;
+          next[1] = oj.x == 5ull && !(oj.y & 1ull) && (oj.y >> 1) < (uint64_t)mok ? (uint32_t)(oj.y >> 1) : e;
+        }
+        for (uint32_t q = 0; q < 2u; ++q) {
+          const uint32_t kk = next[q] >> 6;
+          const uint64_t bit = 1ull << (next[q] & 63u);
+          if (kk == k) {
+            want |= bit;
+          } else {
+            const uint4 o = rec[kk];
+            if (!(fuse_mask(o) & bit)) {
+              rec[kk] = make_uint4(o.x | (uint32_t)bit, o.y | (uint32_t)(bit >> 32), o.z, o.w);
+              if (kk < k) back = min(back, kk);
+            }
+          }
+        }
+      }
+      rec[k] = make_uint4((uint32_t)want, (uint32_t)(want >> 32), (uint32_t)done, (uint32_t)(done >> 32));
+      k = back < k ? back : k + 1u;
+    }
+    uint32_t count = 0;
+    for (uint32_t k = 0; k < nrec; ++k) {
+      const uint4 r = rec[k];
+      rec[k] = make_uint4(r.x, r.y, count, 0u);
+      count += (uint32_t)__popcll(fuse_mask(r));
+    }
+    // a program one eighth of whose entries are writes into itself would leave
+    // them after a few steps
+    if (8u * writes >= entries && writes) t[0] = make_uint4(0u, FO_MEM, 0u, 0u);
+    uint4* dst = out + (po >> 1);
+    for (uint32_t k = 0; k < nrec; ++k) {
+      for (uint64_t m = fuse_mask(rec[k]); m; m &= m - 1ull) {
+        const uint32_t e = 64u * k + (uint32_t)__ffsll((long long)m) - 1u;
+        uint4 x = t[e];
+        const uint32_t a = x.w & 0xFFFFu, f = x.w >> 16;
+        x.w = fuse_rank(rec[a >> 6], a) | (fuse_rank(rec[f >> 6], f) << 16);
+        *dst++ = x;
       }
     }
   }
@@ -356,6 +440,81 @@ __device__ __forceinline__ void run_epoch_loop(Mem M, const uint64_t* T, uint64_
   }
 }
 
+// About `epoch` VM-steps of every active lane (epoch / 2 entries of the lanes
+// that run from them, then `epoch` steps one instruction at a time for the
+// rest; half as many entries measured 9 % slower on 1M template programs:
+// every return to the scheduler waits for the next VM's state). Lanes that stall wait in place until `wait` of them
+// have (or none runs on), then take general steps together until they can
+// enter their entries again or stop. A VM that leaves its entries for good --
+// it wrote into its program, or its i lies outside them for a few steps --
+// runs from its memory (run_epoch_loop, which does not watch its writes) until
+// the next pack.
+constexpr uint32_t kFuseChunk = 8;     // entries between two looks at the stalled lanes
+constexpr uint32_t kFuseOutside = 32;  // general steps at no entry's start before a VM leaves them: more than an
+                                       // entry holds (a run that a stop has cut goes on inside an entry)
+
+template <bool MASKED, bool CLASSIC, class Mem>
+__device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64_t* Y, const Params& P, Regs& r,
+                                                Fused& F, const DevState& S, uint32_t vm, Hist& h, bool& active,
+                                                uint32_t& final_st, uint32_t epoch, uint32_t idle_exit) {
+  const uint32_t fm = __ballot_sync(FULL, active && F.on);
+  bool stall = active && r.clean && !F.on;               // a stop has cut the run of an entry: on to the next one
+  if (fm) {
+    const uint32_t wait = idle_exit ? idle_exit : 8u;
+    const uint32_t zero = P.ellp & 1u;                   // the stride of the tapes is even
+    for (uint32_t it = (epoch + 1u) / 2u; it;) {
+      const uint32_t c = min(it, kFuseChunk);
+      it -= c;
+      if (active && F.on) {
+        if constexpr (std::is_same<Mem, NarrowView>::value) {
+          uint32_t a32 = (uint32_t)r.a;
+          const uint32_t wm32 = (uint32_t)P.wmask;
+          if (wm32 == 0xFFFFFFFFu)
+            fused_loop_ptx_narrow<false, CLASSIC>(M.M, T, Y, P.ell, P.s, wm32, fm, c, zero, a32, F, r.left, r.u0, r.y0);
+          else
+            fused_loop_ptx_narrow<true, CLASSIC>(M.M, T, Y, P.ell, P.s, wm32, fm, c, zero, a32, F, r.left, r.u0, r.y0);
+          r.a = a32;
+        } else {
+          fused_loop_ptx<MASKED, CLASSIC>(M, T, Y, P.ell, P.s, P.wmask, fm, c, zero, r.a, F, r.left, r.u0, r.y0);
+        }
+        stall = fuse_stalled(F, r, P);
+      }
+      const uint32_t sm = __ballot_sync(FULL, stall && F.on);
+      if (sm == fm || (uint32_t)__popc(sm) >= wait) break;
+    }
+  }
+  if (stall && F.on && (F.op.y & FO_HALT)) {
+    r.ip = 2u * F.op.x;
+    active = false;
+    final_st = ST_HALTED;
+  } else if (stall) {
+    const FuseProg G = fuse_prog(S, vm, r.ilim);
+    CodeView<Mem> V{M, G.plen};
+    if (F.on) r.ip = 2u * (F.op.y & FO_COUNT ? fuse_instr(G, F.cur) : F.op.x);
+    r.have = false;
+    for (uint32_t out = 0; active && stall;) {
+      const uint32_t st = step_general<MASKED, false, false, CLASSIC>(V, T, Y, P, r, h);
+      if (st != CONT) {
+        active = false;
+        final_st = st;
+      } else {
+        fuse_enter(G, F, r);
+        stall = F.on ? fuse_stalled(F, r, P) : r.clean && out++ < kFuseOutside;
+      }
+    }
+    if (active && !F.on) {
+      r.clean = false;
+      prime(M, r);
+    }
+  }
+  if (__any_sync(FULL, active && !F.on)) {
+    bool slow = active && !F.on;
+    const bool was = slow;
+    run_epoch_loop<MASKED, CLASSIC>(M, T, Y, P, r, h, slow, final_st, epoch, idle_exit);
+    if (was) active = slow;
+  }
+}
+
 // ------------------------------------------------------------------ persistent, staged in SMEM
 template <bool MASKED, bool CHECKED, bool HIST, bool VOTE, bool LOOP = false>
 __global__ void __launch_bounds__(256) k_persist(DevState S, Params P, Queue Q, uint32_t ncap,
@@ -480,8 +639,12 @@ __global__ void __launch_bounds__(256) k_persist(DevState S, Params P, Queue Q, 
 // end no VM waits in a busy lane's prefetch slot while other lanes idle.
 enum : uint32_t { PF_EMPTY = 0, PF_ID = 1, PF_REGS = 2, PF_NONE = 3 };   // PF_REGS: entries warmed in L2
 
+//
+// FUSE: the programs have fused entries. Batches without them keep a kernel of
+// their own: both loops in one kernel spill more, and 1,024 random programs
+// took 333 instead of 319 us a pass.
 template <bool MASKED, bool CHECKED, bool HIST, bool VOTE, bool CLASSIC = false, bool LOOP = false,
-          bool NARROW = false>
+          bool NARROW = false, bool FUSE = false>
 __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Queue Q, uint32_t epoch,
                                                        uint32_t idle_exit) {
   static_assert(!LOOP || (!CHECKED && !HIST && !VOTE), "the epoch loop serves WRAP select steps without counters");
@@ -517,6 +680,7 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
   int32_t vm = -1;
   bool active = false;
   uint32_t final_st = ST_RUNNING;
+  Fused F{};
   std::conditional_t<NARROW, NarrowView, uint64_t*> M{};
   attach_mem(M, S, 0ull);
   const uint64_t* T = S.tape;
@@ -528,6 +692,7 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
     // ---- boundary: retire stopped VMs
     if (vm >= 0 && !active) {
       store_regs(S, (uint32_t)vm, r, final_st);
+      if (FUSE && !r.clean) S.codedirty[vm] = 1;
       vm = -1;
     }
     // swap in the prefetched VM (its loads were issued a boundary ago)
@@ -540,7 +705,8 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
         attach_mem(M, S, moff);
         T = S.tape + (uint64_t)pf_vm * P.ellp;
         Y = S.y + (uint64_t)pf_vm * P.sp;
-        if (!VOTE) prime(M, r);
+        if (FUSE) fuse_attach(S, pf_vm, r, F);
+        if (!VOTE && !F.on) prime(M, r);
         active = true;
       }
       pf = PF_EMPTY;
@@ -556,6 +722,10 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
       asm volatile("prefetch.global.L2 [%0];" :: "l"(S.uhead + pf_vm));
       asm volatile("prefetch.global.L2 [%0];" :: "l"(S.ylen + pf_vm));
       asm volatile("prefetch.global.L2 [%0];" :: "l"(S.mem_off + pf_vm));
+      if (FUSE) {
+        asm volatile("prefetch.global.L2 [%0];" :: "l"(S.codedirty + pf_vm));
+        if (!S.prog_of_vm) asm volatile("prefetch.global.L2 [%0];" :: "l"(S.prog_off + pf_vm));
+      }
       pf = PF_REGS;
     }
     // ---- new queue positions
@@ -620,7 +790,8 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
         attach_mem(M, S, moff);
         T = S.tape + (uint64_t)pf_vm * P.ellp;
         Y = S.y + (uint64_t)pf_vm * P.sp;
-        if (!VOTE) prime(M, r);
+        if (FUSE) fuse_attach(S, pf_vm, r, F);
+        if (!VOTE && !F.on) prime(M, r);
         active = true;
       }
     }
@@ -628,7 +799,9 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
     if (__all_sync(FULL, vm < 0 && pf == PF_NONE)) break;
 
     // ---- run
-    if constexpr (LOOP) run_epoch_loop<MASKED, CLASSIC>(M, T, Y, P, r, h, active, final_st, epoch, idle_exit);
+    if constexpr (FUSE) run_epoch_fused<MASKED, CLASSIC>(M, T, Y, P, r, F, S, (uint32_t)vm, h, active, final_st, epoch,
+                                                            idle_exit);
+    else if constexpr (LOOP) run_epoch_loop<MASKED, CLASSIC>(M, T, Y, P, r, h, active, final_st, epoch, idle_exit);
     else run_epoch<MASKED, CHECKED, HIST, VOTE, true, CLASSIC>(M, T, Y, P, r, h, active, final_st, epoch);
   }
   flush_hist<HIST>(P, h);
@@ -684,6 +857,7 @@ __global__ void __launch_bounds__(128, 6) k_serve(ServeArgs A, Params P0) {
   uint32_t vm = 0;
   bool active = false;
   uint32_t final_st = ST_RUNNING;
+  Fused F{};
   uint64_t* M = nullptr;
   const uint64_t* T = nullptr;
   uint64_t* Y = nullptr;
@@ -748,7 +922,10 @@ __global__ void __launch_bounds__(128, 6) k_serve(ServeArgs A, Params P0) {
             M = sd.S.mem + moff;
             T = sd.S.tape + (uint64_t)v * P.ellp;
             Y = sd.S.y + (uint64_t)v * P.sp;
-            if (!CHECKED) prime(M, r);
+            if (!CHECKED) {
+              fuse_attach(sd.S, v, r, F);
+              if (!F.on) prime(M, r);
+            }
             active = true;
           } else {
             serve_finish(A, sl);                // already stopped: nothing to run
@@ -789,7 +966,8 @@ __global__ void __launch_bounds__(128, 6) k_serve(ServeArgs A, Params P0) {
     if constexpr (CHECKED) {
       run_epoch<MASKED, true, false, false, false, CLASSIC>(M, T, Y, P, r, h, active, final_st, A.epoch);
     } else {
-      run_epoch_loop<MASKED, CLASSIC>(M, T, Y, P, r, h, active, final_st, A.epoch, 0u);
+      run_epoch_fused<MASKED, CLASSIC>(M, T, Y, P, r, F, A.slots[slot < 0 ? 0 : slot].S, vm, h, active, final_st,
+                                       A.epoch, 0u);
     }
   }
   __syncthreads();
@@ -1167,15 +1345,20 @@ GlobalFn global_select(const StepVariant& v) {
   if (v.narrow) {
     if (v.hist) return k_persist_gl<true, false, true, false, CL, false, true>;
     if (v.block) return k_persist_gl<true, false, false, false, CL, false, true>;
-    return k_persist_gl<true, false, false, false, CL, true, true>;
+    return v.fuse ? k_persist_gl<true, false, false, false, CL, true, true, true>
+                  : k_persist_gl<true, false, false, false, CL, true, true>;
   }
   if (v.checked)
     return v.hist ? k_persist_gl<false, true, true, false, CL> : k_persist_gl<false, true, false, false, CL>;
   if (v.masked)
     return v.hist ? k_persist_gl<true, false, true, false, CL>
-                  : (v.block ? k_persist_gl<true, false, false, false, CL> : k_persist_gl<true, false, false, false, CL, true>);
+                  : (v.block ? k_persist_gl<true, false, false, false, CL>
+                             : (v.fuse ? k_persist_gl<true, false, false, false, CL, true, false, true>
+                                       : k_persist_gl<true, false, false, false, CL, true>));
   return v.hist ? k_persist_gl<false, false, true, false, CL>
-                : (v.block ? k_persist_gl<false, false, false, false, CL> : k_persist_gl<false, false, false, false, CL, true>);
+                : (v.block ? k_persist_gl<false, false, false, false, CL>
+                           : (v.fuse ? k_persist_gl<false, false, false, false, CL, true, false, true>
+                                     : k_persist_gl<false, false, false, false, CL, true>));
 }
 
 PlainFn pick_plain(const StepVariant& v) {
@@ -1270,6 +1453,22 @@ cudaError_t launch_pack(const DevState& S, const uint64_t* prog, const int32_t* 
   return cudaGetLastError();
 }
 
+cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint64_t* prog_off, const uint32_t* bound,
+                        uint32_t num_programs, uint64_t wmask, bool classic, bool own, uint4* tmp, uint4* out,
+                        uint4* recs, cudaStream_t stream) {
+  if (!num_programs) return cudaSuccess;
+  uint32_t blocks = (num_programs + 127u) / 128u;
+  const uint32_t cap = (uint32_t)num_sms() * 16u;   // more blocks gain nothing (latency of each lane's scan)
+  if (blocks > cap) blocks = cap;
+  if (prog32)
+    k_fuse<int32_t><<<blocks, 128, 0, stream>>>(prog32, prog_off, bound, num_programs, wmask, classic, own, tmp, out,
+                                                recs);
+  else
+    k_fuse<uint64_t><<<blocks, 128, 0, stream>>>(prog, prog_off, bound, num_programs, wmask, classic, own, tmp, out,
+                                                 recs);
+  return cudaGetLastError();
+}
+
 using SharedFn = void (*)(DevState, Params, const uint64_t*, const uint64_t*, const uint32_t*, const uint32_t*,
                          uint32_t, uint32_t);
 
@@ -1328,7 +1527,8 @@ StepVariant shape_variant(StepVariant v, const PersistShape& sh) {
 }
 
 int persist_configure(const StepVariant& var, PersistShape& sh) {
-  const void* fn = persist_symbol(shape_variant(var, sh), sh.staged);
+  StepVariant v = shape_variant(var, sh);
+  const void* fn = persist_symbol(v, sh.staged);
   const size_t per_warp = sh.staged ? (32ull + 32ull * sh.slot_words) * 8ull : 0u;
   sh.smem = per_warp * sh.warps;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem) != cudaSuccess) {
@@ -1339,6 +1539,11 @@ int persist_configure(const StepVariant& var, PersistShape& sh) {
   // keep it as L1 for the M slabs in HBM
   cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
                        sh.staged ? (int)cudaSharedmemCarveoutMaxShared : (int)cudaSharedmemCarveoutMaxL1);
+  if (!sh.staged) {   // programs are loaded after the plan is made: the form with fused entries too (same bounds)
+    v.fuse = true;
+    cudaFuncSetAttribute(persist_symbol(v, false), cudaFuncAttributePreferredSharedMemoryCarveout,
+                         (int)cudaSharedmemCarveoutMaxL1);
+  }
   cudaGetLastError();
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, (int)(32u * sh.warps), sh.smem) != cudaSuccess) {
@@ -1362,7 +1567,8 @@ cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Para
   Queue q = Q;
   const uint64_t lanes = (uint64_t)grid * sh.warps * 32u;
   q.soft_end = Q.count > lanes ? (uint32_t)(Q.count - lanes) : 0u;
-  const StepVariant v = shape_variant(var, sh);
+  StepVariant v = shape_variant(var, sh);
+  v.fuse = S.fops != nullptr;
   if (sh.staged)
     pick_staged(v)<<<grid, 32u * sh.warps, sh.smem, stream>>>(S, P, q, sh.ncap, sh.slot_words, sh.epoch,
                                                                  sh.refill_min,
@@ -1451,10 +1657,11 @@ ServeFn pick_serve(const StepVariant& v) {
 int serve_configure(const StepVariant& var, ServeShape& sh) {
   const ServeFn fn = pick_serve(var);
   // the kernels a request's admission launches while the serving kernel is
-  // resident (state resets, pack, ring fill and publish) ask for the same L1/shared split,
+  // resident (state resets, fuse, pack, ring fill and publish) ask for the same L1/shared split,
   // so that an SM can host them beside it
   const void* beside[] = {(const void*)fn, (const void*)k_pack<uint64_t>, (const void*)k_pack<int32_t>,
-                          (const void*)k_ring_fill, (const void*)k_ring_publish, (const void*)k_fill};
+                          (const void*)k_ring_fill, (const void*)k_ring_publish, (const void*)k_fill,
+                          (const void*)k_fuse<uint64_t>, (const void*)k_fuse<int32_t>};
   for (const void* f : beside)
     cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxL1);
   cudaGetLastError();

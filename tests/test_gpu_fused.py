@@ -1,0 +1,120 @@
+"""Fused entries (runs of instructions decoded when programs are loaded)
+against the oracle, at the sizes and forms where they can go wrong: programs
+around the 64 instructions of a mask record, jumps back to earlier records,
+jumps on constants, wide constants, program words read and written as data,
+operands at the end of memory, runs stopped inside an entry and resumed, and
+programs shared by machines of different memories. Needs a GPU."""
+import numpy as np
+import pytest
+
+from paper_2604_12902_gb300 import workloads as W
+from tests.helpers import assert_same_state, oracle_state
+
+pytestmark = pytest.mark.gpu
+LOD, ADD, MUL, STO, BNZ, RD, PRI = 1, 2, 3, 4, 5, 6, 7
+
+
+@pytest.fixture(scope="module")
+def rasp():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2604_12902_gb300 import rasp as R
+    R.lib()
+    return R
+
+
+def machines(V, m, w, seed, extra=24, p_code=0.02, shared=0):
+    """V machines of m instructions: opcodes weighted to the fused form, small
+    and wide constants, data words mostly behind the program, jump targets
+    mostly even; a few operands in the program or past the memory."""
+    rng = np.random.default_rng(seed)
+    P = shared or V
+    n = 2 * m + extra
+    op = rng.choice([LOD, ADD, MUL, STO, BNZ, RD, PRI, 0, 9], size=(P, m),
+                    p=[.30, .24, .08, .17, .12, .04, .03, .01, .01])
+    data = rng.integers(2 * m, n, (P, m))
+    near = rng.integers(2 * m, 2 * m + 4, (P, m))                 # the same few words: stores that are read at once
+    arg = np.where(rng.random((P, m)) < .5, near, data)
+    arg = np.where(rng.random((P, m)) < p_code, rng.integers(0, 2 * m, (P, m)), arg)
+    arg = np.where(rng.random((P, m)) < .01, rng.integers(n, n + 3, (P, m)), arg)
+    target = 2 * rng.integers(0, m, (P, m)) + (rng.random((P, m)) < .03)
+    wide = rng.choice([-1, 1, 0, 2, -32768, 32767, 32768, 70000, -(1 << 31), (1 << 31) - 1], size=(P, m))
+    const = np.where(rng.random((P, m)) < .1, wide, rng.integers(-3, 4, (P, m)))
+    arg = np.where(op == BNZ, target, np.where(op == LOD, const, arg))
+    prog = np.empty((P, 2 * m), np.int64)
+    prog[:, 0::2], prog[:, 1::2] = op, arg
+    ell, s = 5, 3
+    tape = rng.integers(-1000, 1000, V * ell)
+    caps = rng.integers(1, 900, V).astype(np.uint64)
+    pvm = rng.integers(0, P, V).astype(np.uint32) if shared else None
+    mem = (n + rng.integers(0, 9, V) if shared else np.full(V, n)).astype(np.uint32)
+    return W.Workload("fused", prog.reshape(-1), np.arange(P + 1, dtype=np.uint64) * np.uint64(2 * m), mem, tape,
+                      np.arange(V + 1, dtype=np.uint64) * np.uint64(ell), caps, ell, s, w, pvm)
+
+
+def check(rasp, wl, budgets, what, classic=False, i32=True, **kw):
+    flags = kw.pop("flags", 0) | (rasp.ISA_CLASSIC if classic else 0)
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s, word_bits=wl.w, flags=flags, **kw) as b:
+        if i32:
+            rasp.rasp_load_programs_i32(b.h, wl.programs, wl.prog_off, wl.prog_of_vm)
+            b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+        else:
+            b.load_workload(wl)
+        for _ in range(2):                                        # from c_0 twice: a reset forgets written programs
+            for t in budgets:
+                b.run(t)
+                st, _ = oracle_state(wl, budget=t, threads=8, classic=classic)
+                assert_same_state(b.read_state(), st, wl.ell, wl.s, what="%s, budget %d" % (what, t))
+            b.reset()
+
+
+@pytest.mark.parametrize("w", [64, 48, 32, 20, 6])
+@pytest.mark.parametrize("m", [1, 2, 31, 64, 65, 130])
+def test_entries_match_the_oracle(rasp, m, w):
+    wl = machines(700, m, w, seed=1000 * m + w)
+    check(rasp, wl, [3, 20, 21, 200, 1000], "m=%d w=%d" % (m, w), i32=(m + w) % 2 == 0)
+
+
+@pytest.mark.parametrize("w", [64, 32])
+def test_classic_set(rasp, w):
+    check(rasp, machines(700, 70, w, seed=5), [7, 64, 1000], "classic w=%d" % w, classic=True)
+
+
+@pytest.mark.parametrize("p_code", [0.0, 0.3])
+def test_long_programs_and_code_words(rasp, p_code):
+    check(rasp, machines(150, 513, 64, seed=6, p_code=p_code), [100, 1000], "m=513 code %.1f" % p_code)
+    check(rasp, machines(300, 64, 64, seed=7, p_code=p_code, extra=2), [50, 1000], "no room beside the program")
+
+
+def test_shared_programs_on_several_memory_sizes(rasp):
+    wl = machines(1500, 40, 64, seed=8, shared=37)
+    check(rasp, wl, [30, 1000], "prog_of_vm", i32=False)
+    check(rasp, wl, [30, 1000], "prog_of_vm int32")
+
+
+def test_reloading_other_programs_under_a_graph(rasp):
+    """A captured run must not keep the entries of the programs loaded before."""
+    a, c = machines(600, 20, 64, seed=9, extra=120), machines(600, 60, 64, seed=10, extra=40)
+    assert np.array_equal(a.mem_words, c.mem_words)
+    with rasp.Batch(a.mem_words, a.ell, a.s, flags=rasp.CUDA_GRAPH) as b:
+        for wl in (a, c, a):
+            b.load_workload(wl)
+            b.run(400)
+            st, _ = oracle_state(wl, budget=400, threads=8)
+            assert_same_state(b.read_state(), st, wl.ell, wl.s, what="reload")
+
+
+def test_restored_memories_run_from_memory(rasp):
+    """A checkpoint whose memory differs from the loaded program's words."""
+    a, c = machines(300, 30, 64, seed=11), machines(300, 30, 64, seed=12)
+    with rasp.Batch(a.mem_words, a.ell, a.s) as b:
+        b.load_workload(a)
+        with rasp.Batch(c.mem_words, c.ell, c.s) as d:
+            d.load_workload(c)
+            st = d.read_state()
+        b.load_inputs(c.tapes, c.tape_off, c.caps)
+        b.load_state(st)
+        b.run(500)
+        want, _ = oracle_state(c, budget=500, threads=8)
+        assert_same_state(b.read_state(), want, c.ell, c.s, what="restored")
