@@ -97,7 +97,7 @@ struct rasp_batch {
   uint64_t wmask = ~0ull;
   std::vector<uint32_t> h_n;
   std::vector<uint64_t> h_memoff;
-  uint64_t mem_words = 0;      // sum of padded n
+  uint64_t mem_words = 0;      // words of the M arena: sum of slab_words(n)
   Layout L{};
   char* base = nullptr;
   bool owns = false;
@@ -235,6 +235,16 @@ Layout make_layout(uint64_t V, uint64_t mem_words, uint32_t ellp, uint32_t sp, u
 }
 
 uint32_t even(uint32_t x) { return (x + 1u) & ~1u; }
+
+// Words from one VM's slab to the next: n rounded up to even; on the
+// shared-program schedule to an odd number of word pairs. Its lanes run one
+// program nearly in step and touch the same offset of 32 slabs: with slabs a
+// multiple of 128 bytes apart all of these lie in the same L1 banks (32
+// cycles for such a load in place of about 8).
+uint64_t slab_words(const rasp_config* cfg, uint32_t n) {
+  const uint32_t e = even(n);
+  return (cfg->flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED && !(e & 2u) ? e + 2ull : e;
+}
 
 StepVariant variant_of(const rasp_batch* b) {
   StepVariant v{};
@@ -479,7 +489,7 @@ int rasp_batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* m
   if (rc) return rc;
   if (!out_bytes) return fail(RASP_EINVAL, "out_bytes is NULL");
   uint64_t mw = 0;
-  for (uint64_t v = 0; v < num_vms; ++v) mw += even(mem_words[v]);
+  for (uint64_t v = 0; v < num_vms; ++v) mw += slab_words(cfg, mem_words[v]);
   *out_bytes = make_layout(num_vms, mw, even(cfg->in_cap), even(cfg->out_cap), narrow_layout(cfg, true) ? 4u : 8u).total +
                ALIGN;
   return RASP_OK;
@@ -515,7 +525,7 @@ int rasp::create_batch(const rasp_config* cfg, uint64_t num_vms, const uint32_t*
   uint64_t off = 0;
   for (uint64_t v = 0; v < num_vms; ++v) {
     b->h_memoff[v] = off;
-    off += even(mem_words[v]);
+    off += slab_words(cfg, mem_words[v]);
   }
   b->mem_words = off;
   b->narrow = narrow_layout(cfg, plan);
@@ -657,10 +667,34 @@ int rasp_load_programs_i32(rasp_batch* b, const int32_t* words, const uint64_t* 
 
 namespace {
 
+// The 4-byte word offset in the program area where programs loaded as 4-byte
+// words are kept: 16-byte aligned.
+uint64_t kept_words_at(const rasp_batch* b) { return (b->mem_words + 3ull) & ~3ull; }
+
 // Whether the fused entries may read program words as data: not where the
 // shared-program schedule packs memories without them.
 bool owns_code(const rasp_batch* b) {
   return !b->shared_programs && (b->cfg.flags & RASP_SCHED_MASK) != RASP_SCHED_SHARED;
+}
+
+// Whether most of the programs write into themselves (an eighth of their
+// instructions or more), by a look at up to 64 of them: their VMs would leave
+// the entries at once, and the kernel without entries runs them faster (65,536
+// random programs with n = 256: 212 us a run against 275).
+template <class W>
+bool self_writing(const W* words, const uint64_t* offsets, uint64_t num_programs) {
+  const uint64_t looks = std::min<uint64_t>(num_programs, 64);
+  uint64_t writing = 0;
+  for (uint64_t q = 0; q < looks; ++q) {
+    const uint64_t p = q * num_programs / looks;
+    const uint64_t len = offsets[p + 1] - offsets[p], seen = std::min<uint64_t>(len, 1024);
+    const W* w = words + offsets[p];
+    uint64_t writes = 0;
+    for (uint64_t k = 0; k + 1 < seen; k += 2)
+      writes += (w[k] == 4 || w[k] == 6) && w[k + 1] >= 0 && (uint64_t)w[k + 1] < len ? 1 : 0;
+    writing += writes && 16 * writes >= seen ? 1 : 0;
+  }
+  return 2 * writing > looks;
 }
 
 // The place of the fused entries (at most 16 bytes per instruction, 8 per
@@ -674,7 +708,7 @@ uint4* place_fused(const rasp_batch* b, uint64_t total, bool keep32) {
   const StepVariant v = variant_of(b);
   if (!total || v.checked || v.hist || v.vote || v.block || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
   const uint64_t lo = keep32 && owns_code(b) ? 0 : 8ull * total;
-  const uint64_t end = keep32 ? 4ull * ((b->mem_words + 1ull) & ~1ull) : 8ull * b->mem_words;
+  const uint64_t end = keep32 ? 4ull * kept_words_at(b) : 8ull * b->mem_words;
   if (lo + 8ull * total > end || 8ull * total > (b->narrow ? 4ull : 8ull) * b->mem_words) return nullptr;
   return reinterpret_cast<uint4*>(reinterpret_cast<char*>(b->d_prog) + lo);
 }
@@ -703,14 +737,15 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   // copy has already replaced the earlier ones.
   //
   // 4-byte words are kept in the upper half of the program area, at word
-  // offset h = mem_words rounded up to even (8-byte aligned), when their
+  // offset h = mem_words rounded up to a multiple of four (k_widen reads them
+  // 16 bytes at a time), when their
   // widened copy [0, 8 total) bytes stays below that offset (2 total <= h)
   // and they end inside the area: the pack then reads them there and the
   // widening waits until a kernel needs 8-byte words. Otherwise they are
   // staged in the M arena (>= 4 total bytes, overwritten by the pack) and
   // widened into the program area before the pack.
   cudaStream_t st = b->stream;
-  const uint64_t h = (b->mem_words + 1ull) & ~1ull;
+  const uint64_t h = kept_words_at(b);
   const bool keep32 = word_size == 4 && 2ull * total <= h && 4ull * (h + total) <= 8ull * b->mem_words;
   int32_t* staged = keep32 ? reinterpret_cast<int32_t*>(b->d_prog) + h : reinterpret_cast<int32_t*>(b->S.mem);
   if (total)
@@ -770,7 +805,9 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   CK(cudaStreamSynchronize(st));   // the caller's buffers are read before the call returns
   // fused entries: their place, and the smallest memory that runs each program
   const uint32_t* bound = b->S.n;
-  b->S.fops = place_fused(b, total, keep32);
+  const bool from_memory = total && (word_size == 8 ? self_writing((const int64_t*)words, offsets, num_programs)
+                                                    : self_writing((const int32_t*)words, offsets, num_programs));
+  b->S.fops = from_memory ? nullptr : place_fused(b, total, keep32);
   b->S.frec = (const uint4*)(b->base + b->L.off_frec);
   b->S.prog_off = b->d_progoff;
   b->S.prog_of_vm = b->shared_programs ? b->d_progvm : nullptr;
@@ -1044,7 +1081,11 @@ int rasp_read_state(rasp_batch* b, uint64_t first, uint64_t count, rasp_state_vi
   uint64_t need = 0;
   if (out->mem) CK(materialize(b, st));      // a lazily packed batch: program words into the slabs first
   if (out->mem) {
-    for (uint64_t v = first; v < first + count; ++v) need += b->h_n[v];
+    bool uniform = true;
+    for (uint64_t v = first; v < first + count; ++v) {
+      need += b->h_n[v];
+      uniform = uniform && b->h_n[v] == b->h_n[first];
+    }
     if (out->mem_words < need) return fail(RASP_EINVAL, "mem holds %llu words, the range needs %llu",
                                            (unsigned long long)out->mem_words, (unsigned long long)need);
     const uint64_t lo = b->h_memoff[first];
@@ -1054,6 +1095,10 @@ int rasp_read_state(rasp_batch* b, uint64_t first, uint64_t count, rasp_state_vi
       CK(cudaMemcpyAsync(m32.data(), S.mem32 + lo, 4 * (hi - lo), cudaMemcpyDeviceToHost, st));
     } else if (need == hi - lo) {
       CK(cudaMemcpyAsync(out->mem, S.mem + lo, 8 * need, cudaMemcpyDeviceToHost, st));
+    } else if (uniform) {                    // equal slabs: one strided copy
+      const uint64_t pitch = count > 1 ? b->h_memoff[first + 1] - lo : b->h_n[first];
+      CK(cudaMemcpy2DAsync(out->mem, 8ull * b->h_n[first], S.mem + lo, 8ull * pitch, 8ull * b->h_n[first], count,
+                           cudaMemcpyDeviceToHost, st));
     } else {
       mbuf.resize(hi - lo);
       CK(cudaMemcpyAsync(mbuf.data(), S.mem + lo, 8 * (hi - lo), cudaMemcpyDeviceToHost, st));

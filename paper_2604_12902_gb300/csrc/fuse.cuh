@@ -360,6 +360,10 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs&
 #define RASP_F_FETCH_GL \
       "mad.wide.u32 ad1, j, 16, %11;\n\t" \
       "@!px ld.global.nc.v4.u32 {%1, %2, %3, %4}, [ad1];\n\t"
+// entries in shared memory (%11 = their 32-bit address)
+#define RASP_F_FETCH_SH \
+      "mad.lo.u32 t0, j, 16, %11;\n\t" \
+      "@!px ld.shared.v4.u32 {%1, %2, %3, %4}, [t0];\n\t"
 #define RASP_F_REGS \
       ".reg .pred px, pr, p1, p2, pt;\n\t" \
       ".reg .b32 c, t0, ye, j, it;\n\t" \
@@ -408,9 +412,9 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs&
       RASP_F_TEST("p1", "0x40000000") \
       "add.u64 im, %0, -1;\n\t" \
       "setp.lt.and.u64 pt, im, %18, p1;\n\t"
-#define RASP_FW_OPERANDS \
+#define RASP_FW_OPERANDS(TAB) \
   : "+l"(a), "+r"(F.op.x), "+r"(F.op.y), "+r"(F.op.z), "+r"(F.op.w), "+r"(F.cur), "+r"(left), "+r"(u0), "+r"(y0) \
-  : "r"(iters), "l"(M), "l"(F.tab), "l"(T), "l"(Y), "r"(ell), "r"(s), "r"(mask), "l"(wmask),                    \
+  : "r"(iters), "l"(M), TAB, "l"(T), "l"(Y), "r"(ell), "r"(s), "r"(mask), "l"(wmask),                    \
     "l"(wmask >> 1), "r"(zero)                                                                                   \
   : "memory"
 
@@ -420,15 +424,30 @@ __device__ __forceinline__ void fused_loop_ptx(uint64_t* M, const uint64_t* T, u
                                                Fused& F, uint32_t& left, uint32_t& u0, uint32_t& y0) {
   if constexpr (MASKED && CLASSIC) {
     asm volatile(RASP_FW_A RASP_FW_SUB RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_CLASSIC
-                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS);
+                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS("l"(F.tab)));
   } else if constexpr (MASKED) {
     asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
-                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS);
+                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS("l"(F.tab)));
   } else if constexpr (CLASSIC) {
     asm volatile(RASP_FW_A RASP_FW_SUB RASP_FW_B RASP_FW_PT_CLASSIC RASP_F_NEXT(RASP_F_FETCH_GL)
-                 RASP_FW_OPERANDS);
+                 RASP_FW_OPERANDS("l"(F.tab)));
   } else {
-    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS);
+    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS("l"(F.tab)));
+  }
+}
+
+// The entries of a shared program in shared memory (word opcode set).
+template <bool MASKED>
+__device__ __forceinline__ void fused_loop_ptx_sh(uint64_t* M, uint32_t tab, const uint64_t* T, uint64_t* Y,
+                                                  uint32_t ell, uint32_t s, uint64_t wmask, uint32_t mask,
+                                                  uint32_t iters, uint32_t zero, uint64_t& a, Fused& F,
+                                                  uint32_t& left, uint32_t& u0, uint32_t& y0) {
+  if constexpr (MASKED) {
+    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
+                 RASP_F_NEXT(RASP_F_FETCH_SH) RASP_FW_OPERANDS("r"(tab)));
+  } else {
+    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_SH)
+                 RASP_FW_OPERANDS("r"(tab)));
   }
 }
 

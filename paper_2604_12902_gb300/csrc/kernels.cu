@@ -456,7 +456,8 @@ constexpr uint32_t kFuseOutside = 32;  // general steps at no entry's start befo
 template <bool MASKED, bool CLASSIC, class Mem>
 __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64_t* Y, const Params& P, Regs& r,
                                                 Fused& F, const DevState& S, uint32_t vm, Hist& h, bool& active,
-                                                uint32_t& final_st, uint32_t epoch, uint32_t idle_exit) {
+                                                uint32_t& final_st, uint32_t epoch, uint32_t idle_exit,
+                                                uint32_t shared_tab = 0) {
   const uint32_t fm = __ballot_sync(FULL, active && F.on);
   bool stall = active && r.clean && !F.on;               // a stop has cut the run of an entry: on to the next one
   if (fm) {
@@ -474,6 +475,9 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
           else
             fused_loop_ptx_narrow<true, CLASSIC>(M.M, T, Y, P.ell, P.s, wm32, fm, c, zero, a32, F, r.left, r.u0, r.y0);
           r.a = a32;
+        } else if constexpr (std::is_same<Mem, ShView>::value) {
+          fused_loop_ptx_sh<MASKED>(M.M, shared_tab, T, Y, P.ell, P.s, P.wmask, fm, c, zero, r.a, F, r.left, r.u0,
+                                    r.y0);
         } else {
           fused_loop_ptx<MASKED, CLASSIC>(M, T, Y, P.ell, P.s, P.wmask, fm, c, zero, r.a, F, r.left, r.u0, r.y0);
         }
@@ -489,7 +493,10 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
     final_st = ST_HALTED;
   } else if (stall) {
     const FuseProg G = fuse_prog(S, vm, r.ilim);
-    CodeView<Mem> V{M, G.plen};
+    const auto V = [&] {
+      if constexpr (std::is_same<Mem, ShView>::value) return M;     // notices writes into the program itself
+      else return CodeView<Mem>{M, G.plen};
+    }();
     if (F.on) r.ip = 2u * (F.op.y & FO_COUNT ? fuse_instr(G, F.cur) : F.op.x);
     r.have = false;
     for (uint32_t out = 0; active && stall;) {
@@ -503,7 +510,7 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
       }
     }
     if (active && !F.on) {
-      r.clean = false;
+      if constexpr (!std::is_same<Mem, ShView>::value) r.clean = false;   // (a shared program's view watches writes)
       prime(M, r);
     }
   }
@@ -1064,7 +1071,9 @@ __global__ void __launch_bounds__(128) k_shared(DevState S, Params P, const uint
 // clean VM loaded from the shared copy); at each epoch boundary the lanes
 // whose VM stopped store it and take the next VMs of the program (one
 // shared-memory atomic per warp).
-template <bool MASKED>
+// FUSE: clean VMs run from the program's fused entries, held in shared memory
+// behind its words.
+template <bool MASKED, bool FUSE>
 __global__ void __launch_bounds__(128, 7) k_shared_loop(DevState S, Params P, const uint64_t* __restrict__ prog,
                                                         const uint64_t* __restrict__ prog_off,
                                                         const uint32_t* __restrict__ pv_off,
@@ -1079,6 +1088,15 @@ __global__ void __launch_bounds__(128, 7) k_shared_loop(DevState S, Params P, co
     const uint64_t po = prog_off[p];
     const uint32_t plen = (uint32_t)(prog_off[p + 1] - po);
     for (uint32_t k = threadIdx.x; k < plen; k += blockDim.x) ps[k] = prog[po + k] & P.wmask;
+    uint32_t tab = 0;
+    if constexpr (FUSE) {
+      const uint32_t nrec = (plen + 127u) / 128u;
+      const uint4* rec = S.frec + (po >> 7) + p;
+      const uint32_t count = nrec ? rec[nrec - 1u].z + (uint32_t)__popcll(fuse_mask(rec[nrec - 1u])) : 0u;
+      uint4* ent = reinterpret_cast<uint4*>(ps + plen);
+      for (uint32_t k = threadIdx.x; k < count; k += blockDim.x) ent[k] = S.fops[(po >> 1) + k];
+      tab = smem_addr(ent);
+    }
     if (threadIdx.x == 0) next = 0;
     __syncthreads();
     const uint32_t first = pv_off[p], count = pv_off[p + 1] - first;
@@ -1090,6 +1108,7 @@ __global__ void __launch_bounds__(128, 7) k_shared_loop(DevState S, Params P, co
     ShView V{S.mem, ps, plen};
     const uint64_t* T = S.tape;
     uint64_t* Y = S.y;
+    Fused F{};
     for (;;) {
       // boundary: retire stopped VMs, then refill idle lanes
       if (vm >= 0 && !active) {
@@ -1115,7 +1134,8 @@ __global__ void __launch_bounds__(128, 7) k_shared_loop(DevState S, Params P, co
               T = S.tape + (uint64_t)v * P.ellp;
               Y = S.y + (uint64_t)v * P.sp;
               vm = (int32_t)v;
-              prime(V, r);
+              if constexpr (FUSE) fuse_enter(fuse_prog(S, v, r.ilim), F, r);
+              if (!F.on) prime(V, r);
               active = true;
             }
           } else {
@@ -1125,7 +1145,10 @@ __global__ void __launch_bounds__(128, 7) k_shared_loop(DevState S, Params P, co
       }
       if (__all_sync(FULL, vm < 0 && !more)) break;
       if (!__any_sync(FULL, active)) continue;
-      run_epoch_loop<MASKED, false>(V, T, Y, P, r, h, active, final_st, epoch, 0u);
+      if constexpr (FUSE)
+        run_epoch_fused<MASKED, false>(V, T, Y, P, r, F, S, (uint32_t)vm, h, active, final_st, epoch, 0u, tab);
+      else
+        run_epoch_loop<MASKED, false>(V, T, Y, P, r, h, active, final_st, epoch, 0u);
     }
     __syncthreads();   // every lane done with this program's copy
   }
@@ -1476,15 +1499,21 @@ SharedFn pick_shared(const StepVariant& v) {
   if (v.checked) return v.hist ? k_shared<false, true, true> : k_shared<false, true, false>;
   if (v.hist) return v.masked ? k_shared<true, false, true> : k_shared<false, false, true>;
   if (v.block) return v.masked ? k_shared<true, false, false> : k_shared<false, false, false>;
-  return v.masked ? k_shared_loop<true> : k_shared_loop<false>;
+  if (v.fuse) return v.masked ? k_shared_loop<true, true> : k_shared_loop<false, true>;
+  return v.masked ? k_shared_loop<true, false> : k_shared_loop<false, false>;
 }
 
 cudaError_t launch_shared(const StepVariant& var, const DevState& S, const Params& P, const uint64_t* prog,
                           const uint64_t* prog_off, const uint32_t* pv_off, const uint32_t* pv_ids,
                           uint32_t num_programs, uint32_t max_plen, uint32_t epoch, cudaStream_t stream) {
   if (!num_programs) return cudaSuccess;
-  const size_t smem = (size_t)((max_plen + 1u) & ~1u) * 8u;
-  SharedFn fn = pick_shared(var);
+  size_t smem = (size_t)((max_plen + 1u) & ~1u) * 8u;
+  // the entries take at most as much again; where that would leave an SM fewer
+  // than two CTAs, the programs run one instruction at a time
+  StepVariant v = var;
+  v.fuse = S.fops != nullptr && !v.checked && !v.hist && !v.block && 2u * smem <= 96u * 1024u;
+  if (v.fuse) smem *= 2u;
+  SharedFn fn = pick_shared(v);
   if (smem > 48u * 1024u) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return cudaGetLastError();

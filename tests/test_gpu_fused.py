@@ -93,6 +93,28 @@ def test_shared_programs_on_several_memory_sizes(rasp):
     check(rasp, wl, [30, 1000], "prog_of_vm int32")
 
 
+@pytest.mark.parametrize("w", [64, 20])
+@pytest.mark.parametrize("m", [1, 40, 64, 129])
+def test_shared_program_schedule(rasp, m, w):
+    """Entries in shared memory beside the program, VMs that read and write
+    program words, memories read back midway (which fills the slabs)."""
+    for p_code in (0.0, 0.1):
+        wl = machines(900, m, w, seed=20 + m + w, shared=11, p_code=p_code)
+        check(rasp, wl, [30, 31, 1000], "shared m=%d w=%d code %.1f" % (m, w, p_code), flags=rasp.SCHED_SHARED,
+              i32=m != 40)
+
+
+def test_self_writing_programs(rasp):
+    """Batches in which all, some or few programs mostly write into themselves."""
+    a = W.random_programs(num_vms=512, seed=3, mem_words=200)
+    check(rasp, a, [20, 256], "all")
+    c = machines(512, 32, 64, seed=13, extra=136)
+    for every in (2, 9):
+        prog = np.where((np.arange(512) % every == 0)[:, None], a.programs.reshape(512, -1), c.programs.reshape(512, -1))
+        wl = W.Workload("mixed", prog.reshape(-1), a.prog_off, c.mem_words, c.tapes, c.tape_off, c.caps, c.ell, c.s)
+        check(rasp, wl, [20, 1000], "every %d" % every)
+
+
 def test_reloading_other_programs_under_a_graph(rasp):
     """A captured run must not keep the entries of the programs loaded before."""
     a, c = machines(600, 20, 64, seed=9, extra=120), machines(600, 60, 64, seed=10, extra=40)
