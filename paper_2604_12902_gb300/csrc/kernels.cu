@@ -25,7 +25,6 @@
 
 namespace rasp {
 
-constexpr uint32_t FULL = 0xffffffffu;
 constexpr uint32_t WAIT_LIMIT = 1u << 22;   // mbarrier polls before giving up (default; the
                                            // staged kernel takes its limit as an argument)
 
@@ -351,92 +350,6 @@ __device__ __forceinline__ void run_epoch(Mem M, const uint64_t* T, uint64_t* Y,
         break;
       }
     }
-  }
-}
-
-// Run up to `epoch` steps of every active lane with the epoch loop of
-// fast_loop_ptx (WRAP, no counters, select dispatch). Each round runs the
-// loop for at most the smallest step countdown of the warp; then the lanes
-// whose step needs the general path (the loop left by a warp vote, nothing
-// of that step applied) or whose countdown ended take one step with
-// step_general, and every active lane re-enters the loop together. A round
-// with general steps counts one more step of the epoch, so the epoch always
-// ends. With idle_exit > 0 the epoch also ends once that many lanes that were
-// running at its start have stopped, so that they are refilled sooner.
-template <bool MASKED, bool CLASSIC, class Mem>
-__device__ __forceinline__ void run_epoch_loop(Mem M, const uint64_t* T, uint64_t* Y, const Params& P,
-                                               Regs& r, Hist& h, bool& active, uint32_t& final_st, uint32_t epoch,
-                                               uint32_t idle_exit) {
-  const uint32_t mask0 = __ballot_sync(FULL, active);
-  uint32_t mask = mask0;
-  uint32_t k = epoch;
-  while (k && mask) {
-    uint32_t done = 0;
-    bool general = false;
-    if (active) {
-      uint32_t kk = min(k, __reduce_min_sync(mask, r.left));
-      uint32_t rare = 0;
-      if (kk) {
-        const uint32_t k0 = kk;
-        uint32_t hv = r.have ? 1u : 0u;
-        uint64_t co = r.cur.x, cj = r.cur.y;
-        if constexpr (std::is_same<Mem, ShView>::value) {
-          // clean: code from the shared program (fetch limit min(plen, ilim)),
-          // data accesses below plen through the general step
-          const bool cl = r.clean;
-          rare = fast_loop_ptx_sh<MASKED>(M.M, cl ? M.Pg : M.M, cl ? M.plen : 0u, T, Y, r.n, P.ell, P.s,
-                                          cl ? min(M.plen, r.ilim) : r.ilim, P.wmask, mask, r.a, co, cj, r.ip,
-                                          r.u0, r.y0, hv, kk);
-        } else if constexpr (std::is_same<Mem, NarrowView>::value) {
-          // 4-byte words: the loop runs on 32-bit values (w <= 32)
-          uint32_t a32 = (uint32_t)r.a, co32 = (uint32_t)co, cj32 = (uint32_t)cj;
-          const uint32_t wm32 = (uint32_t)P.wmask;
-          if (wm32 == 0xFFFFFFFFu)
-            rare = fast_loop_ptx_narrow<false, CLASSIC>(M.M, T, Y, r.n, P.ell, P.s, r.ilim, wm32, mask, a32, co32,
-                                                        cj32, r.ip, r.u0, r.y0, hv, kk);
-          else
-            rare = fast_loop_ptx_narrow<true, CLASSIC>(M.M, T, Y, r.n, P.ell, P.s, r.ilim, wm32, mask, a32, co32,
-                                                       cj32, r.ip, r.u0, r.y0, hv, kk);
-          r.a = a32;
-          co = co32;
-          cj = cj32;
-        } else if constexpr (std::is_same<Mem, SmemView>::value) {
-          // M, tape and y in shared memory: generic addresses, word opcode set
-          rare = fast_loop_ptx_gen<MASKED>(M.M, T, Y, r.n, P.ell, P.s, r.ilim, P.wmask, mask, r.a, co, cj, r.ip,
-                                           r.u0, r.y0, hv, kk);
-        } else {
-          rare = fast_loop_ptx<MASKED, CLASSIC>(M, T, Y, r.n, P.ell, P.s, r.ilim, P.wmask, mask, r.a, co, cj, r.ip,
-                                                r.u0, r.y0, hv, kk);
-        }
-        r.cur.x = co;
-        r.cur.y = cj;
-        r.have = hv != 0u;
-        done = k0 - kk;
-        r.left -= done;
-      }
-      general = rare || r.left == 0u;
-      if (general) {
-        if (r.ip >= r.ilim) {
-          // the loop took i (+) 2 = ip + 2 unreduced (ibase = 0): reduce it
-          const uint64_t i = (uint64_t)r.ip & P.wmask;
-          r.ip = mod_n(i, r.n);
-          r.ibase = i - r.ip;
-        }
-        r.have = false;
-        const uint32_t st = step_general<MASKED, false, false, CLASSIC>(M, T, Y, P, r, h);
-        if (st == CONT) {
-          prime(M, r);
-        } else {
-          active = false;
-          final_st = st;
-        }
-      }
-    }
-    done = __shfl_sync(FULL, done, __ffs(mask) - 1);        // the same in every lane of the mask
-    k -= done;
-    if (__any_sync(FULL, general) && k) k -= 1u;
-    mask = __ballot_sync(FULL, active);
-    if (idle_exit && (uint32_t)__popc(mask0 & ~mask) >= idle_exit) break;
   }
 }
 
