@@ -93,8 +93,8 @@ enum rasp_semantics {
                                           in budget rounds (4096 x 8^k steps)
                                           with the still-running VMs compacted
                                           between rounds; by default only
-                                          batches larger than the resident
-                                          lanes do                             */
+                                          batches larger than half of the
+                                          resident lanes do                    */
 #define RASP_STEP_BLOCK        0x20000u /* HBM-slab persistent schedule: evaluate
                                           every step as one predicated block
                                           (the earlier form) instead of the

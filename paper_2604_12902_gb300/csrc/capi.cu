@@ -829,7 +829,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   if (word_size == 4 && total && !keep32) CK(launch_widen(staged, b->d_prog, total, st));
   if (b->S.fops)
     CK(launch_fuse(b->d_prog, b->prog32, b->d_progoff, bound, b->num_programs, b->wmask, variant_of(b).classic,
-                   owns_code(b), reinterpret_cast<uint4*>(b->S.mem), const_cast<uint4*>(b->S.fops),
+                   owns_code(b), b->narrow, reinterpret_cast<uint4*>(b->S.mem), const_cast<uint4*>(b->S.fops),
                    const_cast<uint4*>(b->S.frec), st));
   CK(fill_bytes(b->d_hist, 0, 8 * 10, st));
   b->code_lazy = pack_lazy(b);
@@ -930,11 +930,11 @@ namespace {
 // the launch group that are still RUNNING are compacted into a dense queue:
 // the few long-running VMs then fill whole warps instead of each keeping a
 // warp busy whose other lanes have nothing left to run. Rounds are used for
-// launch groups larger than the resident lanes (whose lanes are refilled
-// from the queue, so that the survivors end up scattered), or always with
-// RASP_BUDGET_ROUNDS; a group that fits the resident lanes runs in one launch,
-// which also lets concurrent batches (the serving pool) share the GPU without
-// waiting for SMs at every round.
+// launch groups larger than half of the resident lanes, or always with
+// RASP_BUDGET_ROUNDS. Fewer VMs leave so few survivors that they run faster
+// scattered, a lane or two per warp, than packed into warps that wait for the
+// slowest of 32 lanes (131,072 search programs to 10^5 steps: 12.4 ms in one
+// launch, 11.2 in rounds; 32,768: 8.8 and 10.1; uneven 131,072: 5.2 and 4.3).
 constexpr uint64_t kRound0 = 4096;
 constexpr uint64_t kRoundGrowth = 8;
 constexpr int kMaxRounds = 6;
@@ -974,7 +974,7 @@ int enqueue_run(rasp_batch* b, cudaStream_t st, uint64_t max_steps) {
       std::vector<uint64_t> budgets;
       const uint64_t limit = std::min(max_steps, b->max_cap);
       const uint64_t lanes = (uint64_t)g.shape.grid * g.shape.warps * 32u;
-      const bool rounds = (b->cfg.flags & RASP_BUDGET_ROUNDS) || g.count > lanes;
+      const bool rounds = (b->cfg.flags & RASP_BUDGET_ROUNDS) || g.count > lanes / 2;
       for (uint64_t r = kRound0; rounds && r < limit && (int)budgets.size() < kMaxRounds; r *= kRoundGrowth)
         budgets.push_back(r);
       budgets.push_back(max_steps);

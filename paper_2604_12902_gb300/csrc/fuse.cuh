@@ -14,7 +14,8 @@
 // instructions from one instruction on that fits the form
 //
 //   a <- imm1 | a <- a op M[j1], op = ADD or MUL (SUB), or y :: M[j1] (PRI) |
-//   M[k] <- a (STO) or the next tape word (RD) | a <- imm2 | a <- a + M[j2] | BNZ t
+//   M[k] <- a (STO) or the next tape word (RD) | a <- imm2 | a <- a + M[j2] |
+//   BNZ t, or, in the loop on 4-byte words, M[k2] <- a (STO)
 //
 // (every part optional, in this order) with jumps on constants followed. Only
 // the entries that runs from instruction 0 can reach are kept, in instruction
@@ -51,6 +52,7 @@ enum : uint32_t {
   FO_LD2 = 0x1000u << 16,     // a <- a + M[j2]
   FO_FWD = 0x2000u << 16,     // a <- a + the value STO wrote (j2 = k)
   FO_BNZ = 0x4000u << 16,     // jump to t if the condition holds, else f
+  FO_ST2 = 0x8000u << 16,     // M[t] <- a (no jump: t holds k2)
   FO_HALT = 0x8000u << 16,    // (stall) a fixed point: an invalid opcode
   FO_MEM = 0x4000u << 16,     // (stall, entry 0) the program mostly writes into itself: run it from memory
 };
@@ -71,10 +73,14 @@ __device__ __forceinline__ ulonglong2 fuse_pair(const int32_t* src, uint32_t k, 
 // at least n words: `mok` instructions lie where i (+) 2 and the pair need no
 // reduction. own: M holds the program words (they may be read as data).
 // The state of the scan is the next free part of the form (stage 0 imm1,
-// 1 op, 2 store, 3 imm2, 4 add, 5 jump) and a constant not yet placed.
+// 1 op, 2 store, 3 imm2, 4 add, 5 second store or jump) and a constant not yet
+// placed. two: entries may hold the second store. It takes the slowest loops of
+// the halting workload from 3.1 to 4.0 VM-steps per entry (run of 2^18 programs
+// 121 -> 92 ms), and costs 6 of about 65 instructions on 8-byte words, where
+// the template and uneven batches gain little from it (1.96 -> 2.05 ms).
 template <class W>
 __device__ __forceinline__ uint4 fuse_one(const W* src, uint32_t e, uint32_t plen, uint32_t n, uint32_t mok,
-                                          uint64_t wmask, bool classic, bool own) {
+                                          uint64_t wmask, bool classic, bool own, bool two) {
   uint32_t p = e, stage = 0, cnt = 0, flags = 0, j1 = 0, k = 0, j2 = 0, i1 = 0, i2 = 0, t = e, f = e;
   bool pend = false;
   uint64_t cv = 0;
@@ -92,7 +98,7 @@ __device__ __forceinline__ uint4 fuse_one(const W* src, uint32_t e, uint32_t ple
         cnt += 1u;
         continue;
       }
-      if (!target || p + 1u >= mok) break;
+      if (!target || p + 1u >= mok || (flags & FO_ST2)) break;
       flags |= FO_BNZ;
       t = (uint32_t)(j >> 1);
       p += 1u;
@@ -148,6 +154,15 @@ __device__ __forceinline__ uint4 fuse_one(const W* src, uint32_t e, uint32_t ple
         flags |= FO_STO;
         k = jm;
         stage = 3u;
+      } else if (op == 4u && two && stage <= (pend ? 3u : 5u)) {
+        if (pend) {
+          flags |= FO_L2;
+          i2 = (uint32_t)cv & 0xFFFFu;
+          pend = false;
+        }
+        flags |= FO_ST2;
+        t = jm;
+        stage = 6u;
       } else if (op == 6u && stage <= 2u) {
         flags |= FO_RD;
         k = jm;
@@ -292,7 +307,7 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs&
   if (F.on && !(F.op.y & FO_COUNT) && (F.op.y & FO_MEM)) F.on = r.clean = false;
 }
 
-// `iters` entries of every lane of `mask` (all of them call it together).
+// `iters` (even) entries of every lane of `mask` (all of them call it together).
 // Word sizes: 8-byte words of M and a 64-bit accumulator, or (narrow, w <= 32)
 // 4-byte words and 32-bit arithmetic. Per entry: the dynamic guards (px, a
 // lane that stalls clears its flags and so applies nothing), both loads, the
@@ -353,7 +368,18 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs&
       "@!px mov.b32 %5, j;\n\t" \
       "@!px sub.u32 %6, %6, c;\n\t" \
       FETCH \
+      "}"
+#define RASP_F_LOOP1(BODY) \
+      BODY \
       "add.u32 it, it, -1;\n\t" \
+      "setp.ne.u32 p1, it, 0;\n\t" \
+      "@p1 bra.uni RASP_FLOOP;\n\t" \
+      "}"
+// two entries per turn (iters is even): 0.81 -> 0.79 ms for the entries in
+// shared memory, slower for the others (2^20 templates 1.98 -> 2.18 ms)
+#define RASP_F_LOOP2(BODY) \
+      BODY BODY \
+      "add.u32 it, it, -2;\n\t" \
       "setp.ne.u32 p1, it, 0;\n\t" \
       "@p1 bra.uni RASP_FLOOP;\n\t" \
       "}"
@@ -366,16 +392,13 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs&
       "@!px ld.shared.v4.u32 {%1, %2, %3, %4}, [t0];\n\t"
 #define RASP_F_REGS \
       ".reg .pred px, pr, p1, p2, pt;\n\t" \
-      ".reg .b32 c, t0, ye, j, it;\n\t" \
+      ".reg .b32 c, t0, ye, j, it, zz;\n\t" \
       ".reg .b64 ad1, ad2, ads;\n\t"
 
 // 8-byte words. %17 = 2^w - 1 (masked), %18 = its half (classic condition).
+#define RASP_FW_HEAD "{\n\t" RASP_F_REGS ".reg .b64 v1, v2, im;\n\t" "mov.b32 it, %9;\n\tRASP_FLOOP:\n\t"
 #define RASP_FW_A \
-      "{\n\t" RASP_F_REGS \
-      ".reg .b64 v1, v2, im;\n\t" \
-      "mov.b32 it, %9;\n\t" \
-      "RASP_FLOOP:\n\t" \
-      RASP_F_GUARD RASP_F_ADDR("8") \
+      "{\n\t" RASP_F_GUARD RASP_F_ADDR("8") \
       "@p1 ld.global.u64 v1, [ad1];\n\t" \
       "@p2 ld.global.u64 v2, [ad2];\n\t" \
       "cvt.s32.s16 t0, %3;\n\t" \
@@ -392,8 +415,8 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs&
       RASP_F_TEST("p1", "0x02000000") \
       "cvt.u32.u64 t0, v1;\n\t" \
       "cvt.u32.u64 j, v2;\n\t" \
-      "lop3.b32 t0, t0, j, %19, 0xA8;\n\t" \
-      "cvt.u64.u32 im, t0;\n\t" \
+      "lop3.b32 zz, t0, j, %19, 0xA8;\n\t" \
+      "cvt.u64.u32 im, zz;\n\t" \
       "xor.b64 im, im, %0;\n\t" \
       "@p1 st.global.u64 [ads], im;\n\t" \
       RASP_F_IO("ld.global.u64", "st.global.u64", "v1", "im") \
@@ -420,19 +443,25 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs&
 
 template <bool MASKED, bool CLASSIC>
 __device__ __forceinline__ void fused_loop_ptx(uint64_t* M, const uint64_t* T, uint64_t* Y, uint32_t ell, uint32_t s,
-                                               uint64_t wmask, uint32_t mask, uint32_t iters, uint32_t zero, uint64_t& a,
-                                               Fused& F, uint32_t& left, uint32_t& u0, uint32_t& y0) {
+                                               uint64_t wmask, uint32_t mask, uint32_t iters, uint32_t zero,
+                                               uint64_t& a, Fused& F, uint32_t& left, uint32_t& u0, uint32_t& y0) {
   if constexpr (MASKED && CLASSIC) {
-    asm volatile(RASP_FW_A RASP_FW_SUB RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_CLASSIC
-                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS("l"(F.tab)));
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP1(
+        RASP_FW_A RASP_FW_SUB RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_CLASSIC
+        RASP_F_NEXT(RASP_F_FETCH_GL))
+                 RASP_FW_OPERANDS("l"(F.tab)));
   } else if constexpr (MASKED) {
-    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
-                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS("l"(F.tab)));
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP1(
+        RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
+        RASP_F_NEXT(RASP_F_FETCH_GL))
+                 RASP_FW_OPERANDS("l"(F.tab)));
   } else if constexpr (CLASSIC) {
-    asm volatile(RASP_FW_A RASP_FW_SUB RASP_FW_B RASP_FW_PT_CLASSIC RASP_F_NEXT(RASP_F_FETCH_GL)
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP1(
+        RASP_FW_A RASP_FW_SUB RASP_FW_B RASP_FW_PT_CLASSIC RASP_F_NEXT(RASP_F_FETCH_GL))
                  RASP_FW_OPERANDS("l"(F.tab)));
   } else {
-    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FW_OPERANDS("l"(F.tab)));
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP1(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_GL))
+                 RASP_FW_OPERANDS("l"(F.tab)));
   }
 }
 
@@ -443,22 +472,21 @@ __device__ __forceinline__ void fused_loop_ptx_sh(uint64_t* M, uint32_t tab, con
                                                   uint32_t iters, uint32_t zero, uint64_t& a, Fused& F,
                                                   uint32_t& left, uint32_t& u0, uint32_t& y0) {
   if constexpr (MASKED) {
-    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
-                 RASP_F_NEXT(RASP_F_FETCH_SH) RASP_FW_OPERANDS("r"(tab)));
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP2(
+        RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
+        RASP_F_NEXT(RASP_F_FETCH_SH))
+                 RASP_FW_OPERANDS("r"(tab)));
   } else {
-    asm volatile(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_SH)
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP2(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_SH))
                  RASP_FW_OPERANDS("r"(tab)));
   }
 }
 
 // 4-byte words (w <= 32). Tape words and outputs are 8-byte words whose high
 // halves are zero. %17 = 2^w - 1, %18 = its half.
+#define RASP_FN_HEAD "{\n\t" RASP_F_REGS ".reg .b32 v1, v2, im;\n\t" "mov.b32 it, %9;\n\tRASP_FLOOP:\n\t"
 #define RASP_FN_A \
-      "{\n\t" RASP_F_REGS \
-      ".reg .b32 v1, v2, im;\n\t" \
-      "mov.b32 it, %9;\n\t" \
-      "RASP_FLOOP:\n\t" \
-      RASP_F_GUARD RASP_F_ADDR("4") \
+      "{\n\t" RASP_F_GUARD RASP_F_ADDR("4") \
       "@p1 ld.global.u32 v1, [ad1];\n\t" \
       "@p2 ld.global.u32 v2, [ad2];\n\t" \
       "cvt.s32.s16 im, %3;\n\t" \
@@ -472,8 +500,8 @@ __device__ __forceinline__ void fused_loop_ptx_sh(uint64_t* M, uint32_t tab, con
 #define RASP_FN_MASK "and.b32 %0, %0, %17;\n\t"
 #define RASP_FN_B \
       RASP_F_TEST("p1", "0x02000000") \
-      "lop3.b32 t0, v1, v2, %19, 0xA8;\n\t" \
-      "xor.b32 t0, t0, %0;\n\t" \
+      "lop3.b32 zz, v1, v2, %19, 0xA8;\n\t" \
+      "xor.b32 t0, zz, %0;\n\t" \
       "@p1 st.global.u32 [ads], t0;\n\t" \
       RASP_F_IO("ld.global.u32", "st.global.u32", "v1", "im") \
       RASP_F_TEST("p1", "0x20000000") \
@@ -483,6 +511,12 @@ __device__ __forceinline__ void fused_loop_ptx_sh(uint64_t* M, uint32_t tab, con
       "@p1 mov.b32 %0, im;\n\t" \
       RASP_F_TEST("p1", "0x30000000") \
       "@p1 add.u32 %0, %0, v2;\n\t"
+#define RASP_FN_ST2 \
+      "and.b32 j, %4, 0xFFFF;\n\t" \
+      "mad.wide.u32 ads, j, 4, %10;\n\t" \
+      "setp.lt.s32 p1, ye, 0;\n\t" \
+      "xor.b32 t0, zz, %0;\n\t" \
+      "@p1 st.global.u32 [ads], t0;\n\t"
 #define RASP_FN_PT_WORD \
       RASP_F_TEST("p1", "0x40000000") \
       "setp.ne.and.u32 pt, %0, 0, p1;\n\t"
@@ -503,15 +537,25 @@ __device__ __forceinline__ void fused_loop_ptx_narrow(uint32_t* M, const uint64_
                                                       uint32_t zero, uint32_t& a, Fused& F, uint32_t& left,
                                                       uint32_t& u0, uint32_t& y0) {
   if constexpr (MASK && CLASSIC) {
-    asm volatile(RASP_FN_A RASP_FN_SUB RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_PT_CLASSIC
-                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FN_OPERANDS);
+    asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
+        RASP_FN_A RASP_FN_SUB RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_ST2 RASP_FN_PT_CLASSIC
+        RASP_F_NEXT(RASP_F_FETCH_GL))
+                 RASP_FN_OPERANDS);
   } else if constexpr (MASK) {
-    asm volatile(RASP_FN_A RASP_FN_MUL RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_PT_WORD
-                 RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FN_OPERANDS);
+    asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
+        RASP_FN_A RASP_FN_MUL RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_ST2 RASP_FN_PT_WORD
+        RASP_F_NEXT(RASP_F_FETCH_GL))
+                 RASP_FN_OPERANDS);
   } else if constexpr (CLASSIC) {
-    asm volatile(RASP_FN_A RASP_FN_SUB RASP_FN_B RASP_FN_PT_CLASSIC RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FN_OPERANDS);
+    asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
+        RASP_FN_A RASP_FN_SUB RASP_FN_B RASP_FN_ST2 RASP_FN_PT_CLASSIC
+        RASP_F_NEXT(RASP_F_FETCH_GL))
+                 RASP_FN_OPERANDS);
   } else {
-    asm volatile(RASP_FN_A RASP_FN_MUL RASP_FN_B RASP_FN_PT_WORD RASP_F_NEXT(RASP_F_FETCH_GL) RASP_FN_OPERANDS);
+    asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
+        RASP_FN_A RASP_FN_MUL RASP_FN_B RASP_FN_ST2 RASP_FN_PT_WORD
+        RASP_F_NEXT(RASP_F_FETCH_GL))
+                 RASP_FN_OPERANDS);
   }
 }
 

@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) k_pack(DevState S, const W* __restrict__ 
 template <class W>
 __global__ void __launch_bounds__(128) k_fuse(const W* __restrict__ prog, const uint64_t* __restrict__ prog_off,
                                               const uint32_t* __restrict__ bound, uint32_t num_programs,
-                                              uint64_t wmask, uint32_t classic, uint32_t own, uint4* tmp,
+                                              uint64_t wmask, uint32_t classic, uint32_t own, uint32_t two, uint4* tmp,
                                               uint4* __restrict__ out, uint4* recs) {
   for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < num_programs; p += gridDim.x * blockDim.x) {
     const uint64_t po = prog_off[p];
@@ -155,10 +155,10 @@ __global__ void __launch_bounds__(128) k_fuse(const W* __restrict__ prog, const 
       while (want & ~done) {
         const uint32_t e = 64u * k + (uint32_t)__ffsll((long long)(want & ~done)) - 1u;
         done |= 1ull << (e & 63u);
-        const uint4 x = fuse_one(prog + po, e, plen, n, mok, wmask, classic != 0u, own != 0u);
+        const uint4 x = fuse_one(prog + po, e, plen, n, mok, wmask, classic != 0u, own != 0u, two != 0u);
         t[e] = x;
         entries += 1u;
-        uint32_t next[2] = {x.w >> 16, x.w & 0xFFFFu};
+        uint32_t next[2] = {x.w >> 16, x.y & FO_BNZ ? x.w & 0xFFFFu : x.w >> 16};
         if (!(x.y & FO_COUNT)) {                         // a stall: where its instruction may go on
           const ulonglong2 oj = fuse_pair(prog + po, 2u * e, wmask);
           const bool valid = oj.x - 1ull < 7ull;
@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(128) k_fuse(const W* __restrict__ prog, const 
         const uint32_t e = 64u * k + (uint32_t)__ffsll((long long)m) - 1u;
         uint4 x = t[e];
         const uint32_t a = x.w & 0xFFFFu, f = x.w >> 16;
-        x.w = fuse_rank(rec[a >> 6], a) | (fuse_rank(rec[f >> 6], f) << 16);
+        const uint32_t taken = (x.y & FO_COUNT) && (x.y & FO_BNZ) ? fuse_rank(rec[a >> 6], a) : a;
+        x.w = taken | (fuse_rank(rec[f >> 6], f) << 16);
         *dst++ = x;
       }
     }
@@ -362,7 +363,7 @@ __device__ __forceinline__ void run_epoch(Mem M, const uint64_t* T, uint64_t* Y,
 // it wrote into its program, or its i lies outside them for a few steps --
 // runs from its memory (run_epoch_loop, which does not watch its writes) until
 // the next pack.
-constexpr uint32_t kFuseChunk = 8;     // entries between two looks at the stalled lanes
+constexpr uint32_t kFuseChunk = 16;    // entries between two looks at the stalled lanes (uneven 4.95 -> 4.85 ms, from 8)
 constexpr uint32_t kFuseOutside = 32;  // general steps at no entry's start before a VM leaves them: more than an
                                        // entry holds (a run that a stop has cut goes on inside an entry)
 
@@ -376,7 +377,7 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
   if (fm) {
     const uint32_t wait = idle_exit ? idle_exit : 8u;
     const uint32_t zero = P.ellp & 1u;                   // the stride of the tapes is even
-    for (uint32_t it = (epoch + 1u) / 2u; it;) {
+    for (uint32_t it = (epoch + 3u) / 4u * 2u; it;) {
       const uint32_t c = min(it, kFuseChunk);
       it -= c;
       if (active && F.on) {
@@ -400,7 +401,7 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
       if (sm == fm || (uint32_t)__popc(sm) >= wait) break;
     }
   }
-  if (stall && F.on && (F.op.y & FO_HALT)) {
+  if (stall && F.on && !(F.op.y & FO_COUNT) && (F.op.y & FO_HALT)) {
     r.ip = 2u * F.op.x;
     active = false;
     final_st = ST_HALTED;
@@ -1390,17 +1391,17 @@ cudaError_t launch_pack(const DevState& S, const uint64_t* prog, const int32_t* 
 }
 
 cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint64_t* prog_off, const uint32_t* bound,
-                        uint32_t num_programs, uint64_t wmask, bool classic, bool own, uint4* tmp, uint4* out,
+                        uint32_t num_programs, uint64_t wmask, bool classic, bool own, bool two, uint4* tmp, uint4* out,
                         uint4* recs, cudaStream_t stream) {
   if (!num_programs) return cudaSuccess;
   uint32_t blocks = (num_programs + 127u) / 128u;
   const uint32_t cap = (uint32_t)num_sms() * 16u;   // more blocks gain nothing (latency of each lane's scan)
   if (blocks > cap) blocks = cap;
   if (prog32)
-    k_fuse<int32_t><<<blocks, 128, 0, stream>>>(prog32, prog_off, bound, num_programs, wmask, classic, own, tmp, out,
+    k_fuse<int32_t><<<blocks, 128, 0, stream>>>(prog32, prog_off, bound, num_programs, wmask, classic, own, two, tmp, out,
                                                 recs);
   else
-    k_fuse<uint64_t><<<blocks, 128, 0, stream>>>(prog, prog_off, bound, num_programs, wmask, classic, own, tmp, out,
+    k_fuse<uint64_t><<<blocks, 128, 0, stream>>>(prog, prog_off, bound, num_programs, wmask, classic, own, two, tmp, out,
                                                  recs);
   return cudaGetLastError();
 }
