@@ -777,6 +777,85 @@ __device__ __forceinline__ uint32_t fast_loop_ptx_sh(uint64_t* M, const uint64_t
   return rare;
 }
 
+// The epoch loop under CHECKED semantics (w = 64): the steps of fast_loop_ptx
+// with signed overflow of ADD and MUL (SUB in the classic set) among the
+// guards. It depends on the operand, so operand and next pair are loaded
+// before the vote (both together, the pair into registers of its own), and
+// nothing is applied before it. An address or fetch outside [0, n) leaves the
+// loop as in fast_loop_ptx, and the general step finds the fault.
+#define RASP_CLOOP_B \
+      RASP_LOOP_B1 \
+      "and.pred pq, po, pad;\n\t" \
+      "or.pred px, px, pq;\n\t" \
+      "setp.eq.u32 p6, ol, 6;\n\t" \
+      "setp.ge.and.u32 pq, %4, %14, p6;\n\t" \
+      "or.pred px, px, pq;\n\t" \
+      "setp.eq.and.u32 pq, jl, %3, pt;\n\t" \
+      "or.pred px, px, pq;\n\t" \
+      "and.b32 t0, m, 0x8C;\n\t" \
+      "setp.ne.and.u32 pop, t0, 0, !px;\n\t" \
+      "mad.wide.u32 ado, jl, 8, %9;\n\t" \
+      "@pop ld.global.u64 v, [ado];\n\t" \
+      "add.u32 nip, %3, 2;\n\t" \
+      "selp.b32 nip, jl, nip, pt;\n\t" \
+      "shf.l.wrap.b32 t1, nip, nip, 31;\n\t" \
+      "setp.lt.and.u32 pe, t1, %13, !px;\n\t" \
+      "mad.wide.u32 adn, nip, 8, %9;\n\t" \
+      "@pe ld.global.v2.u64 {no, nj}, [adn];\n\t" \
+      "setp.eq.u32 p2, ol, 2;\n\t" \
+      "setp.eq.u32 p3, ol, 3;\n\t" \
+      "add.u64 sm, %0, v;\n\t" \
+      "xor.b64 x1, %0, sm;\n\t" \
+      "xor.b64 x2, v, sm;\n\t" \
+      "and.b64 x1, x1, x2;\n\t" \
+      "setp.lt.and.s64 pq, x1, 0, p2;\n\t" \
+      "or.pred px, px, pq;\n\t"
+#define RASP_CLOOP_MUL \
+      "mul.lo.u64 pd, %0, v;\n\t" \
+      "mul.hi.s64 x1, %0, v;\n\t" \
+      "shr.s64 x2, pd, 63;\n\t" \
+      "setp.ne.and.s64 pq, x1, x2, p3;\n\t"
+#define RASP_CLOOP_SUB \
+      "sub.u64 pd, %0, v;\n\t" \
+      "xor.b64 x1, %0, v;\n\t" \
+      "xor.b64 x2, %0, pd;\n\t" \
+      "and.b64 x1, x1, x2;\n\t" \
+      "setp.lt.and.s64 pq, x1, 0, p3;\n\t"
+#define RASP_CLOOP_C \
+      "or.pred px, px, pq;\n\t" \
+      "vote.sync.any.pred pany, px, %16;\n\t" \
+      "@pany bra.uni RASP_DONE;\n\t" \
+      "mov.b32 %3, nip;\n\t" \
+      "xor.b32 t1, jl, nip;\n\t" \
+      "setp.eq.u32 p1, ol, 1;\n\t" \
+      "mad.wide.u32 adt, %4, 8, %10;\n\t" \
+      "@p6 ld.global.u64 tv, [adt];\n\t" \
+      "setp.eq.u32 p4, ol, 4;\n\t" \
+      "@p4 st.global.u64 [ado], %0;\n\t" \
+      "@p6 st.global.u64 [ado], tv;\n\t" \
+      "or.pred pw, p4, p6;\n\t" \
+      "@p1 mov.b64 %0, %2;\n\t" \
+      "@p2 mov.b64 %0, sm;\n\t" \
+      "@p3 mov.b64 %0, pd;\n\t" \
+      "@pe mov.b64 %1, no;\n\t" \
+      "@pe mov.b64 %2, nj;\n\t"
+template <bool CLASSIC>
+__device__ __forceinline__ uint32_t fast_loop_ptx_checked(uint64_t* M, const uint64_t* T, uint64_t* Y, uint32_t n,
+                                                          uint32_t ell, uint32_t s, uint32_t ilim, uint64_t wmask,
+                                                          uint32_t mask, uint64_t& a, uint64_t& co, uint64_t& cj,
+                                                          uint32_t& ip, uint32_t& u0, uint32_t& y0, uint32_t& have,
+                                                          uint32_t& kk) {
+  uint32_t rare;
+  if constexpr (CLASSIC) {
+    asm volatile("{\n\t.reg .b64 no, nj, sm, pd, x1, x2;\n\t" RASP_LOOP_A RASP_LOOP_PZ_CLASSIC RASP_CLOOP_B
+                 RASP_CLOOP_SUB RASP_CLOOP_C RASP_LOOP_D "\n\t}" RASP_LOOP_OPERANDS);
+  } else {
+    asm volatile("{\n\t.reg .b64 no, nj, sm, pd, x1, x2;\n\t" RASP_LOOP_A RASP_LOOP_PZ_WORD RASP_CLOOP_B
+                 RASP_CLOOP_MUL RASP_CLOOP_C RASP_LOOP_D "\n\t}" RASP_LOOP_OPERANDS);
+  }
+  return rare;
+}
+
 // The epoch loop of a narrow batch (w <= 32, M in 4-byte words): the same
 // steps as fast_loop_ptx with 32-bit words and 32-bit arithmetic (every word
 // and a are below 2^w <= 2^32, so a word's high half is never looked at and
@@ -980,7 +1059,7 @@ __device__ __forceinline__ uint32_t one_step(Mem M, const uint64_t* __restrict__
 }
 
 // Run up to `epoch` steps of every active lane with the epoch loop of
-// fast_loop_ptx (WRAP, no counters, select dispatch). Each round runs the
+// fast_loop_ptx (no counters, select dispatch; CHECKED on 8-byte slabs). Each round runs the
 // loop for at most the smallest step countdown of the warp; then the lanes
 // whose step needs the general path (the loop left by a warp vote, nothing
 // of that step applied) or whose countdown ended take one step with
@@ -988,7 +1067,7 @@ __device__ __forceinline__ uint32_t one_step(Mem M, const uint64_t* __restrict__
 // with general steps counts one more step of the epoch, so the epoch always
 // ends. With idle_exit > 0 the epoch also ends once that many lanes that were
 // running at its start have stopped, so that they are refilled sooner.
-template <bool MASKED, bool CLASSIC, class Mem>
+template <bool MASKED, bool CLASSIC, bool CHECKED = false, class Mem>
 __device__ __forceinline__ void run_epoch_loop(Mem M, const uint64_t* T, uint64_t* Y, const Params& P,
                                                Regs& r, Hist& h, bool& active, uint32_t& final_st, uint32_t epoch,
                                                uint32_t idle_exit) {
@@ -1029,6 +1108,9 @@ __device__ __forceinline__ void run_epoch_loop(Mem M, const uint64_t* T, uint64_
           // M, tape and y in shared memory: generic addresses, word opcode set
           rare = fast_loop_ptx_gen<MASKED>(M.M, T, Y, r.n, P.ell, P.s, r.ilim, P.wmask, mask, r.a, co, cj, r.ip,
                                            r.u0, r.y0, hv, kk);
+        } else if constexpr (CHECKED) {
+          rare = fast_loop_ptx_checked<CLASSIC>(M, T, Y, r.n, P.ell, P.s, r.ilim, P.wmask, mask, r.a, co, cj, r.ip,
+                                                r.u0, r.y0, hv, kk);
         } else {
           rare = fast_loop_ptx<MASKED, CLASSIC>(M, T, Y, r.n, P.ell, P.s, r.ilim, P.wmask, mask, r.a, co, cj, r.ip,
                                                 r.u0, r.y0, hv, kk);
@@ -1048,7 +1130,7 @@ __device__ __forceinline__ void run_epoch_loop(Mem M, const uint64_t* T, uint64_
           r.ibase = i - r.ip;
         }
         r.have = false;
-        const uint32_t st = step_general<MASKED, false, false, CLASSIC>(M, T, Y, P, r, h);
+        const uint32_t st = step_general<MASKED, CHECKED, false, CLASSIC>(M, T, Y, P, r, h);
         if (st == CONT) {
           prime(M, r);
         } else {

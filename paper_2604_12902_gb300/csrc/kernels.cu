@@ -568,7 +568,7 @@ template <bool MASKED, bool CHECKED, bool HIST, bool VOTE, bool CLASSIC = false,
           bool NARROW = false, bool FUSE = false>
 __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Queue Q, uint32_t epoch,
                                                        uint32_t idle_exit) {
-  static_assert(!LOOP || (!CHECKED && !HIST && !VOTE), "the epoch loop serves WRAP select steps without counters");
+  static_assert(!LOOP || (!HIST && !VOTE), "the epoch loop serves select steps without counters");
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t lt = (1u << lane) - 1u;
   Hist h;
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
     // ---- run
     if constexpr (FUSE) run_epoch_fused<MASKED, CLASSIC>(M, T, Y, P, r, F, S, (uint32_t)vm, h, active, final_st, epoch,
                                                             idle_exit);
-    else if constexpr (LOOP) run_epoch_loop<MASKED, CLASSIC>(M, T, Y, P, r, h, active, final_st, epoch, idle_exit);
+    else if constexpr (LOOP) run_epoch_loop<MASKED, CLASSIC, CHECKED>(M, T, Y, P, r, h, active, final_st, epoch, idle_exit);
     else run_epoch<MASKED, CHECKED, HIST, VOTE, true, CLASSIC>(M, T, Y, P, r, h, active, final_st, epoch);
   }
   flush_hist<HIST>(P, h);
@@ -843,10 +843,8 @@ __global__ void __launch_bounds__(128, 6) k_serve(ServeArgs A, Params P0) {
             M = sd.S.mem + moff;
             T = sd.S.tape + (uint64_t)v * P.ellp;
             Y = sd.S.y + (uint64_t)v * P.sp;
-            if (!CHECKED) {
-              fuse_attach(sd.S, v, r, F);
-              if (!F.on) prime(M, r);
-            }
+            if (!CHECKED) fuse_attach(sd.S, v, r, F);
+            if (!F.on) prime(M, r);
             active = true;
           } else {
             serve_finish(A, sl);                // already stopped: nothing to run
@@ -885,7 +883,7 @@ __global__ void __launch_bounds__(128, 6) k_serve(ServeArgs A, Params P0) {
     idle = 0;
     // ---- run an epoch
     if constexpr (CHECKED) {
-      run_epoch<MASKED, true, false, false, false, CLASSIC>(M, T, Y, P, r, h, active, final_st, A.epoch);
+      run_epoch_loop<MASKED, CLASSIC, true>(M, T, Y, P, r, h, active, final_st, A.epoch, 0u);
     } else {
       run_epoch_fused<MASKED, CLASSIC>(M, T, Y, P, r, F, A.slots[slot < 0 ? 0 : slot].S, vm, h, active, final_st,
                                        A.epoch, 0u);
@@ -1286,7 +1284,8 @@ GlobalFn global_select(const StepVariant& v) {
                   : k_persist_gl<true, false, false, false, CL, true, true>;
   }
   if (v.checked)
-    return v.hist ? k_persist_gl<false, true, true, false, CL> : k_persist_gl<false, true, false, false, CL>;
+    return v.hist ? k_persist_gl<false, true, true, false, CL>
+                  : (v.block ? k_persist_gl<false, true, false, false, CL> : k_persist_gl<false, true, false, false, CL, true>);
   if (v.masked)
     return v.hist ? k_persist_gl<true, false, true, false, CL>
                   : (v.block ? k_persist_gl<true, false, false, false, CL>

@@ -93,8 +93,8 @@ __global__ void __launch_bounds__(256) k_static_compact(const uint8_t* __restric
 
 // Persistent warps over the queued ids: each lane runs one VM (memory in
 // HBM) until it stops, then the warp claims new ids for its idle lanes. The
-// steps run as epochs of run_epoch_loop (32,768 template programs: 0.68 -> 0.45 ms a call, against one step at a time),
-// CHECKED ones one at a time.
+// steps run as epochs of run_epoch_loop (32,768 template programs: 0.68 ->
+// 0.45 ms a call, against one step at a time).
 template <bool MASKED, bool CHECKED>
 __global__ void __launch_bounds__(128) k_static_persist(DevState S, Params P, uint32_t* __restrict__ scratch,
                                                         uint32_t epoch) {
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(128) k_static_persist(DevState S, Params P, ui
           M = S.mem + S.mem_off[vm];
           T = S.tape + (uint64_t)vm * P.ellp;
           Y = S.y + (uint64_t)vm * P.sp;
-          if (!CHECKED) prime(M, r);
+          prime(M, r);
           active = true;
         } else {
           exhausted = true;
@@ -135,18 +135,7 @@ __global__ void __launch_bounds__(128) k_static_persist(DevState S, Params P, ui
       }
     }
     if (__all_sync(0xffffffffu, exhausted && !active)) break;
-    if constexpr (!CHECKED) {
-      run_epoch_loop<MASKED, false>(M, T, Y, P, r, h, active, final_st, epoch, 0u);
-    } else if (active) {
-      for (uint32_t t = 0; t < epoch; ++t) {
-        const uint32_t s = one_step<false, true, false, false>(M, T, Y, P, r, h);
-        if (s != CONT) {
-          active = false;
-          final_st = s;
-          break;
-        }
-      }
-    }
+    run_epoch_loop<MASKED, false, CHECKED>(M, T, Y, P, r, h, active, final_st, epoch, 0u);
     if (vm >= 0 && !active) {
       store_regs(S, (uint32_t)vm, r, final_st);
       vm = -1;

@@ -104,6 +104,27 @@ def test_shared_program_schedule(rasp, m, w):
               i32=m != 40)
 
 
+@pytest.mark.parametrize("classic", [False, True])
+@pytest.mark.parametrize("m", [8, 64])
+def test_checked_loop(rasp, m, classic):
+    """The epoch loop under CHECKED semantics: overflows of large data at every
+    step of a run, faulting addresses and fetches, runs stopped and resumed."""
+    wl = machines(900, m, 64, seed=30 + m)
+    rng = np.random.default_rng(m)
+    big = rng.integers(-(1 << 31), 1 << 31, wl.tapes.size) << rng.choice([0, 16, 32], wl.tapes.size)
+    wl.tapes = big.astype(np.int64)
+    prog = wl.programs.reshape(900, -1)
+    prog[:, 0:2 * min(4, m // 2):2], prog[:, 1:2 * min(4, m // 2):2] = RD, 2 * m + np.arange(min(4, m // 2))
+    flags = rasp.ISA_CLASSIC if classic else 0
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s, semantics=rasp.CHECKED, flags=flags) as b:
+        b.load_workload(wl)
+        for t in (5, 6, 100, 1000):
+            b.run(t)
+            st, _ = oracle_state(wl, budget=t, threads=8, checked=True, classic=classic)
+            assert_same_state(b.read_state(), st, wl.ell, wl.s, what="checked, budget %d" % t)
+    assert {3, 4} <= set(st.status.tolist()) and (st.steps[st.status == 3] > 6).any()
+
+
 def test_self_writing_programs(rasp):
     """Batches in which all, some or few programs mostly write into themselves."""
     a = W.random_programs(num_vms=512, seed=3, mem_words=200)
