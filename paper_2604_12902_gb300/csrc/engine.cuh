@@ -67,6 +67,7 @@ struct Queue {
   const uint32_t* dcount;     // persistent HBM-slab kernel: if set, the number of ids is read
                               // here at launch (written by an earlier kernel on the stream) and
                               // soft_end is derived from it
+  uint32_t lanes;             // lanes of each warp that take VMs (set by the launcher)
 };
 
 // Registers of one machine while it runs. The instruction counter is kept
