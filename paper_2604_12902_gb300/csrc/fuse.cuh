@@ -69,136 +69,109 @@ __device__ __forceinline__ ulonglong2 fuse_pair(const int32_t* src, uint32_t k, 
   return make_ulonglong2((uint64_t)(int64_t)q.x & wmask, (uint64_t)(int64_t)q.y & wmask);
 }
 
-// The entry of instruction e of a program of `plen` words (src) on memories of
-// at least n words: `mok` instructions lie where i (+) 2 and the pair need no
-// reduction. own: M holds the program words (they may be read as data).
-// The state of the scan is the next free part of the form (stage 0 imm1,
-// 1 op, 2 store, 3 imm2, 4 add, 5 second store or jump) and a constant not yet
-// placed. two: entries may hold the second store. It takes the slowest loops of
-// the halting workload from 3.1 to 4.0 VM-steps per entry (run of 2^18 programs
-// 121 -> 92 ms), and costs 6 of about 65 instructions on 8-byte words, where
-// the template and uneven batches gain little from it (1.96 -> 2.05 ms).
-template <class W>
-__device__ __forceinline__ uint4 fuse_one(const W* src, uint32_t e, uint32_t plen, uint32_t n, uint32_t mok,
-                                          uint64_t wmask, bool classic, bool own, bool two) {
-  uint32_t p = e, stage = 0, cnt = 0, flags = 0, j1 = 0, k = 0, j2 = 0, i1 = 0, i2 = 0, t = e, f = e;
-  bool pend = false;
-  uint64_t cv = 0;
-  while (cnt < kFuseMaxCount) {
-    const ulonglong2 oj = fuse_pair(src, 2u * p, wmask);
-    const uint64_t j = oj.y;
-    if (oj.x - 1ull >= 7ull) break;
-    const uint32_t op = (uint32_t)oj.x;
+// The scan of one run: instructions are taken as long as they fit. Its state is
+// the next free part of the form (stage 0 imm1, 1 op, 2 store, 3 imm2, 4 add,
+// 5 second store or jump) and a constant in a that is not yet placed.
+// plen: words of the program; n: the smallest memory that runs it; mok:
+// instructions whose pair and i (+) 2 need no reduction; own: M holds the
+// program words (they may be read as data); two: entries may hold the second
+// store. It takes the slowest loops of the halting workload from 3.1 to 4.0
+// VM-steps per entry (run of 2^18 programs 121 -> 92 ms), and costs 6 of about
+// 65 instructions on 8-byte words, where the template and uneven batches gain
+// little from it (1.96 -> 2.05 ms).
+struct FuseScan {
+  uint32_t e, p, stage, cnt, flags, j1, k, j2, i1, i2, t, cv;
+  bool pend, jump;      // a holds the constant cv (16 bits); a jump on it is taken
+
+  __device__ __forceinline__ void start(uint32_t at) {
+    e = p = at;
+    stage = cnt = flags = j1 = k = j2 = i1 = i2 = cv = 0u;
+    t = at;
+    pend = jump = false;
+  }
+
+  // Take instruction (o, j) at p; false when the run has ended (at p).
+  __device__ __forceinline__ bool step(uint64_t o, uint64_t j, uint32_t plen, uint32_t n, uint32_t mok,
+                                       uint64_t wmask, bool classic, bool own, bool two) {
+    const uint32_t op = o - 1ull < 7ull ? (uint32_t)o : 0u;
+    const uint32_t jm = (uint32_t)j;
+    const bool room = p + 1u < mok;
+    bool ok = room, go = true;
+    uint32_t np = p + 1u;
     if (op == 5u) {
-      const bool target = !(j & 1ull) && (j >> 1) < (uint64_t)mok && j != 2ull * p;
+      const bool target = !(jm & 1u) && (j >> 1) < (uint64_t)mok && jm != 2u * p;
       if (pend) {                                        // a is a constant: the jump is decided
-        const bool taken = classic ? (cv - 1ull) < (wmask >> 1) : cv != 0ull;
-        if (taken ? !target : p + 1u >= mok) break;
-        p = taken ? (uint32_t)(j >> 1) : p + 1u;
-        cnt += 1u;
-        continue;
-      }
-      if (!target || p + 1u >= mok || (flags & FO_ST2)) break;
-      flags |= FO_BNZ;
-      t = (uint32_t)(j >> 1);
-      p += 1u;
-      cnt += 1u;
-      break;
-    }
-    if (p + 1u >= mok) break;
-    if (op == 1u) {
-      if (stage > 3u) break;
-      const uint64_t sx = (uint64_t)(int64_t)(int16_t)(uint16_t)j & wmask;
-      if (sx == j) {
-        pend = true;
-        cv = j;
-      } else {                                           // a wide constant: read from the program word itself
-        if (!own || 2u * p + 1u > 0xFFFFu) break;
-        if (stage == 0u) {
-          flags |= FO_L1 | FO_ADD;
-          j1 = 2u * p + 1u;
-          stage = 2u;
-        } else {
-          flags |= FO_L2 | FO_LD2;
-          j2 = 2u * p + 1u;
-          stage = 5u;
-        }
-        pend = false;
-      }
-    } else {
-      if (j >= (uint64_t)n || j > 0xFFFFull) break;
-      const uint32_t jm = (uint32_t)j;
-      const bool code = jm < plen;
-      if (code && (op == 4u || op == 6u || !own)) break;
-      // a constant is placed in imm1 while the form is empty
-      const bool first = pend && stage == 0u;
-      if (op == 2u && (stage <= 1u && (!pend || first))) {
-        flags |= FO_ADD;
-        j1 = jm;
-        stage = 2u;
-      } else if (op == 2u && stage <= (pend ? 3u : 4u)) {
-        if ((flags & FO_RD) && jm == k) break;           // the tape word is not at hand
-        if (pend) {
-          flags |= FO_L2;
-          i2 = (uint32_t)cv & 0xFFFFu;
-          pend = false;
-        }
-        flags |= (flags & FO_STO) && jm == k ? FO_FWD : FO_LD2;
-        j2 = jm;
-        stage = 5u;
-      } else if (op == 3u && stage <= 1u && (!pend || first)) {
-        flags |= FO_MUL;
-        j1 = jm;
-        stage = 2u;
-      } else if (op == 4u && stage <= 2u && (!pend || first)) {
-        flags |= FO_STO;
-        k = jm;
-        stage = 3u;
-      } else if (op == 4u && two && stage <= (pend ? 3u : 5u)) {
-        if (pend) {
-          flags |= FO_L2;
-          i2 = (uint32_t)cv & 0xFFFFu;
-          pend = false;
-        }
-        flags |= FO_ST2;
-        t = jm;
-        stage = 6u;
-      } else if (op == 6u && stage <= 2u) {
-        flags |= FO_RD;
-        k = jm;
-        stage = 3u;
-      } else if (op == 7u && stage <= 1u) {
-        flags |= FO_PRI;
-        j1 = jm;
-        stage = 2u;
+        ok = jump ? target : room;
+        np = jump ? jm >> 1 : np;
       } else {
-        break;
+        ok = target && room && !(flags & FO_ST2);
+        if (ok) {
+          flags |= FO_BNZ;
+          t = jm >> 1;
+        }
+        go = false;
       }
-      if (first) {
-        flags |= FO_L1;
-        i1 = (uint32_t)cv & 0xFFFFu;
-        pend = false;
+    } else if (op == 1u) {
+      const bool small = ((uint64_t)(int64_t)(int16_t)(uint16_t)j & wmask) == j;
+      ok = room && stage <= 3u && (small || (own && 2u * p + 1u <= 0xFFFFu));
+      if (ok) {
+        pend = small;
+        cv = jm & 0xFFFFu;
+        jump = classic ? j - 1ull < (wmask >> 1) : j != 0ull;
+        if (!small) {                                    // a wide constant: 0 + the program word itself
+          const bool first = stage == 0u;
+          flags |= first ? FO_L1 | FO_ADD : FO_L2 | FO_LD2;
+          j1 = first ? 2u * p + 1u : j1;
+          j2 = first ? j2 : 2u * p + 1u;
+          stage = first ? 2u : 5u;
+        }
       }
-    }
-    p += 1u;
-    cnt += 1u;
-  }
-  if (pend) {                                            // the constant that a holds after the run
-    if (stage == 0u) {
-      flags |= FO_L1;
-      i1 = (uint32_t)cv & 0xFFFFu;
     } else {
-      flags |= FO_L2;
-      i2 = (uint32_t)cv & 0xFFFFu;
+      // parts that take an address, by opcode 2 ADD, 3 MUL, 4 STO, 6 RD, 7 PRI:
+      // the last stage that may take it, the stage behind it, its flag; RD and
+      // PRI do not use a, so a constant may wait past them
+      const uint32_t at = 4u * op;
+      const uint32_t last = (0x12021100u >> at) & 15u, behind = (0x23032200u >> at) & 15u;
+      const uint32_t flag = op == 2u ? FO_ADD : op == 3u ? FO_MUL : op == 4u ? FO_STO : op == 6u ? FO_RD : FO_PRI;
+      const bool code = jm < plen, store = op == 4u || op == 6u;
+      const bool one = stage <= last && (!pend || stage == 0u || op >= 6u);
+      const bool late = !one && stage <= (pend ? 3u : op == 2u ? 4u : 5u) &&
+                        (op == 2u ? !((flags & FO_RD) && jm == k) : op == 4u && two);
+      ok = room && op != 0u && j < (uint64_t)n && j <= 0xFFFFull && !(code && (store || !own)) && (one || late);
+      if (ok) {
+        if (pend && (one ? stage == 0u : true)) {        // the constant's place: imm1 while the form is empty
+          flags |= one ? FO_L1 : FO_L2;
+          i1 = one ? cv : i1;
+          i2 = one ? i2 : cv;
+          pend = false;
+        }
+        const uint32_t second = op == 4u ? FO_ST2 : ((flags & FO_STO) && jm == k ? FO_FWD : FO_LD2);
+        flags |= one ? flag : second;
+        j1 = one && !store ? jm : j1;
+        k = one && store ? jm : k;
+        j2 = !one && op == 2u ? jm : j2;
+        t = !one && op == 4u ? jm : t;
+        stage = one ? behind : (op == 2u ? 5u : 6u);
+      }
     }
+    if (ok) {
+      p = np;
+      cnt += 1u;
+    }
+    return ok && go && cnt < kFuseMaxCount;
   }
-  if (!cnt) {
-    const bool halt = fuse_pair(src, 2u * e, wmask).x - 1ull >= 7ull;
-    return make_uint4(e, halt ? FO_HALT : 0u, 0u, e | (e << 16));
+
+  // The entry, once the run has ended at an instruction of opcode o.
+  __device__ __forceinline__ uint4 entry(uint64_t o) {
+    if (!cnt) return make_uint4(e, o - 1ull >= 7ull ? FO_HALT : 0u, 0u, e | (e << 16));
+    if (pend) {                                          // the constant that a holds after the run
+      flags |= stage == 0u ? FO_L1 : FO_L2;
+      i1 = stage == 0u ? cv : i1;
+      i2 = stage == 0u ? i2 : cv;
+    }
+    return make_uint4(j1 | (k << 16), j2 | flags | (cnt << 16), i1 | (i2 << 16), t | (p << 16));
   }
-  f = p;
-  return make_uint4(j1 | (k << 16), j2 | flags | (cnt << 16), i1 | (i2 << 16), t | (f << 16));
-}
+};
 
 // ------------------------------------------------------------------ the lane's side
 // A VM's data view while it takes general steps beside the fused loop: a
@@ -297,13 +270,31 @@ __device__ __forceinline__ void fuse_enter(const FuseProg& G, Fused& F, const Re
   F.op = __ldg(G.tab + q);
 }
 
+// What fuse_attach reads of VM v before its registers are armed, so that a
+// kernel can issue these loads beside the registers'.
+struct FuseRow {
+  uint64_t po, pe;      // the program's words
+  uint32_t p;
+  uint32_t dirty;
+};
+__device__ __forceinline__ FuseRow fuse_row(const DevState& S, uint32_t v) {
+  FuseRow w;
+  w.dirty = S.codedirty[v];
+  w.p = S.prog_of_vm ? S.prog_of_vm[v] : v;
+  w.po = S.prog_off[w.p];
+  w.pe = S.prog_off[w.p + 1];
+  return w;
+}
+
 // VM v's entries (after arm_regs); without them it runs one instruction at a time.
-__device__ __forceinline__ void fuse_attach(const DevState& S, uint32_t v, Regs& r, Fused& F) {
-  F.on = false;
-  r.clean = false;
-  if (S.fops == nullptr || S.codedirty[v]) return;
-  r.clean = true;
-  fuse_enter(fuse_prog(S, v, r.ilim), F, r);
+__device__ __forceinline__ void fuse_attach(const DevState& S, const FuseRow& w, Regs& r, Fused& F) {
+  r.clean = w.dirty == 0u;
+  FuseProg G;
+  G.plen = (uint32_t)(w.pe - w.po);
+  G.mok = min(G.plen, r.ilim) >> 1;
+  G.tab = S.fops + (w.po >> 1);
+  G.rec = S.frec + (w.po >> 7) + w.p;
+  fuse_enter(G, F, r);
   if (F.on && !(F.op.y & FO_COUNT) && (F.op.y & FO_MEM)) F.on = r.clean = false;
 }
 

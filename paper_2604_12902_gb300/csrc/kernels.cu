@@ -126,10 +126,10 @@ __global__ void __launch_bounds__(256) k_pack(DevState S, const W* __restrict__ 
 // The fused entries of every program (fuse.cuh), one program per lane: the
 // entries reached from instruction 0 are decoded one after the other (an
 // entry names the next ones), kept by instruction in `tmp`, and then written
-// densely with their jumps renumbered. A lane reads only the instructions
-// that runs start at, about 1.1 times each: 1M template programs in 0.3 ms,
-// against 2.6 ms with one instruction per lane (7 of 32 lanes active, every
-// run of every instruction decoded).
+// densely with their jumps renumbered. One turn of the loop takes one
+// instruction in every lane, whatever run it is in. 262,144 template programs
+// take 0.43 ms (16 of 32 lanes active, issue slots half used); with one
+// instruction per lane and every entry decoded 0.65 ms (7 lanes active).
 // bound: the smallest memory that runs program p. tmp: 16 bytes per
 // instruction (at half the program's offset).
 template <class W>
@@ -148,40 +148,52 @@ __global__ void __launch_bounds__(128) k_fuse(const W* __restrict__ prog, const 
     for (uint32_t k = 0; k < nrec; ++k) rec[k] = make_uint4(k == 0u && mok ? 1u : 0u, 0u, 0u, 0u);
     uint32_t entries = 0, writes = 0;                    // reached, and of them writes into the program
     // records in order; a target before the current record starts over from there
-    for (uint32_t k = 0; k < nrec;) {
-      uint32_t back = ~0u;
-      uint4 r = rec[k];
-      uint64_t want = fuse_mask(r), done = ((uint64_t)r.w << 32) | r.z;
-      while (want & ~done) {
-        const uint32_t e = 64u * k + (uint32_t)__ffsll((long long)(want & ~done)) - 1u;
-        done |= 1ull << (e & 63u);
-        const uint4 x = fuse_one(prog + po, e, plen, n, mok, wmask, classic != 0u, own != 0u, two != 0u);
-        t[e] = x;
-        entries += 1u;
-        uint32_t next[2] = {x.w >> 16, x.y & FO_BNZ ? x.w & 0xFFFFu : x.w >> 16};
-        if (!(x.y & FO_COUNT)) {                         // a stall: where its instruction may go on
-          const ulonglong2 oj = fuse_pair(prog + po, 2u * e, wmask);
-          const bool valid = oj.x - 1ull < 7ull;
-          writes += (oj.x == 4ull || oj.x == 6ull) && oj.y < (uint64_t)plen ? 1u : 0u;
-          next[0] = valid && e + 1u < mok ? e + 1u : e;
-          next[1] = oj.x == 5ull && !(oj.y & 1ull) && (oj.y >> 1) < (uint64_t)mok ? (uint32_t)(oj.y >> 1) : e;
-        }
-        for (uint32_t q = 0; q < 2u; ++q) {
-          const uint32_t kk = next[q] >> 6;
-          const uint64_t bit = 1ull << (next[q] & 63u);
-          if (kk == k) {
-            want |= bit;
-          } else {
-            const uint4 o = rec[kk];
-            if (!(fuse_mask(o) & bit)) {
-              rec[kk] = make_uint4(o.x | (uint32_t)bit, o.y | (uint32_t)(bit >> 32), o.z, o.w);
-              if (kk < k) back = min(back, kk);
-            }
+    uint32_t k = 0, back = ~0u;
+    uint64_t want = mok ? 1ull : 0ull, done = 0;
+    FuseScan f;
+    f.start(0u);
+    bool more = mok != 0u;
+    while (more) {
+      const ulonglong2 oj = fuse_pair(prog + po, 2u * f.p, wmask);
+      if (f.step(oj.x, oj.y, plen, n, mok, wmask, classic != 0u, own != 0u, two != 0u)) continue;
+      // the run has ended: its entry, the instructions it goes on to, the next one to decode
+      t[f.e] = f.entry(oj.x);
+      entries += 1u;
+      uint32_t next[2] = {f.p, f.flags & FO_BNZ ? f.t : f.p};
+      if (!f.cnt) {                                      // a stall: where its instruction may go on
+        const bool valid = oj.x - 1ull < 7ull;
+        writes += (oj.x == 4ull || oj.x == 6ull) && oj.y < (uint64_t)plen ? 1u : 0u;
+        next[0] = valid && f.e + 1u < mok ? f.e + 1u : f.e;
+        next[1] = oj.x == 5ull && !(oj.y & 1ull) && (oj.y >> 1) < (uint64_t)mok ? (uint32_t)(oj.y >> 1) : f.e;
+      }
+      done |= 1ull << (f.e & 63u);
+#pragma unroll
+      for (uint32_t q = 0; q < 2u; ++q) {
+        const uint32_t kk = next[q] >> 6;
+        const uint64_t bit = 1ull << (next[q] & 63u);
+        if (kk == k) {
+          want |= bit;
+        } else {
+          const uint4 o = rec[kk];
+          if (!(fuse_mask(o) & bit)) {
+            rec[kk] = make_uint4(o.x | (uint32_t)bit, o.y | (uint32_t)(bit >> 32), o.z, o.w);
+            if (kk < k) back = min(back, kk);
           }
         }
       }
-      rec[k] = make_uint4((uint32_t)want, (uint32_t)(want >> 32), (uint32_t)done, (uint32_t)(done >> 32));
-      k = back < k ? back : k + 1u;
+      while (!(want & ~done)) {                          // the record is done: on to the next, or back
+        rec[k] = make_uint4((uint32_t)want, (uint32_t)(want >> 32), (uint32_t)done, (uint32_t)(done >> 32));
+        k = back < k ? back : k + 1u;
+        back = ~0u;
+        if (k >= nrec) {
+          more = false;
+          break;
+        }
+        const uint4 r = rec[k];
+        want = fuse_mask(r);
+        done = ((uint64_t)r.w << 32) | r.z;
+      }
+      if (more) f.start(64u * k + (uint32_t)__ffsll((long long)(want & ~done)) - 1u);
     }
     uint32_t count = 0;
     for (uint32_t k = 0; k < nrec; ++k) {
@@ -363,7 +375,9 @@ __device__ __forceinline__ void run_epoch(Mem M, const uint64_t* T, uint64_t* Y,
 // it wrote into its program, or its i lies outside them for a few steps --
 // runs from its memory (run_epoch_loop, which does not watch its writes) until
 // the next pack.
-constexpr uint32_t kFuseChunk = 16;    // entries between two looks at the stalled lanes (uneven 4.95 -> 4.85 ms, from 8)
+constexpr uint32_t kFuseChunk = 16;    // entries between two looks at the stalled lanes (from 8: uneven
+                                       // 4.95 -> 4.85 ms); 12 stalled lanes end an epoch (templates 1.89 ms,
+                                       // 8: 1.93, 4: 2.08)
 constexpr uint32_t kFuseOutside = 32;  // general steps at no entry's start before a VM leaves them: more than an
                                        // entry holds (a run that a stop has cut goes on inside an entry)
 
@@ -375,7 +389,7 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
   const uint32_t fm = __ballot_sync(FULL, active && F.on);
   bool stall = active && r.clean && !F.on;               // a stop has cut the run of an entry: on to the next one
   if (fm) {
-    const uint32_t wait = idle_exit ? idle_exit : 8u;
+    const uint32_t wait = idle_exit ? idle_exit : 12u;
     const uint32_t zero = P.ellp & 1u;                   // the stride of the tapes is even
     for (uint32_t it = (epoch + 3u) / 4u * 2u; it;) {
       const uint32_t c = min(it, kFuseChunk);
@@ -618,15 +632,19 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
     }
     // swap in the prefetched VM (its loads were issued a boundary ago)
     if (vm < 0 && pf == PF_REGS) {
-      if (S.status[pf_vm] == ST_RUNNING) {
-        load_regs(S, P, pf_vm, r);
-        const uint64_t moff = S.mem_off[pf_vm];
+      // every load of the VM's state goes out at once (vm < 0: r is free)
+      const uint32_t st = S.status[pf_vm];
+      const uint64_t moff = S.mem_off[pf_vm];
+      FuseRow row{};
+      if (FUSE) row = fuse_row(S, pf_vm);
+      load_regs(S, P, pf_vm, r);
+      if (st == ST_RUNNING) {
         arm_regs(P, r);
         vm = (int32_t)pf_vm;
         attach_mem(M, S, moff);
         T = S.tape + (uint64_t)pf_vm * P.ellp;
         Y = S.y + (uint64_t)pf_vm * P.sp;
-        if (FUSE) fuse_attach(S, pf_vm, r, F);
+        if (FUSE) fuse_attach(S, row, r, F);
         if (!VOTE && !F.on) prime(M, r);
         active = true;
       }
@@ -703,15 +721,19 @@ __global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Que
       // an idle lane in the tail starts its VM at once (waiting on the loads
       // here) instead of two boundaries later
       pf = PF_EMPTY;
-      if (S.status[pf_vm] == ST_RUNNING) {
-        load_regs(S, P, pf_vm, r);
-        const uint64_t moff = S.mem_off[pf_vm];
+      // every load of the VM's state goes out at once (vm < 0: r is free)
+      const uint32_t st = S.status[pf_vm];
+      const uint64_t moff = S.mem_off[pf_vm];
+      FuseRow row{};
+      if (FUSE) row = fuse_row(S, pf_vm);
+      load_regs(S, P, pf_vm, r);
+      if (st == ST_RUNNING) {
         arm_regs(P, r);
         vm = (int32_t)pf_vm;
         attach_mem(M, S, moff);
         T = S.tape + (uint64_t)pf_vm * P.ellp;
         Y = S.y + (uint64_t)pf_vm * P.sp;
-        if (FUSE) fuse_attach(S, pf_vm, r, F);
+        if (FUSE) fuse_attach(S, row, r, F);
         if (!VOTE && !F.on) prime(M, r);
         active = true;
       }
@@ -839,6 +861,7 @@ __global__ void __launch_bounds__(128, 6) k_serve(ServeArgs A, Params P0) {
           const ServeSlot& sd = A.slots[sl];
           slot = (int32_t)sl;
           vm = v;
+          r.clean = false;
           if (sd.S.status[v] == ST_RUNNING) {
             P.budget = sd.budget;
             load_regs(sd.S, P, v, r);
@@ -847,7 +870,8 @@ __global__ void __launch_bounds__(128, 6) k_serve(ServeArgs A, Params P0) {
             M = sd.S.mem + moff;
             T = sd.S.tape + (uint64_t)v * P.ellp;
             Y = sd.S.y + (uint64_t)v * P.sp;
-            if (!CHECKED) fuse_attach(sd.S, v, r, F);
+            F.on = false;
+            if (!CHECKED && sd.S.fops) fuse_attach(sd.S, fuse_row(sd.S, v), r, F);
             if (!F.on) prime(M, r);
             active = true;
           } else {
