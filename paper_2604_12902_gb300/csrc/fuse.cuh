@@ -351,14 +351,35 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, const FuseRow& w,
       "@pr " ST " [ad1], " V ";\n\t" \
       "@pr add.u32 %8, %8, 1;\n\t" \
       "RASP_FNOIO:\n\t"
+// Both entries that may come next are loaded beside the operands (f into the
+// entry's own registers, whose fields have been taken apart by then), so that
+// an entry waits for one round of loads and not for two in a row.
+#define RASP_F_AHEAD(FETCH) \
+      "shr.s32 i2, %3, 16;\n\t" \
+      "and.b32 jt, %4, 0xFFFF;\n\t" \
+      "shr.u32 jf, %4, 16;\n\t" \
+      RASP_F_TEST("pb", "0x40000000") \
+      FETCH
+#define RASP_F_FETCH_GL \
+      "mad.wide.u32 ad1, jf, 16, %11;\n\t" \
+      "mad.wide.u32 ad2, jt, 16, %11;\n\t" \
+      "@!px ld.global.nc.v4.u32 {%1, %2, %3, %4}, [ad1];\n\t" \
+      "@pb ld.global.nc.v4.u32 {tx, ty, tz, tw}, [ad2];\n\t"
+// entries in shared memory (%11 = their 32-bit address)
+#define RASP_F_FETCH_SH \
+      "mad.lo.u32 t0, jf, 16, %11;\n\t" \
+      "mad.lo.u32 j, jt, 16, %11;\n\t" \
+      "@!px ld.shared.v4.u32 {%1, %2, %3, %4}, [t0];\n\t" \
+      "@pb ld.shared.v4.u32 {tx, ty, tz, tw}, [j];\n\t"
 // the next entry, and the VM-steps of this one
-#define RASP_F_NEXT(FETCH) \
-      "and.b32 j, %4, 0xFFFF;\n\t" \
-      "shr.u32 t0, %4, 16;\n\t" \
-      "selp.b32 j, j, t0, pt;\n\t" \
+#define RASP_F_NEXT \
+      "selp.b32 j, jt, jf, pt;\n\t" \
       "@!px mov.b32 %5, j;\n\t" \
       "@!px sub.u32 %6, %6, c;\n\t" \
-      FETCH \
+      "@pt mov.b32 %1, tx;\n\t" \
+      "@pt mov.b32 %2, ty;\n\t" \
+      "@pt mov.b32 %3, tz;\n\t" \
+      "@pt mov.b32 %4, tw;\n\t" \
       "}"
 #define RASP_F_LOOP1(BODY) \
       BODY \
@@ -374,26 +395,20 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, const FuseRow& w,
       "setp.ne.u32 p1, it, 0;\n\t" \
       "@p1 bra.uni RASP_FLOOP;\n\t" \
       "}"
-#define RASP_F_FETCH_GL \
-      "mad.wide.u32 ad1, j, 16, %11;\n\t" \
-      "@!px ld.global.nc.v4.u32 {%1, %2, %3, %4}, [ad1];\n\t"
-// entries in shared memory (%11 = their 32-bit address)
-#define RASP_F_FETCH_SH \
-      "mad.lo.u32 t0, j, 16, %11;\n\t" \
-      "@!px ld.shared.v4.u32 {%1, %2, %3, %4}, [t0];\n\t"
 #define RASP_F_REGS \
-      ".reg .pred px, pr, p1, p2, pt;\n\t" \
-      ".reg .b32 c, t0, ye, j, it, zz;\n\t" \
+      ".reg .pred px, pr, p1, p2, pt, pb;\n\t" \
+      ".reg .b32 c, t0, ye, j, it, zz, jt, jf, i2, tx, ty, tz, tw;\n\t" \
       ".reg .b64 ad1, ad2, ads;\n\t"
 
 // 8-byte words. %17 = 2^w - 1 (masked), %18 = its half (classic condition).
 #define RASP_FW_HEAD "{\n\t" RASP_F_REGS ".reg .b64 v1, v2, im;\n\t" "mov.b32 it, %9;\n\tRASP_FLOOP:\n\t"
-#define RASP_FW_A \
+#define RASP_FW_A(FETCH) \
       "{\n\t" RASP_F_GUARD RASP_F_ADDR("8") \
       "@p1 ld.global.u64 v1, [ad1];\n\t" \
       "@p2 ld.global.u64 v2, [ad2];\n\t" \
       "cvt.s32.s16 t0, %3;\n\t" \
       "cvt.s64.s32 im, t0;\n\t" \
+      RASP_F_AHEAD(FETCH) \
       RASP_F_TEST("p1", "0x00200000") \
       "@p1 mov.b64 %0, im;\n\t" \
       RASP_F_TEST("p1", "0x00400000") \
@@ -413,19 +428,16 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, const FuseRow& w,
       RASP_F_IO("ld.global.u64", "st.global.u64", "v1", "im") \
       RASP_F_TEST("p1", "0x20000000") \
       "@p1 mov.b64 v2, %0;\n\t" \
-      "shr.s32 t0, %3, 16;\n\t" \
-      "cvt.s64.s32 im, t0;\n\t" \
+      "cvt.s64.s32 im, i2;\n\t" \
       RASP_F_TEST("p1", "0x08000000") \
       "@p1 mov.b64 %0, im;\n\t" \
       RASP_F_TEST("p1", "0x30000000") \
       "@p1 add.u64 %0, %0, v2;\n\t"
 #define RASP_FW_PT_WORD \
-      RASP_F_TEST("p1", "0x40000000") \
-      "setp.ne.and.u64 pt, %0, 0, p1;\n\t"
+      "setp.ne.and.u64 pt, %0, 0, pb;\n\t"
 #define RASP_FW_PT_CLASSIC \
-      RASP_F_TEST("p1", "0x40000000") \
       "add.u64 im, %0, -1;\n\t" \
-      "setp.lt.and.u64 pt, im, %18, p1;\n\t"
+      "setp.lt.and.u64 pt, im, %18, pb;\n\t"
 #define RASP_FW_OPERANDS(TAB) \
   : "+l"(a), "+r"(F.op.x), "+r"(F.op.y), "+r"(F.op.z), "+r"(F.op.w), "+r"(F.cur), "+r"(left), "+r"(u0), "+r"(y0) \
   : "r"(iters), "l"(M), TAB, "l"(T), "l"(Y), "r"(ell), "r"(s), "r"(mask), "l"(wmask),                    \
@@ -438,20 +450,20 @@ __device__ __forceinline__ void fused_loop_ptx(uint64_t* M, const uint64_t* T, u
                                                uint64_t& a, Fused& F, uint32_t& left, uint32_t& u0, uint32_t& y0) {
   if constexpr (MASKED && CLASSIC) {
     asm volatile(RASP_FW_HEAD RASP_F_LOOP1(
-        RASP_FW_A RASP_FW_SUB RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_CLASSIC
-        RASP_F_NEXT(RASP_F_FETCH_GL))
+        RASP_FW_A(RASP_F_FETCH_GL) RASP_FW_SUB RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_CLASSIC
+        RASP_F_NEXT)
                  RASP_FW_OPERANDS("l"(F.tab)));
   } else if constexpr (MASKED) {
     asm volatile(RASP_FW_HEAD RASP_F_LOOP1(
-        RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
-        RASP_F_NEXT(RASP_F_FETCH_GL))
+        RASP_FW_A(RASP_F_FETCH_GL) RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
+        RASP_F_NEXT)
                  RASP_FW_OPERANDS("l"(F.tab)));
   } else if constexpr (CLASSIC) {
     asm volatile(RASP_FW_HEAD RASP_F_LOOP1(
-        RASP_FW_A RASP_FW_SUB RASP_FW_B RASP_FW_PT_CLASSIC RASP_F_NEXT(RASP_F_FETCH_GL))
+        RASP_FW_A(RASP_F_FETCH_GL) RASP_FW_SUB RASP_FW_B RASP_FW_PT_CLASSIC RASP_F_NEXT)
                  RASP_FW_OPERANDS("l"(F.tab)));
   } else {
-    asm volatile(RASP_FW_HEAD RASP_F_LOOP1(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_GL))
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP1(RASP_FW_A(RASP_F_FETCH_GL) RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT)
                  RASP_FW_OPERANDS("l"(F.tab)));
   }
 }
@@ -464,11 +476,11 @@ __device__ __forceinline__ void fused_loop_ptx_sh(uint64_t* M, uint32_t tab, con
                                                   uint32_t& left, uint32_t& u0, uint32_t& y0) {
   if constexpr (MASKED) {
     asm volatile(RASP_FW_HEAD RASP_F_LOOP2(
-        RASP_FW_A RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
-        RASP_F_NEXT(RASP_F_FETCH_SH))
+        RASP_FW_A(RASP_F_FETCH_SH) RASP_FW_MUL RASP_FW_MASK RASP_FW_B RASP_FW_MASK RASP_FW_PT_WORD
+        RASP_F_NEXT)
                  RASP_FW_OPERANDS("r"(tab)));
   } else {
-    asm volatile(RASP_FW_HEAD RASP_F_LOOP2(RASP_FW_A RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT(RASP_F_FETCH_SH))
+    asm volatile(RASP_FW_HEAD RASP_F_LOOP2(RASP_FW_A(RASP_F_FETCH_SH) RASP_FW_MUL RASP_FW_B RASP_FW_PT_WORD RASP_F_NEXT)
                  RASP_FW_OPERANDS("r"(tab)));
   }
 }
@@ -476,11 +488,12 @@ __device__ __forceinline__ void fused_loop_ptx_sh(uint64_t* M, uint32_t tab, con
 // 4-byte words (w <= 32). Tape words and outputs are 8-byte words whose high
 // halves are zero. %17 = 2^w - 1, %18 = its half.
 #define RASP_FN_HEAD "{\n\t" RASP_F_REGS ".reg .b32 v1, v2, im;\n\t" "mov.b32 it, %9;\n\tRASP_FLOOP:\n\t"
-#define RASP_FN_A \
+#define RASP_FN_A(FETCH) \
       "{\n\t" RASP_F_GUARD RASP_F_ADDR("4") \
       "@p1 ld.global.u32 v1, [ad1];\n\t" \
       "@p2 ld.global.u32 v2, [ad2];\n\t" \
       "cvt.s32.s16 im, %3;\n\t" \
+      RASP_F_AHEAD(FETCH) \
       RASP_F_TEST("p1", "0x00200000") \
       "@p1 mov.b32 %0, im;\n\t" \
       RASP_F_TEST("p1", "0x00400000") \
@@ -497,24 +510,20 @@ __device__ __forceinline__ void fused_loop_ptx_sh(uint64_t* M, uint32_t tab, con
       RASP_F_IO("ld.global.u32", "st.global.u32", "v1", "im") \
       RASP_F_TEST("p1", "0x20000000") \
       "@p1 mov.b32 v2, %0;\n\t" \
-      "shr.s32 im, %3, 16;\n\t" \
       RASP_F_TEST("p1", "0x08000000") \
-      "@p1 mov.b32 %0, im;\n\t" \
+      "@p1 mov.b32 %0, i2;\n\t" \
       RASP_F_TEST("p1", "0x30000000") \
       "@p1 add.u32 %0, %0, v2;\n\t"
 #define RASP_FN_ST2 \
-      "and.b32 j, %4, 0xFFFF;\n\t" \
-      "mad.wide.u32 ads, j, 4, %10;\n\t" \
+      "mad.wide.u32 ads, jt, 4, %10;\n\t" \
       "setp.lt.s32 p1, ye, 0;\n\t" \
       "xor.b32 t0, zz, %0;\n\t" \
       "@p1 st.global.u32 [ads], t0;\n\t"
 #define RASP_FN_PT_WORD \
-      RASP_F_TEST("p1", "0x40000000") \
-      "setp.ne.and.u32 pt, %0, 0, p1;\n\t"
+      "setp.ne.and.u32 pt, %0, 0, pb;\n\t"
 #define RASP_FN_PT_CLASSIC \
-      RASP_F_TEST("p1", "0x40000000") \
       "add.u32 im, %0, -1;\n\t" \
-      "setp.lt.and.u32 pt, im, %18, p1;\n\t"
+      "setp.lt.and.u32 pt, im, %18, pb;\n\t"
 #define RASP_FN_OPERANDS \
   : "+r"(a), "+r"(F.op.x), "+r"(F.op.y), "+r"(F.op.z), "+r"(F.op.w), "+r"(F.cur), "+r"(left), "+r"(u0), "+r"(y0) \
   : "r"(iters), "l"(M), "l"(F.tab), "l"(T), "l"(Y), "r"(ell), "r"(s), "r"(mask), "r"(wmask),                    \
@@ -529,23 +538,23 @@ __device__ __forceinline__ void fused_loop_ptx_narrow(uint32_t* M, const uint64_
                                                       uint32_t& u0, uint32_t& y0) {
   if constexpr (MASK && CLASSIC) {
     asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
-        RASP_FN_A RASP_FN_SUB RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_ST2 RASP_FN_PT_CLASSIC
-        RASP_F_NEXT(RASP_F_FETCH_GL))
+        RASP_FN_A(RASP_F_FETCH_GL) RASP_FN_SUB RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_ST2 RASP_FN_PT_CLASSIC
+        RASP_F_NEXT)
                  RASP_FN_OPERANDS);
   } else if constexpr (MASK) {
     asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
-        RASP_FN_A RASP_FN_MUL RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_ST2 RASP_FN_PT_WORD
-        RASP_F_NEXT(RASP_F_FETCH_GL))
+        RASP_FN_A(RASP_F_FETCH_GL) RASP_FN_MUL RASP_FN_MASK RASP_FN_B RASP_FN_MASK RASP_FN_ST2 RASP_FN_PT_WORD
+        RASP_F_NEXT)
                  RASP_FN_OPERANDS);
   } else if constexpr (CLASSIC) {
     asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
-        RASP_FN_A RASP_FN_SUB RASP_FN_B RASP_FN_ST2 RASP_FN_PT_CLASSIC
-        RASP_F_NEXT(RASP_F_FETCH_GL))
+        RASP_FN_A(RASP_F_FETCH_GL) RASP_FN_SUB RASP_FN_B RASP_FN_ST2 RASP_FN_PT_CLASSIC
+        RASP_F_NEXT)
                  RASP_FN_OPERANDS);
   } else {
     asm volatile(RASP_FN_HEAD RASP_F_LOOP1(
-        RASP_FN_A RASP_FN_MUL RASP_FN_B RASP_FN_ST2 RASP_FN_PT_WORD
-        RASP_F_NEXT(RASP_F_FETCH_GL))
+        RASP_FN_A(RASP_F_FETCH_GL) RASP_FN_MUL RASP_FN_B RASP_FN_ST2 RASP_FN_PT_WORD
+        RASP_F_NEXT)
                  RASP_FN_OPERANDS);
   }
 }

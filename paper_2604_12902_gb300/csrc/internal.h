@@ -36,6 +36,7 @@ struct PersistShape {
   bool block;           // one step at a time (the per-step form) instead of the epoch loop
   uint32_t grid;        // CTAs
   uint32_t ctas_per_sm; // resident CTAs per SM (occupancy)
+  uint32_t fuse_ctas;   // HBM-slab: the same for programs with fused entries
   size_t smem;          // dynamic shared memory per CTA
 };
 

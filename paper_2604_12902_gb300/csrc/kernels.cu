@@ -16,6 +16,7 @@
 // `one_step`, or, with the VOTE variant, by warp opcode voting: lanes are
 // grouped by opcode with __match_any_sync and each group runs the handler of
 // its case of the Sec. 2.1 equation.
+#include <algorithm>
 #include <cstdio>
 
 #include "engine.cuh"
@@ -577,10 +578,12 @@ enum : uint32_t { PF_EMPTY = 0, PF_ID = 1, PF_REGS = 2, PF_NONE = 3 };   // PF_R
 //
 // FUSE: the programs have fused entries. Batches without them keep a kernel of
 // their own: both loops in one kernel spill more, and 1,024 random programs
-// took 333 instead of 319 us a pass.
+// took 333 instead of 319 us a pass. With entries 6 CTAs of 80 registers run
+// per SM in place of 7 of 72: 2^20 templates 1.86 ms (7: 1.88), 262,144 uneven
+// 4.56 (4.59), the halting rounds of 2^18 programs 82 (87).
 template <bool MASKED, bool CHECKED, bool HIST, bool VOTE, bool CLASSIC = false, bool LOOP = false,
           bool NARROW = false, bool FUSE = false>
-__global__ void __launch_bounds__(128, 7) k_persist_gl(DevState S, Params P, Queue Q, uint32_t epoch,
+__global__ void __launch_bounds__(128, FUSE ? 6 : 7) k_persist_gl(DevState S, Params P, Queue Q, uint32_t epoch,
                                                        uint32_t idle_exit) {
   static_assert(!LOOP || (!HIST && !VOTE), "the epoch loop serves select steps without counters");
   const uint32_t lane = threadIdx.x & 31u;
@@ -1509,11 +1512,15 @@ int persist_configure(const StepVariant& var, PersistShape& sh) {
   // keep it as L1 for the M slabs in HBM
   cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
                        sh.staged ? (int)cudaSharedmemCarveoutMaxShared : (int)cudaSharedmemCarveoutMaxL1);
-  if (!sh.staged) {   // programs are loaded after the plan is made: the form with fused entries too (same bounds)
+  int fuse_sm = 0;
+  if (!sh.staged) {   // programs are loaded after the plan is made: the form with fused entries too
     v.fuse = true;
-    cudaFuncSetAttribute(persist_symbol(v, false), cudaFuncAttributePreferredSharedMemoryCarveout,
-                         (int)cudaSharedmemCarveoutMaxL1);
+    const void* ff = persist_symbol(v, false);
+    cudaFuncSetAttribute(ff, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxL1);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fuse_sm, ff, (int)(32u * sh.warps), 0) != cudaSuccess)
+      fuse_sm = 0;
   }
+  sh.fuse_ctas = (uint32_t)(fuse_sm > 0 ? fuse_sm : 1);
   cudaGetLastError();
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, (int)(32u * sh.warps), sh.smem) != cudaSuccess) {
@@ -1528,12 +1535,15 @@ int persist_configure(const StepVariant& var, PersistShape& sh) {
 cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Params& P, const Queue& Q,
                            const PersistShape& sh, cudaStream_t stream) {
   if ((!Q.count && !Q.dcount) || !sh.grid) return cudaSuccess;
-  uint32_t grid = sh.grid;
+  StepVariant v = shape_variant(var, sh);
+  v.fuse = S.fops != nullptr;
+  const uint32_t resident = v.fuse ? std::min(sh.grid, sh.fuse_ctas * (uint32_t)num_sms()) : sh.grid;
+  uint32_t grid = resident;
   const uint32_t warps_needed = (Q.count + 31u) / 32u;   // with dcount, Q.count is an upper bound
   uint32_t cta_warps = sh.warps, cta_lanes = 32u;
   const uint32_t max_useful = (warps_needed + sh.warps - 1u) / sh.warps;
   const uint32_t spread = 8u * (uint32_t)num_sms();
-  if (!sh.staged && !Q.dcount && warps_needed < spread && sh.grid * sh.warps >= 2u * spread) {
+  if (!sh.staged && !Q.dcount && warps_needed < spread && resident * sh.warps >= 2u * spread) {
     // Few VMs (under 38,912 on 152 SMs): 8 warps per SM, each with as few lanes
     // as that takes, and four where that would be five to eight: the lanes of a
     // warp wait for one another's misses and general steps. Run kernel, 32
@@ -1554,8 +1564,6 @@ cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Para
   q.lanes = cta_lanes;
   const uint64_t lanes = (uint64_t)grid * cta_warps * cta_lanes;
   q.soft_end = Q.count > lanes ? (uint32_t)(Q.count - lanes) : 0u;
-  StepVariant v = shape_variant(var, sh);
-  v.fuse = S.fops != nullptr;
   if (sh.staged)
     pick_staged(v)<<<grid, 32u * sh.warps, sh.smem, stream>>>(S, P, q, sh.ncap, sh.slot_words, sh.epoch,
                                                                  sh.refill_min,
