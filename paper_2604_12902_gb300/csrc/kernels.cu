@@ -367,10 +367,10 @@ __device__ __forceinline__ void run_epoch(Mem M, const uint64_t* T, uint64_t* Y,
   }
 }
 
-// About `epoch` VM-steps of every active lane (epoch / 2 entries of the lanes
-// that run from them, then `epoch` steps one instruction at a time for the
-// rest; half as many entries measured 9 % slower on 1M template programs:
-// every return to the scheduler waits for the next VM's state). Lanes that stall wait in place until `wait` of them
+// `epoch` entries of every active lane that runs from them, then `epoch` steps
+// one instruction at a time of the rest. (Half as many entries: 2^20 templates
+// 1.86 ms in place of 1.82, a quarter 2.0: every return to the scheduler waits
+// for the next VM's state.) Lanes that stall wait in place until `wait` of them
 // have (or none runs on), then take general steps together until they can
 // enter their entries again or stop. A VM that leaves its entries for good --
 // it wrote into its program, or its i lies outside them for a few steps --
@@ -392,7 +392,7 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
   if (fm) {
     const uint32_t wait = idle_exit ? idle_exit : 12u;
     const uint32_t zero = P.ellp & 1u;                   // the stride of the tapes is even
-    for (uint32_t it = (epoch + 3u) / 4u * 2u; it;) {
+    for (uint32_t it = (epoch + 1u) & ~1u; it;) {
       const uint32_t c = min(it, kFuseChunk);
       it -= c;
       if (active && F.on) {

@@ -24,7 +24,7 @@ def rasp():
     return R
 
 
-def machines(V, m, w, seed, extra=24, p_code=0.02, shared=0):
+def machines(V, m, w, seed, extra=24, p_code=0.02, shared=0, huge=False):
     """V machines of m instructions: opcodes weighted to the fused form, small
     and wide constants, data words mostly behind the program, jump targets
     mostly even; a few operands in the program or past the memory."""
@@ -40,8 +40,14 @@ def machines(V, m, w, seed, extra=24, p_code=0.02, shared=0):
     arg = np.where(rng.random((P, m)) < .01, rng.integers(n, n + 3, (P, m)), arg)
     target = 2 * rng.integers(0, m, (P, m)) + (rng.random((P, m)) < .03)
     wide = rng.choice([-1, 1, 0, 2, -32768, 32767, 32768, 70000, -(1 << 31), (1 << 31) - 1], size=(P, m))
+    if huge:                                                      # words of 8 bytes only
+        far = [1 << 31, (1 << 32) - 1, (1 << 32) + 1, 1 << 62, -(1 << 63), -(1 << 40) + 4, (1 << 48) - 1]
+        wide = np.where(rng.random((P, m)) < .5, wide, rng.choice(far, size=(P, m)))
+        op = np.where(rng.random((P, m)) < .01, (1 << 32) + op, op)
     const = np.where(rng.random((P, m)) < .1, wide, rng.integers(-3, 4, (P, m)))
     arg = np.where(op == BNZ, target, np.where(op == LOD, const, arg))
+    if huge:
+        arg = np.where(rng.random((P, m)) < .02, wide, arg)
     prog = np.empty((P, 2 * m), np.int64)
     prog[:, 0::2], prog[:, 1::2] = op, arg
     ell, s = 5, 3
@@ -74,6 +80,13 @@ def check(rasp, wl, budgets, what, classic=False, i32=True, **kw):
 def test_entries_match_the_oracle(rasp, m, w):
     wl = machines(700, m, w, seed=1000 * m + w)
     check(rasp, wl, [3, 20, 21, 200, 1000], "m=%d w=%d" % (m, w), i32=(m + w) % 2 == 0)
+
+
+@pytest.mark.parametrize("w", [64, 48, 33, 32, 31])
+@pytest.mark.parametrize("classic", [False, True])
+def test_words_beyond_32_bits(rasp, w, classic):
+    wl = machines(1500, 40, w, seed=40 + w, huge=True)
+    check(rasp, wl, [9, 60, 1000], "huge words w=%d" % w, classic=classic, i32=False)
 
 
 @pytest.mark.parametrize("w", [64, 32])
@@ -131,7 +144,8 @@ def test_self_writing_programs(rasp):
     check(rasp, a, [20, 256], "all")
     c = machines(512, 32, 64, seed=13, extra=136)
     for every in (2, 9):
-        prog = np.where((np.arange(512) % every == 0)[:, None], a.programs.reshape(512, -1), c.programs.reshape(512, -1))
+        own = (np.arange(512) % every == 0)[:, None]
+        prog = np.where(own, a.programs.reshape(512, -1), c.programs.reshape(512, -1))
         wl = W.Workload("mixed", prog.reshape(-1), a.prog_off, c.mem_words, c.tapes, c.tape_off, c.caps, c.ell, c.s)
         check(rasp, wl, [20, 1000], "every %d" % every)
 
