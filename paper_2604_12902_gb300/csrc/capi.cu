@@ -97,7 +97,7 @@ struct rasp_batch {
   uint64_t wmask = ~0ull;
   std::vector<uint32_t> h_n;
   std::vector<uint64_t> h_memoff;
-  uint64_t mem_words = 0;      // words of the M arena: sum of slab_words(n)
+  uint64_t mem_words = 0;      // words of the M arena: the padded n and the room between slab groups
   Layout L{};
   char* base = nullptr;
   bool owns = false;
@@ -236,17 +236,16 @@ Layout make_layout(uint64_t V, uint64_t mem_words, uint32_t ellp, uint32_t sp, u
 
 uint32_t even(uint32_t x) { return (x + 1u) & ~1u; }
 
-// Words from one VM's slab to the next: n rounded up to even; on the
-// shared-program schedule to an odd multiple of four words. Its lanes run one
-// program nearly in step and touch the same offset of 32 slabs: with slabs a
-// multiple of 128 bytes apart all of these lie in the same L1 banks (32 cycles
-// for such a load; k_shared_loop on 2^20 VMs 1.2 ms, 0.80 ms so). An odd number
-// of word pairs runs as fast, but its half sectors cost the pack (0.25 ms
-// against 0.19).
-uint64_t slab_words(const rasp_config* cfg, uint32_t n) {
-  const uint32_t e = even(n);
-  return (cfg->flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED ? ((e + 3ull) & ~3ull) | 4ull : e;
-}
+// On the shared-program schedule every second slab is followed by 32 unused
+// bytes: its lanes run one program nearly in step and touch the same offset of
+// 32 slabs, and with slabs a multiple of 128 bytes apart all of these lie in
+// the same L1 banks (32 cycles for such a load; k_shared_loop on 2^20 VMs
+// 1.2 ms, 0.81 ms so; after every fourth slab 0.84, every eighth 0.99). Whole
+// sectors: with 16 bytes the pack took 0.25 ms in place of 0.19. The room is
+// part of every batch, whose size does not depend on the schedule.
+constexpr uint64_t kSlabGroup = 2, kGroupPad = 4;
+uint64_t pad_words(uint64_t num_vms) { return (num_vms - 1) / kSlabGroup * kGroupPad; }
+bool padded_slabs(const rasp_config* cfg) { return (cfg->flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED; }
 
 StepVariant variant_of(const rasp_batch* b) {
   StepVariant v{};
@@ -491,7 +490,8 @@ int rasp_batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* m
   if (rc) return rc;
   if (!out_bytes) return fail(RASP_EINVAL, "out_bytes is NULL");
   uint64_t mw = 0;
-  for (uint64_t v = 0; v < num_vms; ++v) mw += slab_words(cfg, mem_words[v]);
+  for (uint64_t v = 0; v < num_vms; ++v) mw += even(mem_words[v]);
+  mw += pad_words(num_vms);
   *out_bytes = make_layout(num_vms, mw, even(cfg->in_cap), even(cfg->out_cap), narrow_layout(cfg, true) ? 4u : 8u).total +
                ALIGN;
   return RASP_OK;
@@ -526,9 +526,11 @@ int rasp::create_batch(const rasp_config* cfg, uint64_t num_vms, const uint32_t*
   b->h_memoff.resize(num_vms);
   uint64_t off = 0;
   for (uint64_t v = 0; v < num_vms; ++v) {
+    if (v && v % kSlabGroup == 0 && padded_slabs(cfg)) off += kGroupPad;
     b->h_memoff[v] = off;
-    off += slab_words(cfg, mem_words[v]);
+    off += even(mem_words[v]);
   }
+  if (!padded_slabs(cfg)) off += pad_words(num_vms);
   b->mem_words = off;
   b->narrow = narrow_layout(cfg, plan);
   b->L = make_layout(num_vms, off, b->ellp, b->sp, b->narrow ? 4u : 8u);
@@ -828,7 +830,8 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   b->prog64_valid = !b->prog32;
   if (word_size == 4 && total && !keep32) CK(launch_widen(staged, b->d_prog, total, st));
   if (b->S.fops)
-    CK(launch_fuse(b->d_prog, b->prog32, b->d_progoff, bound, b->num_programs, b->wmask, variant_of(b).classic,
+    CK(launch_fuse(b->d_prog, b->prog32, b->d_progoff, bound, b->num_programs, b->max_plen, total / 2u,
+                   b->wmask, variant_of(b).classic,
                    owns_code(b), b->narrow, reinterpret_cast<uint4*>(b->S.mem), const_cast<uint4*>(b->S.fops),
                    const_cast<uint4*>(b->S.frec), st));
   CK(fill_bytes(b->d_hist, 0, 8 * 10, st));
@@ -1097,10 +1100,18 @@ int rasp_read_state(rasp_batch* b, uint64_t first, uint64_t count, rasp_state_vi
       CK(cudaMemcpyAsync(m32.data(), S.mem32 + lo, 4 * (hi - lo), cudaMemcpyDeviceToHost, st));
     } else if (need == hi - lo) {
       CK(cudaMemcpyAsync(out->mem, S.mem + lo, 8 * need, cudaMemcpyDeviceToHost, st));
-    } else if (uniform) {                    // equal slabs: one strided copy
-      const uint64_t pitch = count > 1 ? b->h_memoff[first + 1] - lo : b->h_n[first];
-      CK(cudaMemcpy2DAsync(out->mem, 8ull * b->h_n[first], S.mem + lo, 8ull * pitch, 8ull * b->h_n[first], count,
-                           cudaMemcpyDeviceToHost, st));
+    } else if (uniform && !(b->h_n[first] & 1u)) {   // equal slabs: whole groups by one strided copy
+      const uint64_t n = b->h_n[first], end = first + count;
+      const uint64_t g0 = std::min(end, (first + kSlabGroup - 1) / kSlabGroup * kSlabGroup);
+      const uint64_t g1 = std::max(g0, end / kSlabGroup * kSlabGroup);
+      auto part = [&](uint64_t v, uint64_t vms, uint64_t rows) {
+        if (!vms || !rows) return cudaSuccess;
+        return cudaMemcpy2DAsync(out->mem + (v - first) * n, 8 * n * vms, S.mem + b->h_memoff[v],
+                                 8 * (n * vms + kGroupPad), 8 * n * vms, rows, cudaMemcpyDeviceToHost, st);
+      };
+      CK(part(first, g0 - first, 1));
+      CK(part(g0, kSlabGroup, (g1 - g0) / kSlabGroup));
+      CK(part(g1, end - g1, 1));
     } else {
       mbuf.resize(hi - lo);
       CK(cudaMemcpyAsync(mbuf.data(), S.mem + lo, 8 * (hi - lo), cudaMemcpyDeviceToHost, st));

@@ -54,7 +54,8 @@ cudaError_t launch_pack(const DevState& S, const uint64_t* prog, const int32_t* 
 // runs them takes a second store (4-byte words); tmp: scratch of
 // 16 bytes per instruction.
 cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint64_t* prog_off, const uint32_t* bound,
-                        uint32_t num_programs, uint64_t wmask, bool classic, bool own, bool two, uint4* tmp, uint4* out,
+                        uint32_t num_programs, uint32_t max_plen, uint64_t instructions, uint64_t wmask,
+                        bool classic, bool own, bool two, uint4* tmp, uint4* out,
                         uint4* recs, cudaStream_t stream);
 
 // Shared-program schedule: one CTA per program (program in shared memory),

@@ -219,6 +219,47 @@ __global__ void __launch_bounds__(128) k_fuse(const W* __restrict__ prog, const 
   }
 }
 
+// The same with an entry for every instruction (entry q = instruction q), one
+// instruction per lane: more work, no chain from entry to entry. A warp takes
+// 64 instructions of a program, blockIdx.y spreads long programs.
+template <class W>
+__global__ void __launch_bounds__(128) k_fuse_all(const W* __restrict__ prog, const uint64_t* __restrict__ prog_off,
+                                                  const uint32_t* __restrict__ bound, uint32_t num_programs,
+                                                  uint64_t wmask, uint32_t classic, uint32_t own, uint32_t two,
+                                                  uint4* __restrict__ out, uint4* __restrict__ recs) {
+  const uint32_t lane = threadIdx.x & 31u, warps = gridDim.y * (blockDim.x >> 5);
+  for (uint32_t p = blockIdx.x; p < num_programs; p += gridDim.x) {
+    const uint64_t po = prog_off[p];
+    const uint32_t plen = (uint32_t)(prog_off[p + 1] - po), n = bound[p];
+    const uint32_t ilim = wmask >= (uint64_t)n - 1u ? n : (uint32_t)(wmask + 1ull);
+    const uint32_t mok = min(plen, ilim) >> 1;
+    for (uint32_t k = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5); 64u * k < plen / 2u; k += warps) {
+      uint32_t writes = 0;
+      for (uint32_t e = 64u * k + lane; e < min(64u * (k + 1u), plen / 2u); e += 32u) {
+        FuseScan f;
+        f.start(e);
+        ulonglong2 oj = make_ulonglong2(0ull, 0ull);
+        if (e < mok) {
+          oj = fuse_pair(prog + po, 2u * e, wmask);
+          writes += (oj.x == 4ull || oj.x == 6ull) && oj.y < (uint64_t)plen ? 1u : 0u;
+          while (f.step(oj.x, oj.y, plen, n, mok, wmask, classic != 0u, own != 0u, two != 0u))
+            oj = fuse_pair(prog + po, 2u * f.p, wmask);
+        }
+        out[(po >> 1) + e] = e < mok ? f.entry(oj.x) : make_uint4(e, 0u, 0u, e | (e << 16));
+      }
+      writes = __reduce_add_sync(FULL, writes);
+      const uint32_t in = min(64u, plen / 2u - 64u * k), with = min(in, mok > 64u * k ? mok - 64u * k : 0u);
+      if (lane == 0u) {
+        const uint64_t mask = with >= 64u ? ~0ull : (1ull << with) - 1ull;
+        recs[(po >> 7) + p + k] = make_uint4((uint32_t)mask, (uint32_t)(mask >> 32), min(64u * k, mok), 0u);
+        // (as in k_fuse, by the program's first 64 instructions)
+        if (k == 0u && writes && 8u * writes >= with) out[po >> 1] = make_uint4(0u, FO_MEM, 0u, 0u);
+      }
+      __syncwarp();
+    }
+  }
+}
+
 // ------------------------------------------------------------------ vote step
 // Warp-synchronous step: every lane of the warp calls it; `active` lanes
 // take part. Lanes are grouped by opcode with __match_any_sync and each group
@@ -1421,9 +1462,27 @@ cudaError_t launch_pack(const DevState& S, const uint64_t* prog, const int32_t* 
 }
 
 cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint64_t* prog_off, const uint32_t* bound,
-                        uint32_t num_programs, uint64_t wmask, bool classic, bool own, bool two, uint4* tmp, uint4* out,
+                        uint32_t num_programs, uint32_t max_plen, uint64_t instructions, uint64_t wmask, bool classic, bool own, bool two, uint4* tmp, uint4* out,
                         uint4* recs, cudaStream_t stream) {
   if (!num_programs) return cudaSuccess;
+  // One program per lane takes at least the chain of the longest program (64
+  // instructions 0.12 ms, 512 0.90 ms), then 0.03 to 0.07 us per 1,000
+  // instructions; one instruction per lane 0.06 to 0.13 us per 1,000: 2,048
+  // templates 24 against 120 us, 16,384 136 and 124, 32,768 268 and 132; 16,384
+  // uneven programs 114 against 903 us. The line is where the chain costs as
+  // much as the work saved. (512: no chain of milliseconds for one program.)
+  if (max_plen / 2u > 512u || instructions <= 24000ull * (max_plen / 2u)) {
+    const uint32_t x = std::min(num_programs, (uint32_t)num_sms() * 16u);
+    const uint32_t rows = (max_plen + 511u) / 512u;        // four records per block
+    const dim3 g(x, std::min(std::max(rows, 1u), 64u));
+    if (prog32)
+      k_fuse_all<int32_t><<<g, 128, 0, stream>>>(prog32, prog_off, bound, num_programs, wmask, classic, own, two, out,
+                                                 recs);
+    else
+      k_fuse_all<uint64_t><<<g, 128, 0, stream>>>(prog, prog_off, bound, num_programs, wmask, classic, own, two, out,
+                                                  recs);
+    return cudaGetLastError();
+  }
   uint32_t blocks = (num_programs + 127u) / 128u;
   const uint32_t cap = (uint32_t)num_sms() * 16u;   // more blocks gain nothing (latency of each lane's scan)
   if (blocks > cap) blocks = cap;
@@ -1656,7 +1715,8 @@ int serve_configure(const StepVariant& var, ServeShape& sh) {
   // so that an SM can host them beside it
   const void* beside[] = {(const void*)fn, (const void*)k_pack<uint64_t>, (const void*)k_pack<int32_t>,
                           (const void*)k_ring_fill, (const void*)k_ring_publish, (const void*)k_fill,
-                          (const void*)k_fuse<uint64_t>, (const void*)k_fuse<int32_t>};
+                          (const void*)k_fuse<uint64_t>, (const void*)k_fuse<int32_t>,
+                          (const void*)k_fuse_all<uint64_t>, (const void*)k_fuse_all<int32_t>};
   for (const void* f : beside)
     cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxL1);
   cudaGetLastError();

@@ -100,6 +100,27 @@ def test_long_programs_and_code_words(rasp, p_code):
     check(rasp, machines(300, 64, 64, seed=7, p_code=p_code, extra=2), [50, 1000], "no room beside the program")
 
 
+@pytest.mark.parametrize("first,count", [(0, 1), (0, 8), (3, 30), (8, 16), (5, 2), (61, 3), (0, 64)])
+def test_reading_ranges_of_padded_slabs(rasp, first, count):
+    wl = machines(64, 20, 64, seed=60, shared=5)
+    wl.mem_words[:] = int(wl.mem_words.max()) + 1 & ~1
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s, flags=rasp.SCHED_SHARED) as b:
+        b.load_workload(wl)
+        b.run(300)
+        whole = b.read_state()["mem"].reshape(64, -1)
+        st, _ = oracle_state(wl, budget=300)
+        assert np.array_equal(whole.reshape(-1).view(np.uint64), st.mem)
+        assert np.array_equal(b.read_state(first, count)["mem"].reshape(count, -1), whole[first:first + count])
+
+
+@pytest.mark.parametrize("w", [64, 32])
+def test_many_short_programs(rasp, w):
+    """Enough instructions (over 2^21) for the decoder that takes a program per
+    lane and keeps only the entries it reaches."""
+    wl = machines(33_000, 65, w, seed=50 + w)
+    check(rasp, wl, [40, 1000], "per lane w=%d" % w, i32=w == 64)
+
+
 def test_shared_programs_on_several_memory_sizes(rasp):
     wl = machines(1500, 40, 64, seed=8, shared=37)
     check(rasp, wl, [30, 1000], "prog_of_vm", i32=False)
