@@ -226,7 +226,7 @@ __device__ __forceinline__ FuseProg fuse_prog(const DevState& S, uint32_t v, uin
 // The entry of instruction e, or ~0.
 __device__ __forceinline__ uint32_t fuse_find(const FuseProg& G, uint32_t e) {
   if (e >= G.mok) return ~0u;
-  const uint4 r = __ldg(G.rec + (e >> 6));
+  const uint4 r = G.rec[e >> 6];
   return (fuse_mask(r) >> (e & 63u)) & 1ull ? fuse_rank(r, e) : ~0u;
 }
 
@@ -235,10 +235,10 @@ __device__ __forceinline__ uint32_t fuse_instr(const FuseProg& G, uint32_t q) {
   uint32_t lo = 0, hi = (G.plen + 127u) / 128u;          // records with z <= q
   while (hi - lo > 1u) {
     const uint32_t mid = (lo + hi) >> 1;
-    if (__ldg(G.rec + mid).z <= q) lo = mid;
+    if (G.rec[mid].z <= q) lo = mid;
     else hi = mid;
   }
-  const uint4 r = __ldg(G.rec + lo);
+  const uint4 r = G.rec[lo];
   uint64_t mask = fuse_mask(r);
   for (uint32_t k = q - r.z; k; --k) mask &= mask - 1ull;
   return 64u * lo + (uint32_t)__ffsll((long long)mask) - 1u;
@@ -267,7 +267,7 @@ __device__ __forceinline__ void fuse_enter(const FuseProg& G, Fused& F, const Re
   F.on = true;
   F.cur = q;
   F.tab = G.tab;
-  F.op = __ldg(G.tab + q);
+  F.op = G.tab[q];
 }
 
 // What fuse_attach reads of VM v before its registers are armed, so that a
@@ -351,6 +351,10 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, const FuseRow& w,
       "@pr " ST " [ad1], " V ";\n\t" \
       "@pr add.u32 %8, %8, 1;\n\t" \
       "RASP_FNOIO:\n\t"
+// Entries are read by plain loads, not by ld.global.nc: the serving kernel
+// stays resident while the entries of new requests are written where those of
+// finished ones lay, and what it reads after claiming a VM has to be ordered by
+// its fence.
 // Both entries that may come next are loaded beside the operands (f into the
 // entry's own registers, whose fields have been taken apart by then), so that
 // an entry waits for one round of loads and not for two in a row.
@@ -363,8 +367,8 @@ __device__ __forceinline__ void fuse_attach(const DevState& S, const FuseRow& w,
 #define RASP_F_FETCH_GL \
       "mad.wide.u32 ad1, jf, 16, %11;\n\t" \
       "mad.wide.u32 ad2, jt, 16, %11;\n\t" \
-      "@!px ld.global.nc.v4.u32 {%1, %2, %3, %4}, [ad1];\n\t" \
-      "@pb ld.global.nc.v4.u32 {tx, ty, tz, tw}, [ad2];\n\t"
+      "@!px ld.global.v4.u32 {%1, %2, %3, %4}, [ad1];\n\t" \
+      "@pb ld.global.v4.u32 {tx, ty, tz, tw}, [ad2];\n\t"
 // entries in shared memory (%11 = their 32-bit address)
 #define RASP_F_FETCH_SH \
       "mad.lo.u32 t0, jf, 16, %11;\n\t" \
