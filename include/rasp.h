@@ -116,7 +116,8 @@ typedef struct rasp_config {
     uint32_t in_cap;     /* l: input tape capacity (u holds l+1 words)         */
     uint32_t out_cap;    /* s: output capacity (y holds s+1 words)             */
     uint32_t flags;      /* RASP_SCHED_* | RASP_DISPATCH_* | RASP_COLLECT_STATS */
-    uint32_t epoch;      /* steps between warp scheduling points; 0 = default  */
+    uint32_t epoch;      /* steps (fused entries, where programs have them)
+                            between warp scheduling points; 0 = default       */
     uint32_t warps_per_cta; /* persistent kernels: warps per CTA (SMEM-staged
                             up to 8, HBM-slab up to 4); 0 = default           */
     uint32_t refill_min; /* persistent kernels: idle lanes that trigger a
@@ -184,6 +185,11 @@ int rasp_batch_create(const rasp_config* cfg, uint64_t num_vms,
  * program v) or [num_vms] program index per VM (one program shared by many
  * VMs, e.g. a rollout of one candidate over many inputs).
  * Resets i = a = 0, steps = 0, status = RUNNING, u_0 = y_0 = 0, y = 0.
+ * WRAP programs are also decoded on the device, into entries of several
+ * instructions that the schedules AUTO, PERSIST_GL and SHARED and the pools run
+ * from while a VM has not written into its program (results do not depend on
+ * it): not with RASP_COLLECT_STATS, RASP_DISPATCH_VOTE or RASP_STEP_BLOCK, nor
+ * where the programs fill more than half of the memories.
  * EINVAL: odd program length, 2m > n of a VM using it, bad index. The copy
  * to the device is issued before the per-program checks run (so that they
  * overlap it); after a failed check the batch holds no programs and
