@@ -1059,6 +1059,16 @@ __device__ __forceinline__ uint32_t one_step(Mem M, const uint64_t* __restrict__
   return step_general<MASKED, CHECKED, HIST, CLASSIC>(M, T, Y, P, r, h);
 }
 
+// The epoch loops take i (+) 2 = ip + 2 unreduced (ibase = 0) and do not fetch
+// there: at the end of memory, or where i (+) 2 wraps at 2^w, they can end an
+// epoch with ip >= ilim. Whoever takes a general step after one reduces it first.
+__device__ __forceinline__ void reduce_ip(const Params& P, Regs& r) {
+  if (r.ip < r.ilim) return;
+  const uint64_t i = (uint64_t)r.ip & P.wmask;
+  r.ip = mod_n(i, r.n);
+  r.ibase = i - r.ip;
+}
+
 // Run up to `epoch` steps of every active lane with the epoch loop of
 // fast_loop_ptx (no counters, select dispatch; CHECKED on 8-byte slabs). Each round runs the
 // loop for at most the smallest step countdown of the warp; then the lanes
@@ -1124,12 +1134,7 @@ __device__ __forceinline__ void run_epoch_loop(Mem M, const uint64_t* T, uint64_
       }
       general = rare || r.left == 0u;
       if (general) {
-        if (r.ip >= r.ilim) {
-          // the loop took i (+) 2 = ip + 2 unreduced (ibase = 0): reduce it
-          const uint64_t i = (uint64_t)r.ip & P.wmask;
-          r.ip = mod_n(i, r.n);
-          r.ibase = i - r.ip;
-        }
+        reduce_ip(P, r);
         r.have = false;
         const uint32_t st = step_general<MASKED, CHECKED, false, CLASSIC>(M, T, Y, P, r, h);
         if (st == CONT) {

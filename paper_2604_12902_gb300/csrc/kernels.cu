@@ -467,7 +467,10 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
       if constexpr (std::is_same<Mem, ShView>::value) return M;     // notices writes into the program itself
       else return CodeView<Mem>{M, G.plen};
     }();
+    // a clean VM of a shared program that has left its entries comes from
+    // run_epoch_loop, whose i (+) 2 may still have to be reduced
     if (F.on) r.ip = 2u * (F.op.y & FO_COUNT ? fuse_instr(G, F.cur) : F.op.x);
+    else reduce_ip(P, r);
     r.have = false;
     for (uint32_t out = 0; active && stall;) {
       const uint32_t st = step_general<MASKED, false, false, CLASSIC>(V, T, Y, P, r, h);
