@@ -433,7 +433,7 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
   if (fm) {
     const uint32_t wait = idle_exit ? idle_exit : 12u;
     const uint32_t zero = P.ellp & 1u;                   // the stride of the tapes is even
-    for (uint32_t it = (epoch + 1u) & ~1u; it;) {
+    for (uint32_t it = (min(epoch, ~1u) + 1u) & ~1u; it;) {   // even, and not zero for the largest epoch
       const uint32_t c = min(it, kFuseChunk);
       it -= c;
       if (active && F.on) {

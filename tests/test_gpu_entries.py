@@ -68,3 +68,18 @@ def test_shared_machines_run_off_the_end_of_memory(rasp, w, epoch):
             st, _ = oracle_state(wl, budget=t, threads=8)
             assert_same_state(b.read_state(), st, wl.ell, wl.s, what="w %d epoch %d budget %d" % (w, epoch, t))
     assert (st.steps > 2 * (2 * 36 + 30)).all() and (st.status == 1).all()
+
+
+@pytest.mark.parametrize("epoch", [1, (1 << 32) - 2, (1 << 32) - 1])
+@pytest.mark.parametrize("shared", [False, True])
+def test_smallest_and_largest_epochs(rasp, shared, epoch):
+    """Every epoch takes a step: entries go in pairs, and the largest count of
+    them must not round up to none."""
+    wl = W.shared_programs(num_programs=4, vms_per_program=64) if shared else W.template_programs(num_vms=256, seed=7)
+    flags = rasp.SCHED_SHARED if shared else rasp.SCHED_AUTO
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s, flags=flags, epoch=epoch) as b:
+        b.load_workload(wl)
+        for t in (50, 4096):
+            b.run(t)
+            st, _ = oracle_state(wl, budget=t, threads=8)
+            assert_same_state(b.read_state(), st, wl.ell, wl.s, what="epoch %d budget %d" % (epoch, t))
