@@ -188,8 +188,9 @@ int rasp_batch_create(const rasp_config* cfg, uint64_t num_vms,
  * WRAP programs are also decoded on the device, into entries of several
  * instructions that the schedules AUTO, PERSIST_GL and SHARED and the pools run
  * from while a VM has not written into its program (results do not depend on
- * it): not with RASP_COLLECT_STATS, RASP_DISPATCH_VOTE or RASP_STEP_BLOCK, nor
- * where the programs fill more than half of the memories.
+ * it; rasp_describe says whether there are any): not with RASP_COLLECT_STATS,
+ * RASP_DISPATCH_VOTE or RASP_STEP_BLOCK, nor where the programs fill more than
+ * half of the memories.
  * EINVAL: odd program length, 2m > n of a VM using it, bad index. The copy
  * to the device is issued before the per-program checks run (so that they
  * overlap it); after a failed check the batch holds no programs and
@@ -314,8 +315,9 @@ int rasp_plan_bucket(rasp_batch* b, uint32_t bucket, uint32_t sched, uint32_t ep
  * run; the bytes of a word of M ("word_bytes": 4 for w <= 32 on the plain
  * and HBM-slab schedules, else 8) and of a program word as the pack reads it
  * ("program_word_bytes": 4 for programs kept as loaded by
- * rasp_load_programs_i32, else 8); whether runs replay a CUDA graph; the
- * autotuner's report. EINVAL if buf is too small. Does not touch the GPU. */
+ * rasp_load_programs_i32, else 8); whether the loaded programs were decoded
+ * into entries ("entries", see rasp_load_programs); whether runs replay a CUDA
+ * graph; the autotuner's report. EINVAL if buf is too small. Does not touch the GPU. */
 int rasp_describe(const rasp_batch* b, char* buf, uint64_t size);
 
 /* ---- running a caller-owned state store without allocating ---------------

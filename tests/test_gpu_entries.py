@@ -1,5 +1,7 @@
-"""Machines beside their fused entries (runs of instructions decoded when
-programs are loaded), against the oracle: code stored or read behind the
+"""Machines with fused entries (runs of instructions decoded when programs are
+loaded; every test here asks rasp_describe whether they were), against the
+oracle: programs of one to many mask records, the limits of 16 bits in an
+entry, memories that differ from the loaded program, code read behind the
 program that runs off the end of memory, and launch settings at the ends of
 their range. Needs a GPU."""
 import numpy as np
@@ -7,6 +9,7 @@ import pytest
 
 from paper_2604_12902_gb300 import workloads as W
 from tests.helpers import assert_same_state, oracle_state
+from tests.test_gpu_fused import machines
 
 pytestmark = pytest.mark.gpu
 LOD, ADD, MUL, STO, BNZ, RD, PRI = 1, 2, 3, 4, 5, 6, 7
@@ -30,6 +33,118 @@ def flat(progs, n, tapes, w=64, s=3, cap=3000, pvm=None):
     return W.Workload("entries", np.concatenate(progs).astype(np.int64), off, np.full(V, n, np.uint32),
                       tapes.astype(np.int64).reshape(-1), np.arange(V + 1, dtype=np.uint64) * np.uint64(ell),
                       np.full(V, cap, np.uint64), ell, s, w, pvm)
+
+
+def check(rasp, wl, budgets, what, classic=False, i32=True, entries=True, **kw):
+    """From c_0 twice through the budgets; `entries`: the programs have them."""
+    flags = kw.pop("flags", 0) | (rasp.ISA_CLASSIC if classic else 0)
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s, word_bits=wl.w, flags=flags, **kw) as b:
+        if i32:
+            rasp.rasp_load_programs_i32(b.h, wl.programs, wl.prog_off, wl.prog_of_vm)
+            b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+        else:
+            b.load_workload(wl)
+        assert b.describe()["entries"] is entries, what
+        for _ in range(2):
+            for t in budgets:
+                b.run(t)
+                st, _ = oracle_state(wl, budget=t, threads=8, classic=classic)
+                assert_same_state(b.read_state(), st, wl.ell, wl.s, what="%s, budget %d" % (what, t))
+            b.reset()
+
+
+@pytest.mark.parametrize("w", [64, 48, 32, 20, 8])
+@pytest.mark.parametrize("m", [31, 64, 65, 130])
+def test_programs_of_one_to_three_records(rasp, m, w):
+    check(rasp, machines(700, m, w, seed=2000 * m + w, extra=2 * m + 8), [3, 20, 21, 200, 1000], "m=%d w=%d" % (m, w),
+          i32=(m + w) % 2 == 0)
+
+
+@pytest.mark.parametrize("w", [64, 48, 33, 32, 31])
+@pytest.mark.parametrize("classic", [False, True])
+def test_words_beyond_32_bits(rasp, w, classic):
+    wl = machines(1500, 40, w, seed=140 + w, extra=90, huge=True)
+    check(rasp, wl, [9, 60, 1000], "huge words w=%d" % w, classic=classic, i32=False)
+    check(rasp, machines(700, 70, w, seed=105, extra=150), [7, 64, 1000], "classic %s w=%d" % (classic, w), classic=classic)
+
+
+@pytest.mark.parametrize("p_code", [0.0, 0.3])
+def test_long_programs_and_code_words(rasp, p_code):
+    check(rasp, machines(150, 513, 64, seed=106, p_code=p_code, extra=1030), [100, 1000], "m=513 code %.1f" % p_code)
+
+
+@pytest.mark.parametrize("w", [64, 32])
+@pytest.mark.parametrize("V,m", [(33_000, 65), (25_000, 150)])
+def test_programs_decoded_per_lane(rasp, V, m, w):
+    """More than 24,000 machines: the decoder that takes a program per lane and
+    keeps only the entries it reaches, over two and three mask records."""
+    check(rasp, machines(V, m, w, seed=150 + w + m, extra=2 * m + 8), [40, 1000], "per lane m=%d w=%d" % (m, w), i32=w == 64)
+
+
+def test_some_programs_write_into_themselves(rasp):
+    """Half of the programs: the batch has entries, those programs run from memory."""
+    a, c = W.random_programs(num_vms=512, seed=103, mem_words=200), machines(512, 32, 64, seed=113, extra=136)
+    own = (np.arange(512) % 16 < 8)[:, None]
+    prog = np.where(own, a.programs.reshape(512, -1), c.programs.reshape(512, -1))
+    check(rasp, W.Workload("mixed", prog.reshape(-1), a.prog_off, c.mem_words, c.tapes, c.tape_off, c.caps, c.ell, c.s),
+          [20, 1000], "half")
+
+
+@pytest.mark.parametrize("w", [64, 32])
+def test_restored_memories_run_from_memory(rasp, w):
+    """A checkpoint whose memory differs from the loaded program's words; the
+    next reset runs the loaded program again."""
+    a, c = machines(300, 30, w, seed=111, extra=64), machines(300, 30, w, seed=112, extra=64)
+    with rasp.Batch(a.mem_words, a.ell, a.s, word_bits=w) as b:
+        b.load_workload(a)
+        assert b.describe()["entries"]
+        with rasp.Batch(c.mem_words, c.ell, c.s, word_bits=w) as d:
+            d.load_workload(c)
+            st = d.read_state()
+        b.load_inputs(c.tapes, c.tape_off, c.caps)
+        b.load_state(st)
+        for t in (60, 500):
+            b.run(t)
+            assert_same_state(b.read_state(), oracle_state(c, budget=t, threads=8)[0], c.ell, c.s, what="restored")
+        b.load_inputs(a.tapes, a.tape_off, a.caps)
+        b.reset()
+        b.run(500)
+        assert_same_state(b.read_state(), oracle_state(a, budget=500, threads=8)[0], a.ell, a.s, what="reset")
+
+
+# ---- the 16-bit fields of an entry
+@pytest.mark.parametrize("w", [64, 32, 17])
+@pytest.mark.parametrize("classic", [False, True])
+def test_operands_around_65535(rasp, w, classic):
+    wl = machines(120, 24, w, seed=160 + w, extra=70_000)
+    n = int(wl.mem_words[0])
+    rng = np.random.default_rng(w)
+    prog = wl.programs.reshape(120, -1, 2)
+    edge = rng.choice([65533, 65534, 65535, 65536, 65537, 65538, n - 2, n - 1, 60, 61], size=prog.shape[:2])
+    mem = np.isin(prog[:, :, 0], (ADD, MUL, STO, RD, PRI)) & (rng.random(prog.shape[:2]) < .7)
+    prog[:, :, 1] = np.where(mem, edge, prog[:, :, 1])
+    check(rasp, wl, [25, 500], "operands at 2^16, w=%d" % w, classic=classic, i32=w != 17)
+
+
+@pytest.mark.parametrize("m,entries", [(65_535, True), (65_536, False)])
+@pytest.mark.parametrize("w", [64, 32])
+def test_longest_programs(rasp, m, entries, w):
+    """Jumps between the first and the last records of 65,535 instructions (one
+    more has no entries), operands and wide constants (a + the program word at
+    2p + 1) on both sides of word 65,535."""
+    V, rng = 24, np.random.default_rng(m + w)
+    op = rng.choice([LOD, ADD, BNZ, PRI, STO], size=(V, m), p=[.32, .34, .25, .05, .04])
+    edge = lambda at, width: np.clip(at + rng.integers(-width, width, (V, m)), 0, None)
+    pick = rng.integers(0, 4, (V, m))
+    target = 2 * np.where(pick == 0, edge(40, 40), np.where(pick == 1, m - 1 - rng.integers(0, 70, (V, m)),
+                          np.where(pick == 2, edge(32_767, 60), rng.integers(0, m, (V, m)))))
+    word = np.where(pick == 0, edge(65_535, 4), np.where(pick == 1, 2 * m - 1 - rng.integers(0, 9, (V, m)),
+                    rng.integers(0, 2 * m, (V, m))))
+    const = np.where(pick == 0, rng.integers(40_000, 1 << 30, (V, m)), rng.integers(-2, 3, (V, m)))
+    arg = np.where(op == BNZ, target, np.where(op == LOD, const, np.where(op == STO, 2 * m + 7 + pick, word)))
+    prog = np.stack([op, arg], axis=2).reshape(V, 2 * m)
+    wl = flat(list(prog), 4 * m + 40, np.zeros((V, 4)), w=w, s=40, cap=20_000)
+    check(rasp, wl, [100, 20_000], "m=%d w=%d" % (m, w), entries=entries, i32=w == 32)
 
 
 def code_from_the_tape(w, seed, V=224, programs=7, k=36):
@@ -63,6 +178,7 @@ def test_shared_machines_run_off_the_end_of_memory(rasp, w, epoch):
     wl = code_from_the_tape(w, seed=70 + w)
     with rasp.Batch(wl.mem_words, wl.ell, wl.s, word_bits=w, flags=rasp.SCHED_SHARED, epoch=epoch) as b:
         b.load_workload(wl)
+        assert b.describe()["entries"]
         for t in (90, 111, 112, 113, 250, 3000):
             b.run(t)
             st, _ = oracle_state(wl, budget=t, threads=8)
@@ -79,6 +195,7 @@ def test_smallest_and_largest_epochs(rasp, shared, epoch):
     flags = rasp.SCHED_SHARED if shared else rasp.SCHED_AUTO
     with rasp.Batch(wl.mem_words, wl.ell, wl.s, flags=flags, epoch=epoch) as b:
         b.load_workload(wl)
+        assert b.describe()["entries"]
         for t in (50, 4096):
             b.run(t)
             st, _ = oracle_state(wl, budget=t, threads=8)
