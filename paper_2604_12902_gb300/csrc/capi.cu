@@ -408,8 +408,7 @@ cudaError_t ensure_prog64(rasp_batch* b, cudaStream_t st) {
 // the HBM-slab epoch loop when the programs have fused entries.
 bool tracks_code(const rasp_batch* b, const Group& g) {
   if (g.sched == RASP_SCHED_SHARED) return true;
-  const StepVariant v = variant_of(b);
-  return g.sched == RASP_SCHED_PERSIST_GL && b->S.fops && !v.checked && !v.hist && !v.vote && !v.block;
+  return g.sched == RASP_SCHED_PERSIST_GL && b->S.fops && runs_entries(variant_of(b));
 }
 
 // Before a run (eagerly, outside any captured graph): where codedirty is not
@@ -709,8 +708,7 @@ bool self_writing(const W* words, const uint64_t* offsets, uint64_t num_programs
 // more than half of the memories), where no kernel would run from them, or
 // where a program has more instructions than an entry can name.
 uint4* place_fused(const rasp_batch* b, uint64_t total, bool keep32) {
-  const StepVariant v = variant_of(b);
-  if (!total || v.checked || v.hist || v.vote || v.block || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
+  if (!total || !runs_entries(variant_of(b)) || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
   const uint64_t lo = keep32 && owns_code(b) ? 0 : 8ull * total;
   const uint64_t end = keep32 ? 4ull * kept_words_at(b) : 8ull * b->mem_words;
   if (lo + 8ull * total > end || 8ull * total > (b->narrow ? 4ull : 8ull) * b->mem_words) return nullptr;
@@ -1508,9 +1506,14 @@ int rasp_describe(const rasp_batch* b, char* buf, uint64_t size) {
   s += "], \"launches\": [";
   first = true;
   for (const Group& g : b->groups) {
+    // what is launched (its first budget round), which few VMs or fused entries make differ from the plan
+    PersistLaunch l{g.shape.grid, g.shape.warps, 32u, false};
+    if (g.sched == RASP_SCHED_PERSIST || g.sched == RASP_SCHED_PERSIST_GL)
+      l = persist_launch(variant_of(b), b->programs_loaded && b->S.fops, g.count, false, g.shape);
     char tmp[256];
-    snprintf(tmp, sizeof(tmp), "%s{\"vms\": %u, \"schedule\": \"%s\", \"grid\": %u}", first ? "" : ", ",
-             g.count, names[std::min<uint32_t>(g.sched >> 4, 4u)], g.shape.grid);
+    snprintf(tmp, sizeof(tmp), "%s{\"vms\": %u, \"schedule\": \"%s\", \"grid\": %u, \"warps_per_cta\": %u, "
+             "\"lanes_per_warp\": %u}", first ? "" : ", ", g.count, names[std::min<uint32_t>(g.sched >> 4, 4u)],
+             l.grid, l.warps, l.lanes);
     s += tmp;
     first = false;
   }

@@ -77,6 +77,21 @@ void plain_configure(const StepVariant& var);
 cudaError_t launch_plain(const StepVariant& var, const DevState& S, const Params& P,
                          const uint32_t* ids, uint32_t count, cudaStream_t stream);
 
+// The run kernels of this variant take fused entries (on the HBM-slab and the
+// shared-program schedule, and in the pools).
+inline bool runs_entries(const StepVariant& v) { return !v.checked && !v.hist && !v.vote && !v.block; }
+
+// What a persistent launch over `count` VMs is: the resident CTAs of the kernel
+// that runs (with fused entries fewer fit an SM), at most as many as the VMs
+// fill; few VMs in the HBM-slab form spread over one-warp CTAs. dense: a
+// compacted queue, of at most `count` VMs.
+struct PersistLaunch {
+  uint32_t grid, warps, lanes;   // CTAs, warps per CTA, lanes of a warp that take VMs
+  bool fuse;
+};
+PersistLaunch persist_launch(const StepVariant& var, bool entries, uint32_t count, bool dense,
+                             const PersistShape& shape);
+
 // Fills grid/smem of `shape` for the current device (occupancy-sized) and
 // returns the resident CTAs per SM (0 if the shape cannot launch).
 int persist_configure(const StepVariant& var, PersistShape& shape);

@@ -1594,18 +1594,18 @@ int persist_configure(const StepVariant& var, PersistShape& sh) {
   return per_sm;
 }
 
-cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Params& P, const Queue& Q,
-                           const PersistShape& sh, cudaStream_t stream) {
-  if ((!Q.count && !Q.dcount) || !sh.grid) return cudaSuccess;
-  StepVariant v = shape_variant(var, sh);
-  v.fuse = S.fops != nullptr;
-  const uint32_t resident = v.fuse ? std::min(sh.grid, sh.fuse_ctas * (uint32_t)num_sms()) : sh.grid;
-  uint32_t grid = resident;
-  const uint32_t warps_needed = (Q.count + 31u) / 32u;   // with dcount, Q.count is an upper bound
-  uint32_t cta_warps = sh.warps, cta_lanes = 32u;
+PersistLaunch persist_launch(const StepVariant& var, bool entries, uint32_t count, bool dense,
+                             const PersistShape& sh) {
+  PersistLaunch l{};
+  l.warps = sh.warps;
+  l.lanes = 32u;
+  l.fuse = entries && !sh.staged && runs_entries(shape_variant(var, sh));
+  const uint32_t resident = l.fuse ? std::min(sh.grid, sh.fuse_ctas * (uint32_t)num_sms()) : sh.grid;
+  l.grid = resident;
+  const uint32_t warps_needed = (count + 31u) / 32u;   // of a dense queue, count is an upper bound
   const uint32_t max_useful = (warps_needed + sh.warps - 1u) / sh.warps;
   const uint32_t spread = 8u * (uint32_t)num_sms();
-  if (!sh.staged && !Q.dcount && warps_needed < spread && resident * sh.warps >= 2u * spread) {
+  if (!sh.staged && !dense && warps_needed < spread && resident * sh.warps >= 2u * spread) {
     // Few VMs (under 38,912 on 152 SMs): 8 warps per SM, each with as few lanes
     // as that takes, and four where that would be five to eight: the lanes of a
     // warp wait for one another's misses and general steps. Run kernel, 32
@@ -1613,25 +1613,34 @@ cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Para
     // 178, 2,048 templates 143 -> 101, 16,384 153 -> 133, 32,768 193 -> 187,
     // 32,768 search programs 8.2 -> 7.3 ms. With 16 warps per SM 2,048
     // templates take 134 us and 16,384 181.
-    cta_warps = 1u;
-    cta_lanes = (Q.count + spread - 1u) / spread;
-    if (cta_lanes > 4u && cta_lanes <= 8u) cta_lanes = 4u;
-    grid = (Q.count + cta_lanes - 1u) / cta_lanes;
-  } else if (grid > max_useful) {
-    grid = max_useful;
+    l.warps = 1u;
+    l.lanes = (count + spread - 1u) / spread;
+    if (l.lanes > 4u && l.lanes <= 8u) l.lanes = 4u;
+    l.grid = (count + l.lanes - 1u) / l.lanes;
+  } else if (l.grid > max_useful) {
+    l.grid = max_useful;
   }
+  return l;
+}
+
+cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Params& P, const Queue& Q,
+                           const PersistShape& sh, cudaStream_t stream) {
+  if ((!Q.count && !Q.dcount) || !sh.grid) return cudaSuccess;
+  const PersistLaunch l = persist_launch(var, S.fops != nullptr, Q.count, Q.dcount != nullptr, sh);
+  StepVariant v = shape_variant(var, sh);
+  v.fuse = l.fuse;
   // the last (resident lanes) positions are the tail: served one VM at a
   // time to idle lanes so that no lane queues a second VM behind a running one
   Queue q = Q;
-  q.lanes = cta_lanes;
-  const uint64_t lanes = (uint64_t)grid * cta_warps * cta_lanes;
+  q.lanes = l.lanes;
+  const uint64_t lanes = (uint64_t)l.grid * l.warps * l.lanes;
   q.soft_end = Q.count > lanes ? (uint32_t)(Q.count - lanes) : 0u;
   if (sh.staged)
-    pick_staged(v)<<<grid, 32u * sh.warps, sh.smem, stream>>>(S, P, q, sh.ncap, sh.slot_words, sh.epoch,
+    pick_staged(v)<<<l.grid, 32u * l.warps, sh.smem, stream>>>(S, P, q, sh.ncap, sh.slot_words, sh.epoch,
                                                                  sh.refill_min,
                                                                  inject_wait_expiry() ? 0u : WAIT_LIMIT);
   else
-    pick_global(v)<<<grid, 32u * cta_warps, 0, stream>>>(S, P, q, sh.epoch, sh.idle_exit);
+    pick_global(v)<<<l.grid, 32u * l.warps, 0, stream>>>(S, P, q, sh.epoch, sh.idle_exit);
   return cudaGetLastError();
 }
 

@@ -200,3 +200,25 @@ def test_smallest_and_largest_epochs(rasp, shared, epoch):
             b.run(t)
             st, _ = oracle_state(wl, budget=t, threads=8)
             assert_same_state(b.read_state(), st, wl.ell, wl.s, what="epoch %d budget %d" % (epoch, t))
+
+
+def test_staged_buckets_keep_their_resident_warps(rasp):
+    """Beside entries the SMEM-staged kernel is launched at its own occupancy."""
+    small, large = (W.template_programs(num_vms=1 << 14, seed=s, mem_words=n) for s, n in ((3, 256), (4, 512)))
+    V = 1 << 14
+    wl = W.Workload("two sizes", np.concatenate([small.programs, large.programs]),
+                    np.concatenate([small.prog_off, large.prog_off[1:] + small.prog_off[-1]]),
+                    np.concatenate([small.mem_words, large.mem_words]), np.concatenate([small.tapes, large.tapes]),
+                    np.concatenate([small.tape_off, large.tape_off[1:] + small.tape_off[-1]]),
+                    np.concatenate([small.caps, large.caps]), small.ell, small.s)
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s) as b:
+        b.load_workload(wl)
+        k = b.describe()["buckets"][0]
+        b.plan_bucket(k["index"], rasp.SCHED_PERSIST)
+        d = b.describe()
+        assert d["entries"] and [x["schedule"] for x in d["launches"]] == ["persist", "persist_gl"]
+        k = d["buckets"][0]
+        assert k["ctas_per_sm"] >= 3 and d["launches"][0]["grid"] == min(k["grid"], V // 32)
+        b.run()
+        st, _ = oracle_state(wl, threads=8)
+        assert_same_state(b.read_state(), st, wl.ell, wl.s, what="staged beside entries")
