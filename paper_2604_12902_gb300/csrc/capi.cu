@@ -1098,18 +1098,27 @@ int rasp_read_state(rasp_batch* b, uint64_t first, uint64_t count, rasp_state_vi
       CK(cudaMemcpyAsync(m32.data(), S.mem32 + lo, 4 * (hi - lo), cudaMemcpyDeviceToHost, st));
     } else if (need == hi - lo) {
       CK(cudaMemcpyAsync(out->mem, S.mem + lo, 8 * need, cudaMemcpyDeviceToHost, st));
-    } else if (uniform && !(b->h_n[first] & 1u)) {   // equal slabs: whole groups by one strided copy
+    } else if (uniform && !(b->h_n[first] & 1u)) {
+      // equal slabs: the whole groups by one strided copy (a pitch has to stay
+      // below 2^31 bytes: larger groups by a copy each), what is left by its own
       const uint64_t n = b->h_n[first], end = first + count;
       const uint64_t g0 = std::min(end, (first + kSlabGroup - 1) / kSlabGroup * kSlabGroup);
       const uint64_t g1 = std::max(g0, end / kSlabGroup * kSlabGroup);
-      auto part = [&](uint64_t v, uint64_t vms, uint64_t rows) {
-        if (!vms || !rows) return cudaSuccess;
-        return cudaMemcpy2DAsync(out->mem + (v - first) * n, 8 * n * vms, S.mem + b->h_memoff[v],
-                                 8 * (n * vms + kGroupPad), 8 * n * vms, rows, cudaMemcpyDeviceToHost, st);
+      const uint64_t row = 8 * n * kSlabGroup;
+      auto slabs = [&](uint64_t v, uint64_t vms) {
+        if (!vms) return cudaSuccess;
+        return cudaMemcpyAsync(out->mem + (v - first) * n, S.mem + b->h_memoff[v], 8 * n * vms,
+                               cudaMemcpyDeviceToHost, st);
       };
-      CK(part(first, g0 - first, 1));
-      CK(part(g0, kSlabGroup, (g1 - g0) / kSlabGroup));
-      CK(part(g1, end - g1, 1));
+      CK(slabs(first, g0 - first));
+      if (row + 8 * kGroupPad < (1ull << 30)) {
+        if (g1 > g0)
+          CK(cudaMemcpy2DAsync(out->mem + (g0 - first) * n, row, S.mem + b->h_memoff[g0], row + 8 * kGroupPad, row,
+                               (g1 - g0) / kSlabGroup, cudaMemcpyDeviceToHost, st));
+      } else {
+        for (uint64_t v = g0; v < g1; v += kSlabGroup) CK(slabs(v, kSlabGroup));
+      }
+      CK(slabs(g1, end - g1));
     } else {
       mbuf.resize(hi - lo);
       CK(cudaMemcpyAsync(mbuf.data(), S.mem + lo, 8 * (hi - lo), cudaMemcpyDeviceToHost, st));

@@ -222,3 +222,21 @@ def test_staged_buckets_keep_their_resident_warps(rasp):
         b.run()
         st, _ = oracle_state(wl, threads=8)
         assert_same_state(b.read_state(), st, wl.ell, wl.s, what="staged beside entries")
+
+
+def test_reading_the_largest_padded_slabs(rasp):
+    """Equal memories of 2^27 words on the shared-program schedule: two of them
+    are more bytes than a strided copy takes as a pitch."""
+    n, V = 1 << 27, 3
+    prog = np.array([LOD, 7, STO, n - 1, LOD, 9, STO, 100, RD, 101, 0, 0])
+    wl = flat([prog], n, np.arange(1, V + 1).reshape(V, 1), pvm=np.zeros(V, np.uint32))
+    want = {1: 7, 2: STO, 0: LOD, 3: n - 1, 4: LOD, 5: 9, 6: STO, 7: 100, 8: RD, 9: 101, 100: 9, n - 1: 7}
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s, flags=rasp.SCHED_SHARED) as b:
+        b.load_workload(wl)
+        b.run()
+        for first, count in ((0, 3), (1, 2)):
+            got = b.read_state(first, count)
+            assert (got["steps"] == 5).all() and (got["status"] == 1).all()
+            for k, slab in enumerate(got.pop("mem").reshape(count, n)):
+                at = np.flatnonzero(slab)
+                assert dict(zip(at.tolist(), slab[at].tolist())) == {**want, 101: first + k + 1}
