@@ -101,7 +101,7 @@ struct rasp_batch {
   Layout L{};
   char* base = nullptr;
   bool owns = false;
-  DevState S{};
+  RunState S{};
   uint64_t* d_prog = nullptr;
   // Programs loaded as 4-byte words are kept as such in the upper half of
   // the program area when they fit beside their widened copy: the pack
@@ -461,7 +461,7 @@ int check_device_error(rasp_batch* b) {
 
 }  // namespace
 
-const DevState& rasp::batch_dev_state(const rasp_batch* b) { return b->S; }
+const RunState& rasp::batch_run_state(const rasp_batch* b) { return b->S; }
 
 Params rasp::batch_params(const rasp_batch* b) {
   Params P{};

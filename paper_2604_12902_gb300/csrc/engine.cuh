@@ -43,6 +43,12 @@ struct DevState {
   const uint64_t* tape;       // u_1..u_l, stride ellp words per VM
   uint64_t* y;                // y_1..y_s, stride sp words per VM
   uint8_t* codedirty;         // 1 if the VM may have written into its program words (NULL: untracked)
+};
+
+// What the kernels that run fused entries take besides. It stays out of DevState:
+// with four more pointers in its arguments the SMEM-staged kernel, which has no
+// use for them, was compiled 8 % slower (2^18 templates 1.85 -> 2.00 ms).
+struct RunState : DevState {
   const uint4* fops;          // fused entries of the programs (fuse.cuh; NULL: none)
   const uint4* frec;          // masks of the instructions that have one
   const uint64_t* prog_off;   // word offset of each program

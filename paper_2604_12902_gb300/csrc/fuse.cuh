@@ -212,7 +212,7 @@ __device__ __forceinline__ uint32_t fuse_rank(uint4 r, uint32_t e) {
   return r.z + (uint32_t)__popcll(fuse_mask(r) & ((1ull << (e & 63u)) - 1ull));
 }
 
-__device__ __forceinline__ FuseProg fuse_prog(const DevState& S, uint32_t v, uint32_t ilim) {
+__device__ __forceinline__ FuseProg fuse_prog(const RunState& S, uint32_t v, uint32_t ilim) {
   const uint32_t p = S.prog_of_vm ? S.prog_of_vm[v] : v;
   const uint64_t po = S.prog_off[p];
   FuseProg G;
@@ -277,7 +277,7 @@ struct FuseRow {
   uint32_t p;
   uint32_t dirty;
 };
-__device__ __forceinline__ FuseRow fuse_row(const DevState& S, uint32_t v) {
+__device__ __forceinline__ FuseRow fuse_row(const RunState& S, uint32_t v) {
   FuseRow w;
   w.dirty = S.codedirty[v];
   w.p = S.prog_of_vm ? S.prog_of_vm[v] : v;
@@ -287,7 +287,7 @@ __device__ __forceinline__ FuseRow fuse_row(const DevState& S, uint32_t v) {
 }
 
 // VM v's entries (after arm_regs); without them it runs one instruction at a time.
-__device__ __forceinline__ void fuse_attach(const DevState& S, const FuseRow& w, Regs& r, Fused& F) {
+__device__ __forceinline__ void fuse_attach(const RunState& S, const FuseRow& w, Regs& r, Fused& F) {
   r.clean = w.dirty == 0u;
   FuseProg G;
   G.plen = (uint32_t)(w.pe - w.po);

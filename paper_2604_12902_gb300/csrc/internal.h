@@ -62,7 +62,7 @@ cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint6
 // lanes run the program's VMs pv_ids[pv_off[p] .. pv_off[p+1]) (epoch loop
 // for WRAP without counters, else one step at a time). The slabs of VMs
 // with codedirty = 0 need not hold their program words.
-cudaError_t launch_shared(const StepVariant& var, const DevState& S, const Params& P, const uint64_t* prog,
+cudaError_t launch_shared(const StepVariant& var, const RunState& S, const Params& P, const uint64_t* prog,
                           const uint64_t* prog_off, const uint32_t* pv_off, const uint32_t* pv_ids,
                           uint32_t num_programs, uint32_t max_plen, uint32_t epoch, cudaStream_t stream);
 
@@ -96,7 +96,7 @@ PersistLaunch persist_launch(const StepVariant& var, bool entries, uint32_t coun
 // returns the resident CTAs per SM (0 if the shape cannot launch).
 int persist_configure(const StepVariant& var, PersistShape& shape);
 
-cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Params& P, const Queue& Q,
+cudaError_t launch_persist(const StepVariant& var, const RunState& S, const Params& P, const Queue& Q,
                            const PersistShape& shape, cudaStream_t stream);
 
 // Halting-time histogram (device): counts[nbins] of HALTED VMs by
@@ -144,7 +144,7 @@ bool inject_wait_expiry();
 // Device descriptor of one admitted request (a "slot"): its batch's state
 // store, the budget of its run and the word written to its completion flag.
 struct ServeSlot {
-  DevState S;
+  RunState S;
   uint64_t budget;       // max_steps of the request's run
   uint32_t num_vms;      // entries with this slot index name VMs below this
   uint32_t gen;          // written to done[slot] when its last VM stops (nonzero)
@@ -196,7 +196,7 @@ int create_batch(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_w
                  rasp_batch** out);
 
 // The state store and step parameters of a batch (for the serving pool).
-const DevState& batch_dev_state(const rasp_batch* b);
+const RunState& batch_run_state(const rasp_batch* b);
 Params batch_params(const rasp_batch* b);
 const uint32_t* batch_queue(const rasp_batch* b);   // VM ids in the batch's queue order (device)
 

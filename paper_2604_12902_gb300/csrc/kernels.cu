@@ -425,7 +425,7 @@ constexpr uint32_t kFuseOutside = 32;  // general steps at no entry's start befo
 
 template <bool MASKED, bool CLASSIC, class Mem>
 __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64_t* Y, const Params& P, Regs& r,
-                                                Fused& F, const DevState& S, uint32_t vm, Hist& h, bool& active,
+                                                Fused& F, const RunState& S, uint32_t vm, Hist& h, bool& active,
                                                 uint32_t& final_st, uint32_t epoch, uint32_t idle_exit,
                                                 uint32_t shared_tab = 0) {
   const uint32_t fm = __ballot_sync(FULL, active && F.on);
@@ -627,7 +627,7 @@ enum : uint32_t { PF_EMPTY = 0, PF_ID = 1, PF_REGS = 2, PF_NONE = 3 };   // PF_R
 // 4.56 (4.59), the halting rounds of 2^18 programs 82 (87).
 template <bool MASKED, bool CHECKED, bool HIST, bool VOTE, bool CLASSIC = false, bool LOOP = false,
           bool NARROW = false, bool FUSE = false>
-__global__ void __launch_bounds__(128, FUSE ? 6 : 7) k_persist_gl(DevState S, Params P, Queue Q, uint32_t epoch,
+__global__ void __launch_bounds__(128, FUSE ? 6 : 7) k_persist_gl(RunState S, Params P, Queue Q, uint32_t epoch,
                                                        uint32_t idle_exit) {
   static_assert(!LOOP || (!HIST && !VOTE), "the epoch loop serves select steps without counters");
   const uint32_t lane = threadIdx.x & 31u;
@@ -995,7 +995,7 @@ __global__ void k_ring_publish(unsigned long long* credits, unsigned long long c
 // k_shared: each lane takes the next VM from a shared-memory counter when
 // its VM stops and steps it with one_step (CHECKED semantics, counters).
 template <bool MASKED, bool CHECKED, bool HIST>
-__global__ void __launch_bounds__(128) k_shared(DevState S, Params P, const uint64_t* __restrict__ prog,
+__global__ void __launch_bounds__(128) k_shared(RunState S, Params P, const uint64_t* __restrict__ prog,
                                                 const uint64_t* __restrict__ prog_off,
                                                 const uint32_t* __restrict__ pv_off,
                                                 const uint32_t* __restrict__ pv_ids, uint32_t num_programs,
@@ -1061,7 +1061,7 @@ __global__ void __launch_bounds__(128) k_shared(DevState S, Params P, const uint
 // FUSE: clean VMs run from the program's fused entries, held in shared memory
 // behind its words.
 template <bool MASKED, bool FUSE>
-__global__ void __launch_bounds__(128, 7) k_shared_loop(DevState S, Params P, const uint64_t* __restrict__ prog,
+__global__ void __launch_bounds__(128, 7) k_shared_loop(RunState S, Params P, const uint64_t* __restrict__ prog,
                                                         const uint64_t* __restrict__ prog_off,
                                                         const uint32_t* __restrict__ pv_off,
                                                         const uint32_t* __restrict__ pv_ids, uint32_t num_programs,
@@ -1334,7 +1334,7 @@ int num_sms() {
 
 using PlainFn = void (*)(DevState, Params, const uint32_t*, uint32_t);
 using StagedFn = void (*)(DevState, Params, Queue, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t);
-using GlobalFn = void (*)(DevState, Params, Queue, uint32_t, uint32_t);
+using GlobalFn = void (*)(RunState, Params, Queue, uint32_t, uint32_t);
 
 template <bool M_, bool C_, bool H_>
 PlainFn plain_fn(bool vote) {
@@ -1498,7 +1498,7 @@ cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint6
   return cudaGetLastError();
 }
 
-using SharedFn = void (*)(DevState, Params, const uint64_t*, const uint64_t*, const uint32_t*, const uint32_t*,
+using SharedFn = void (*)(RunState, Params, const uint64_t*, const uint64_t*, const uint32_t*, const uint32_t*,
                          uint32_t, uint32_t);
 
 SharedFn pick_shared(const StepVariant& v) {
@@ -1509,7 +1509,7 @@ SharedFn pick_shared(const StepVariant& v) {
   return v.masked ? k_shared_loop<true, false> : k_shared_loop<false, false>;
 }
 
-cudaError_t launch_shared(const StepVariant& var, const DevState& S, const Params& P, const uint64_t* prog,
+cudaError_t launch_shared(const StepVariant& var, const RunState& S, const Params& P, const uint64_t* prog,
                           const uint64_t* prog_off, const uint32_t* pv_off, const uint32_t* pv_ids,
                           uint32_t num_programs, uint32_t max_plen, uint32_t epoch, cudaStream_t stream) {
   if (!num_programs) return cudaSuccess;
@@ -1623,7 +1623,7 @@ PersistLaunch persist_launch(const StepVariant& var, bool entries, uint32_t coun
   return l;
 }
 
-cudaError_t launch_persist(const StepVariant& var, const DevState& S, const Params& P, const Queue& Q,
+cudaError_t launch_persist(const StepVariant& var, const RunState& S, const Params& P, const Queue& Q,
                            const PersistShape& sh, cudaStream_t stream) {
   if ((!Q.count && !Q.dcount) || !sh.grid) return cudaSuccess;
   const PersistLaunch l = persist_launch(var, S.fops != nullptr, Q.count, Q.dcount != nullptr, sh);

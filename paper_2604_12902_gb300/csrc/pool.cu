@@ -178,7 +178,7 @@ int publish(rasp_pool* p, Request& r) {
   r.gen = (uint32_t)(r.ticket & 0x7FFFFFFFu) | 0x80000000u;   // nonzero
   *done_word(p, slot) = 0u;
   ServeSlot& hs = p->h_slots[slot];
-  hs.S = batch_dev_state(r.batch);
+  hs.S = batch_run_state(r.batch);
   hs.budget = r.max_steps;
   hs.num_vms = (uint32_t)r.num_vms;
   hs.gen = r.gen;
