@@ -1356,7 +1356,8 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
     tmin = 1e30f;
     for (uint32_t r = 0; r < reps && ce == cudaSuccess; ++r) {
       ce = copy_state(false);
-      b->dirty_valid = dirty_valid0;
+      // the trial's plan may keep codedirty where an earlier run did not
+      b->dirty_valid = dirty_valid0 && !untracked0;
       b->code_lazy = code_lazy0;
       b->ran_untracked = untracked0;
       if (ce == cudaSuccess) ce = settle_dirty(b, st);

@@ -240,3 +240,24 @@ def test_reading_the_largest_padded_slabs(rasp):
             for k, slab in enumerate(got.pop("mem").reshape(count, n)):
                 at = np.flatnonzero(slab)
                 assert dict(zip(at.tolist(), slab[at].tolist())) == {**want, 101: first + k + 1}
+
+
+def test_autotune_after_a_run_that_wrote_code(rasp):
+    """The plain schedule has written HALT over the first instruction of an
+    endless loop: the autotuner's trials must run that memory, where every
+    machine halts at once, and not the loaded program's entries."""
+    at = 14
+    prog = [LOD, 0, STO, 2 * at] + [LOD, 1] * (at - 2) + [LOD, 1, ADD, 60, STO, 60, BNZ, 2 * at]
+    wl = flat([np.array(prog)] * 64, 96, np.zeros((64, 2)), cap=1 << 40)
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s) as b:
+        b.load_workload(wl)
+        assert b.describe()["entries"]
+        k = b.describe()["buckets"][0]["index"]
+        b.plan_bucket(k, rasp.SCHED_PLAIN)
+        b.run(5)
+        rep = b.autotune(max_steps=10_000_000, reps=1)
+        ms = {t["schedule"]: t["ms"] for t in rep["trials"]}
+        assert max(v for name, v in ms.items() if name.startswith("persist_gl")) < 20, ms   # the loop takes seconds
+        b.run()
+        st, _ = oracle_state(wl, threads=8)
+        assert_same_state(b.read_state(), st, wl.ell, wl.s, what="after autotune")
