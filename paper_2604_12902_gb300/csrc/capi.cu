@@ -680,24 +680,33 @@ bool owns_code(const rasp_batch* b) {
   return !b->shared_programs && (b->cfg.flags & RASP_SCHED_MASK) != RASP_SCHED_SHARED;
 }
 
-// Whether most of the programs write into themselves (an eighth of their
-// instructions or more), by a look at up to 64 of them: their VMs would leave
-// the entries at once, and the kernel without entries runs them faster (65,536
-// random programs with n = 256: 212 us a run against 275).
+// Whether most of the programs are better run one instruction at a time, by a
+// look at up to 64 of them: an eighth of their instructions or more write into
+// the program (their VMs would leave the entries at once: 65,536 random programs
+// with n = 256 212 us a run without entries, 275 with), or do not fit an entry
+// though the one-instruction loop takes them in its stride -- operands behind
+// word 65,535, and constants beyond 16 bits where the entries may not read the
+// program words (4,096 machines in a loop of 10 steps with two such operands,
+// n = 70,000: 2.37 ms a run, from entries that they leave 2.52, and 4.4 before
+// few machines were spread over many warps; 131,072 with two wide constants in
+// 12 instructions 8.86 and 10.4 ms).
 template <class W>
-bool self_writing(const W* words, const uint64_t* offsets, uint64_t num_programs) {
+bool poor_entries(const W* words, const uint64_t* offsets, uint64_t num_programs, uint64_t wmask, bool own) {
   const uint64_t looks = std::min<uint64_t>(num_programs, 64);
-  uint64_t writing = 0;
+  uint64_t poor = 0;
   for (uint64_t q = 0; q < looks; ++q) {
-    const uint64_t p = q * num_programs / looks;
+    const uint64_t p = q * (num_programs / looks | 1ull) % num_programs;   // an odd stride: batches may be periodic
     const uint64_t len = offsets[p + 1] - offsets[p], seen = std::min<uint64_t>(len, 1024);
     const W* w = words + offsets[p];
-    uint64_t writes = 0;
-    for (uint64_t k = 0; k + 1 < seen; k += 2)
-      writes += (w[k] == 4 || w[k] == 6) && w[k + 1] >= 0 && (uint64_t)w[k + 1] < len ? 1 : 0;
-    writing += writes && 16 * writes >= seen ? 1 : 0;
+    uint64_t unfit = 0;
+    for (uint64_t k = 0; k + 1 < seen; k += 2) {
+      const uint64_t o = (uint64_t)(int64_t)w[k] & wmask, j = (uint64_t)(int64_t)w[k + 1] & wmask;
+      if (o == 1) unfit += !own && ((uint64_t)(int64_t)(int16_t)(uint16_t)j & wmask) != j ? 1 : 0;
+      else if (o != 5 && o - 1 < 7) unfit += ((o == 4 || o == 6) && j < len) || (j > 0xFFFF) ? 1 : 0;
+    }
+    poor += unfit && 16 * unfit >= seen ? 1 : 0;
   }
-  return 2 * writing > looks;
+  return 2 * poor > looks;
 }
 
 // The place of the fused entries (at most 16 bytes per instruction, 8 per
@@ -807,8 +816,8 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   CK(cudaStreamSynchronize(st));   // the caller's buffers are read before the call returns
   // fused entries: their place, and the smallest memory that runs each program
   const uint32_t* bound = b->S.n;
-  const bool from_memory = total && (word_size == 8 ? self_writing((const int64_t*)words, offsets, num_programs)
-                                                    : self_writing((const int32_t*)words, offsets, num_programs));
+  const bool from_memory = total && (word_size == 8 ? poor_entries((const int64_t*)words, offsets, num_programs, b->wmask, owns_code(b))
+                                                    : poor_entries((const int32_t*)words, offsets, num_programs, b->wmask, owns_code(b)));
   b->S.fops = from_memory ? nullptr : place_fused(b, total, keep32);
   b->S.frec = (const uint4*)(b->base + b->L.off_frec);
   b->S.prog_off = b->d_progoff;

@@ -250,12 +250,21 @@ struct Fused {
   uint4 op;             // the entry at cur (when on)
   uint32_t cur;
   bool on;              // the VM runs from its entries (its i is the entry's instruction)
+  uint32_t mark;        // Regs::left after its last general step
+  uint32_t debt;        // VM-steps that its stalls have cost beyond those its entries ran (kFuseGone: it has left)
 };
+constexpr uint32_t kFuseGone = ~0u;
 
 // The VM's next step needs the general path (or its run may stop here).
 __device__ __forceinline__ bool fuse_stalled(const Fused& F, const Regs& r, const Params& P) {
   const uint32_t c = (F.op.y >> 16) & 31u;
   return c - 1u >= r.left || ((F.op.y & FO_RD) && r.u0 >= P.ell);
+}
+
+// A VM is taken: no stalls yet.
+__device__ __forceinline__ void fuse_begin(Fused& F, const Regs& r) {
+  F.mark = r.left;
+  F.debt = 0u;
 }
 
 // Enter the entries at i if an entry starts there.
@@ -294,6 +303,7 @@ __device__ __forceinline__ void fuse_attach(const RunState& S, const FuseRow& w,
   G.mok = min(G.plen, r.ilim) >> 1;
   G.tab = S.fops + (w.po >> 1);
   G.rec = S.frec + (w.po >> 7) + w.p;
+  fuse_begin(F, r);
   fuse_enter(G, F, r);
   if (F.on && !(F.op.y & FO_COUNT) && (F.op.y & FO_MEM)) F.on = r.clean = false;
 }

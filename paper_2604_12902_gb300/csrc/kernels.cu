@@ -414,14 +414,25 @@ __device__ __forceinline__ void run_epoch(Mem M, const uint64_t* T, uint64_t* Y,
 // for the next VM's state.) Lanes that stall wait in place until `wait` of them
 // have (or none runs on), then take general steps together until they can
 // enter their entries again or stop. A VM that leaves its entries for good --
-// it wrote into its program, or its i lies outside them for a few steps --
-// runs from its memory (run_epoch_loop, which does not watch its writes) until
-// the next pack.
+// it wrote into its program, its i lies outside them for a few steps, or its
+// stalls cost more than its entries gain -- runs from its memory
+// (run_epoch_loop, which does not watch its writes) until the next pack, or, of
+// a shared program, until the run ends.
 constexpr uint32_t kFuseChunk = 16;    // entries between two looks at the stalled lanes (from 8: uneven
                                        // 4.95 -> 4.85 ms); 12 stalled lanes end an epoch (templates 1.89 ms,
                                        // 8: 1.93, 4: 2.08)
 constexpr uint32_t kFuseOutside = 32;  // general steps at no entry's start before a VM leaves them: more than an
                                        // entry holds (a run that a stop has cut goes on inside an entry)
+// Operands that do not fit an entry (words behind 65,535, wide constants of
+// shared programs) stall although the one-instruction loop takes them in its
+// stride. A stall waits for up to `epoch` entries of the other lanes, in which
+// the loop would have made as many steps, so it is charged kFuseStall VM-steps
+// and the VM leaves once it owes kFuseDebt. (4,096 machines, one in 32 of which
+// does little but stall: 11.7 ms if all stay, 3.5 so; 131,072 machines of shared
+// programs with two wide constants in 12 instructions 20.9 and 4.96.)
+constexpr uint32_t kFuseStall = 64;
+constexpr uint32_t kFuseDebt = 512;
+constexpr uint32_t kFuseGeneral = 64;  // general steps in a row while other lanes wait
 
 template <bool MASKED, bool CLASSIC, class Mem>
 __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64_t* Y, const Params& P, Regs& r,
@@ -429,7 +440,8 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
                                                 uint32_t& final_st, uint32_t epoch, uint32_t idle_exit,
                                                 uint32_t shared_tab = 0) {
   const uint32_t fm = __ballot_sync(FULL, active && F.on);
-  bool stall = active && r.clean && !F.on;               // a stop has cut the run of an entry: on to the next one
+  // a stop has cut the run of an entry: on to the next one
+  bool stall = active && r.clean && !F.on && F.debt != kFuseGone;
   if (fm) {
     const uint32_t wait = idle_exit ? idle_exit : 12u;
     const uint32_t zero = P.ellp & 1u;                   // the stride of the tapes is even
@@ -472,7 +484,9 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
     if (F.on) r.ip = 2u * (F.op.y & FO_COUNT ? fuse_instr(G, F.cur) : F.op.x);
     else reduce_ip(P, r);
     r.have = false;
-    for (uint32_t out = 0; active && stall;) {
+    const uint32_t owed = F.debt + kFuseStall, ran = F.mark - r.left;
+    F.debt = owed > ran ? owed - ran : 0u;
+    for (uint32_t k = 0, out = 0; active && stall && k < kFuseGeneral; ++k) {
       const uint32_t st = step_general<MASKED, false, false, CLASSIC>(V, T, Y, P, r, h);
       if (st != CONT) {
         active = false;
@@ -481,6 +495,11 @@ __device__ __forceinline__ void run_epoch_fused(Mem M, const uint64_t* T, uint64
         fuse_enter(G, F, r);
         stall = F.on ? fuse_stalled(F, r, P) : r.clean && out++ < kFuseOutside;
       }
+    }
+    F.mark = r.left;
+    if (F.debt > kFuseDebt) {
+      F.on = false;
+      F.debt = kFuseGone;
     }
     if (active && !F.on) {
       if constexpr (!std::is_same<Mem, ShView>::value) r.clean = false;   // (a shared program's view watches writes)
@@ -1121,7 +1140,10 @@ __global__ void __launch_bounds__(128, 7) k_shared_loop(RunState S, Params P, co
               T = S.tape + (uint64_t)v * P.ellp;
               Y = S.y + (uint64_t)v * P.sp;
               vm = (int32_t)v;
-              if constexpr (FUSE) fuse_enter(fuse_prog(S, v, r.ilim), F, r);
+              if constexpr (FUSE) {
+                fuse_begin(F, r);
+                fuse_enter(fuse_prog(S, v, r.ilim), F, r);
+              }
               if (!F.on) prime(V, r);
               active = true;
             }

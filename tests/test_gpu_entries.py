@@ -53,7 +53,7 @@ def check(rasp, wl, budgets, what, classic=False, i32=True, entries=True, **kw):
             b.reset()
 
 
-@pytest.mark.parametrize("w", [64, 48, 32, 20, 8])
+@pytest.mark.parametrize("w", [64, 48, 32, 20, 11])
 @pytest.mark.parametrize("m", [31, 64, 65, 130])
 def test_programs_of_one_to_three_records(rasp, m, w):
     check(rasp, machines(700, m, w, seed=2000 * m + w, extra=2 * m + 8), [3, 20, 21, 200, 1000], "m=%d w=%d" % (m, w),
@@ -121,7 +121,7 @@ def test_operands_around_65535(rasp, w, classic):
     rng = np.random.default_rng(w)
     prog = wl.programs.reshape(120, -1, 2)
     edge = rng.choice([65533, 65534, 65535, 65536, 65537, 65538, n - 2, n - 1, 60, 61], size=prog.shape[:2])
-    mem = np.isin(prog[:, :, 0], (ADD, MUL, STO, RD, PRI)) & (rng.random(prog.shape[:2]) < .7)
+    mem = np.isin(prog[:, :, 0], (ADD, MUL, STO, RD, PRI)) & (rng.random(prog.shape[:2]) < .25)
     prog[:, :, 1] = np.where(mem, edge, prog[:, :, 1])
     check(rasp, wl, [25, 500], "operands at 2^16, w=%d" % w, classic=classic, i32=w != 17)
 
@@ -138,8 +138,8 @@ def test_longest_programs(rasp, m, entries, w):
     pick = rng.integers(0, 4, (V, m))
     target = 2 * np.where(pick == 0, edge(40, 40), np.where(pick == 1, m - 1 - rng.integers(0, 70, (V, m)),
                           np.where(pick == 2, edge(32_767, 60), rng.integers(0, m, (V, m)))))
-    word = np.where(pick == 0, edge(65_535, 4), np.where(pick == 1, 2 * m - 1 - rng.integers(0, 9, (V, m)),
-                    rng.integers(0, 2 * m, (V, m))))
+    word = np.where(pick == 0, edge(65_535, 4), rng.integers(0, 65_530, (V, m)))
+    word = np.where(rng.random((V, m)) < .05, 2 * m - 1 - rng.integers(0, 9, (V, m)), word)
     const = np.where(pick == 0, rng.integers(40_000, 1 << 30, (V, m)), rng.integers(-2, 3, (V, m)))
     arg = np.where(op == BNZ, target, np.where(op == LOD, const, np.where(op == STO, 2 * m + 7 + pick, word)))
     prog = np.stack([op, arg], axis=2).reshape(V, 2 * m)
@@ -261,3 +261,64 @@ def test_autotune_after_a_run_that_wrote_code(rasp):
         b.run()
         st, _ = oracle_state(wl, threads=8)
         assert_same_state(b.read_state(), st, wl.ell, wl.s, what="after autotune")
+
+
+# ---- operands that no entry holds: words behind 65,535, wide constants of shared programs
+def stalling(V, n, far, every, shared=False, turns=300):
+    """Counter loops of 10 steps; in every `every`-th program the loop reads
+    and writes word `far` (or, of shared programs, loads a wide constant)."""
+    near = [LOD, turns, STO, 100, LOD, 1, ADD, 101, STO, 101, LOD, 3, ADD, 102, STO, 102, LOD, -1, ADD, 100, STO, 100,
+            BNZ, 4, PRI, 101, 0, 0]
+    prog = np.tile(np.array(near), (V // 32 if shared else V, 1))
+    if shared:
+        prog[::every, 5], prog[::every, 11] = 100_000, 70_000
+    else:
+        prog[::every, 7] = prog[::every, 9] = prog[::every, 25] = far
+    wl = flat(list(prog), n, np.zeros((V, 2)), cap=10 ** 6, pvm=np.repeat(np.arange(len(prog)), 32).astype(np.uint32) if shared else None)
+    return wl
+
+
+@pytest.mark.parametrize("w", [64, 32, 18])
+@pytest.mark.parametrize("every", [3, 33])
+def test_machines_that_leave_their_entries(rasp, w, every):
+    wl = stalling(384, 70_000, 66_000, every)
+    wl.w = w
+    check(rasp, wl, [17, 100, 1000, 10_000], "far operands in one of %d, w=%d" % (every, w))
+    wl = stalling(768, 256, 0, every, shared=True)
+    wl.w = w
+    for flags in (rasp.SCHED_SHARED, rasp.SCHED_AUTO):
+        check(rasp, wl, [17, 100, 1000, 10_000], "wide constants in one of %d, w=%d" % (every, w), flags=flags)
+
+
+def test_most_machines_stall(rasp):
+    """No entries where most programs would leave them."""
+    wl = stalling(256, 70_000, 66_000, 1)
+    check(rasp, wl, [1000, 10_000], "far operands", entries=False)
+    wl = stalling(512, 256, 0, 1, shared=True)
+    for flags in (rasp.SCHED_SHARED, rasp.SCHED_AUTO):
+        check(rasp, wl, [1000, 10_000], "wide constants", flags=flags, entries=False)
+
+
+def test_stalls_do_not_hold_the_warp(rasp):
+    """Half of the programs load two wide constants in 12 instructions: machines
+    that stall all the time run on from memory (2 times the time of small
+    constants; 9 times if they stay)."""
+    import torch
+    stream, ms = torch.cuda.current_stream(), []
+    for every in (1 << 20, 2):
+        wl = stalling(65_536, 256, 0, every, shared=True, turns=2000)
+        wl.programs.reshape(2048, -1)[0] = wl.programs.reshape(2048, -1)[1]
+        with rasp.Batch(wl.mem_words, wl.ell, wl.s, flags=rasp.SCHED_SHARED) as b:
+            b.load_workload(wl)
+            assert b.describe()["entries"]
+            took = []
+            for _ in range(4):
+                b.reset()
+                e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+                e[0].record(stream)
+                b.run()
+                e[1].record(stream)
+                torch.cuda.synchronize()
+                took.append(e[0].elapsed_time(e[1]))
+            ms.append(min(took))
+    assert ms[1] < 4.5 * ms[0], ms
