@@ -136,6 +136,8 @@ struct rasp_batch {
   uint32_t* d_pvids = nullptr;
   uint32_t num_programs = 0;
   uint32_t max_plen = 0;
+  uint4* fuse_at = nullptr;    // the place of the programs' fused entries (NULL: they get none); S.fops once decoded
+  bool fuse_own = false;       // the entries may read program words as data (owns_code at the load)
   bool dirty_valid = false;    // codedirty is up to date for the VMs of the schedules that keep it
   bool ran_untracked = false;  // since the last pack a schedule ran that does not keep codedirty
   bool code_lazy = false;      // slabs of VMs with codedirty = 0 lack their program words (lazy pack)
@@ -714,14 +716,61 @@ bool poor_entries(const W* words, const uint64_t* offsets, uint64_t num_programs
 // the pack) in the part of the program area that the programs leave free: behind
 // the 8-byte words, or behind where they would be widened to -- from the start
 // when nothing widens them. NULL where there is no room (programs that fill
-// more than half of the memories), where no kernel would run from them, or
-// where a program has more instructions than an entry can name.
+// more than half of the memories), where no kernel of the batch's options runs
+// from them, or where a program has more instructions than an entry can name.
 uint4* place_fused(const rasp_batch* b, uint64_t total, bool keep32) {
   if (!total || !runs_entries(variant_of(b)) || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
   const uint64_t lo = keep32 && owns_code(b) ? 0 : 8ull * total;
   const uint64_t end = keep32 ? 4ull * kept_words_at(b) : 8ull * b->mem_words;
   if (lo + 8ull * total > end || 8ull * total > (b->narrow ? 4ull : 8ull) * b->mem_words) return nullptr;
   return reinterpret_cast<uint4*>(reinterpret_cast<char*>(b->d_prog) + lo);
+}
+
+// Whether a run of the current plan takes fused entries (a plan not made yet is
+// that of a pool's request).
+bool uses_entries(const rasp_batch* b) {
+  if (!b->fuse_at) return false;
+  bool uses = !b->planned;
+  for (const Group& g : b->groups)
+    uses = uses || g.sched == RASP_SCHED_PERSIST_GL || (g.sched == RASP_SCHED_SHARED && shared_fuses(b->max_plen));
+  return uses;
+}
+
+// The smallest memory that runs each program, for the decoder: S.n where VM v
+// runs program v, else into d_ids2. pvm: the program of each VM (NULL: read back).
+cudaError_t program_bounds(rasp_batch* b, const uint32_t* pvm, cudaStream_t st) {
+  if (!b->shared_programs) return cudaSuccess;
+  std::vector<uint32_t> least(b->num_programs, 1u << 31), read;
+  cudaError_t e = cudaSuccess;
+  if (!pvm) {
+    read.resize(b->V);
+    e = cudaMemcpyAsync(read.data(), b->d_progvm, 4ull * b->V, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    pvm = read.data();
+  }
+  for (uint32_t v = 0; v < b->V; ++v) least[pvm[v]] = std::min(least[pvm[v]], b->h_n[v]);
+  e = cudaMemcpyAsync(b->d_ids2, least.data(), 4ull * b->num_programs, cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
+// Decode the loaded programs into their fused entries (after program_bounds).
+// tmp: 16 bytes of scratch per instruction (NULL: none, as after the pack).
+cudaError_t decode_entries(rasp_batch* b, uint4* tmp, cudaStream_t st) {
+  const cudaError_t e = launch_fuse(b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_ids2 : b->S.n,
+                                    b->num_programs, b->max_plen, b->prog_words / 2u, b->wmask, variant_of(b).classic,
+                                    b->fuse_own, b->narrow, tmp, b->fuse_at, const_cast<uint4*>(b->S.frec), st);
+  if (e == cudaSuccess) b->S.fops = b->fuse_at;
+  return e;
+}
+
+// The plan has come to run from entries after a load that did not make them
+// (eagerly, outside any captured graph).
+cudaError_t late_entries(rasp_batch* b, cudaStream_t st) {
+  if (b->S.fops || !b->fuse_at) return cudaSuccess;
+  drop_graphs(b);                              // captured runs hold the old launch arguments
+  const cudaError_t e = program_bounds(b, nullptr, st);
+  return e == cudaSuccess ? decode_entries(b, nullptr, st) : e;
 }
 
 }  // namespace
@@ -814,33 +863,24 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
     CK(cudaStreamSynchronize(st));
   }
   CK(cudaStreamSynchronize(st));   // the caller's buffers are read before the call returns
-  // fused entries: their place, and the smallest memory that runs each program
-  const uint32_t* bound = b->S.n;
-  const bool from_memory = total && (word_size == 8 ? poor_entries((const int64_t*)words, offsets, num_programs, b->wmask, owns_code(b))
-                                                    : poor_entries((const int32_t*)words, offsets, num_programs, b->wmask, owns_code(b)));
-  b->S.fops = from_memory ? nullptr : place_fused(b, total, keep32);
+  const bool from_memory =
+      total && (word_size == 8 ? poor_entries((const int64_t*)words, offsets, num_programs, b->wmask, owns_code(b))
+                               : poor_entries((const int32_t*)words, offsets, num_programs, b->wmask, owns_code(b)));
+  b->fuse_at = from_memory ? nullptr : place_fused(b, total, keep32);
+  b->fuse_own = owns_code(b);
+  b->S.fops = nullptr;
   b->S.frec = (const uint4*)(b->base + b->L.off_frec);
   b->S.prog_off = b->d_progoff;
   b->S.prog_of_vm = b->shared_programs ? b->d_progvm : nullptr;
-  if (b->S.fops && prog_of_vm) {
-    std::vector<uint32_t> least(num_programs, 1u << 31);
-    for (uint32_t v = 0; v < b->V; ++v) least[prog_of_vm[v]] = std::min(least[prog_of_vm[v]], b->h_n[v]);
-    CK(cudaMemcpyAsync(b->d_ids2, least.data(), 4 * num_programs, cudaMemcpyHostToDevice, st));
-    CK(cudaStreamSynchronize(st));
-    bound = b->d_ids2;
-  }
-  if (!same_args || b->S.fops != fops_before) drop_graphs(b);   // captured runs hold the old launch arguments
+  if (uses_entries(b)) CK(program_bounds(b, prog_of_vm, st));
   // widening, like the pack, is left queued on the stream: it may have to
   // wait for SMs that another batch's run holds, and the host need not
   b->prog32 = keep32 && total ? staged : nullptr;
   b->prog_words = total;
   b->prog64_valid = !b->prog32;
   if (word_size == 4 && total && !keep32) CK(launch_widen(staged, b->d_prog, total, st));
-  if (b->S.fops)
-    CK(launch_fuse(b->d_prog, b->prog32, b->d_progoff, bound, b->num_programs, b->max_plen, total / 2u,
-                   b->wmask, variant_of(b).classic,
-                   owns_code(b), b->narrow, reinterpret_cast<uint4*>(b->S.mem), const_cast<uint4*>(b->S.fops),
-                   const_cast<uint4*>(b->S.frec), st));
+  if (uses_entries(b)) CK(decode_entries(b, reinterpret_cast<uint4*>(b->S.mem), st));
+  if (!same_args || b->S.fops != fops_before) drop_graphs(b);   // captured runs hold the old launch arguments
   CK(fill_bytes(b->d_hist, 0, 8 * 10, st));
   b->code_lazy = pack_lazy(b);
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,
@@ -1028,6 +1068,7 @@ int rasp_run(rasp_batch* b, uint64_t max_steps) {
     const int rc = replan(b);
     if (rc) return rc;
   }
+  if (uses_entries(b)) CK(late_entries(b, b->stream));
   // 8-byte program words for the kernels that read them, eagerly (outside any captured graph)
   if (b->code_lazy || (b->cfg.flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED) CK(ensure_prog64(b, b->stream));
   CK(settle_dirty(b, b->stream));
@@ -1304,6 +1345,7 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
   if (reps == 0) reps = 1;
   CK(apply_uhead_reset(b, b->stream));
   if (b->shared_programs || b->code_lazy) CK(ensure_prog64(b, b->stream));   // the shared-program trials
+  CK(late_entries(b, b->stream));              // the HBM-slab trials run from them
   int rc = check_device_error(b);
   if (rc) return rc;
   cudaStream_t st = b->stream;

@@ -52,7 +52,7 @@ cudaError_t launch_pack(const DevState& S, const uint64_t* prog, const int32_t* 
 // offset in `out`, and their records. bound[p]: the smallest n among the VMs of
 // program p; own: the VMs' memories hold the program words; two: the loop that
 // runs them takes a second store (4-byte words); tmp: scratch of
-// 16 bytes per instruction.
+// 16 bytes per instruction (NULL: an entry for every instruction).
 cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint64_t* prog_off, const uint32_t* bound,
                         uint32_t num_programs, uint32_t max_plen, uint64_t instructions, uint64_t wmask,
                         bool classic, bool own, bool two, uint4* tmp, uint4* out,
@@ -80,6 +80,11 @@ cudaError_t launch_plain(const StepVariant& var, const DevState& S, const Params
 // The run kernels of this variant take fused entries (on the HBM-slab and the
 // shared-program schedule, and in the pools).
 inline bool runs_entries(const StepVariant& v) { return !v.checked && !v.hist && !v.vote && !v.block; }
+
+// The shared-program schedule holds the entries behind the program, where they
+// take at most as much again; where that would leave an SM fewer than two CTAs,
+// the programs run one instruction at a time.
+inline bool shared_fuses(uint32_t max_plen) { return 16ull * ((max_plen + 1u) & ~1u) <= 96u * 1024u; }
 
 // What a persistent launch over `count` VMs is: the resident CTAs of the kernel
 // that runs (with fused entries fewer fit an SM), at most as many as the VMs

@@ -1496,7 +1496,7 @@ cudaError_t launch_fuse(const uint64_t* prog, const int32_t* prog32, const uint6
   // templates 24 against 120 us, 16,384 136 and 124, 32,768 268 and 132; 16,384
   // uneven programs 114 against 903 us. The line is where the chain costs as
   // much as the work saved. (512: no chain of milliseconds for one program.)
-  if (max_plen / 2u > 512u || instructions <= 24000ull * (max_plen / 2u)) {
+  if (!tmp || max_plen / 2u > 512u || instructions <= 24000ull * (max_plen / 2u)) {
     const uint32_t x = std::min(num_programs, (uint32_t)num_sms() * 16u);
     const uint32_t rows = (max_plen + 511u) / 512u;        // four records per block
     const dim3 g(x, std::min(std::max(rows, 1u), 64u));
@@ -1536,10 +1536,8 @@ cudaError_t launch_shared(const StepVariant& var, const RunState& S, const Param
                           uint32_t num_programs, uint32_t max_plen, uint32_t epoch, cudaStream_t stream) {
   if (!num_programs) return cudaSuccess;
   size_t smem = (size_t)((max_plen + 1u) & ~1u) * 8u;
-  // the entries take at most as much again; where that would leave an SM fewer
-  // than two CTAs, the programs run one instruction at a time
   StepVariant v = var;
-  v.fuse = S.fops != nullptr && !v.checked && !v.hist && !v.block && 2u * smem <= 96u * 1024u;
+  v.fuse = S.fops != nullptr && runs_entries(v) && shared_fuses(max_plen);
   if (v.fuse) smem *= 2u;
   SharedFn fn = pick_shared(v);
   if (smem > 48u * 1024u) {

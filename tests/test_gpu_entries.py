@@ -322,3 +322,35 @@ def test_stalls_do_not_hold_the_warp(rasp):
                 took.append(e[0].elapsed_time(e[1]))
             ms.append(min(took))
     assert ms[1] < 4.5 * ms[0], ms
+
+
+@pytest.mark.parametrize("i32", [False, True])
+@pytest.mark.parametrize("sched", [0x10, 0x20], ids=["plain", "staged"])
+def test_entries_only_where_a_plan_runs_from_them(rasp, sched, i32):
+    """The plain and SMEM-staged schedules load without decoding; a plan that
+    moves to the HBM-slab schedule (pinned or autotuned, also midway, under a
+    graph, with programs shared) decodes before it runs."""
+    for shared in (0, 9):
+        wl = machines(600, 40, 64, seed=170 + shared, extra=100, shared=shared)
+        part, full = (oracle_state(wl, budget=t, threads=8)[0] for t in (33, 1000))
+        for how in ("pinned", "midway", "autotuned"):
+            with rasp.Batch(wl.mem_words, wl.ell, wl.s, flags=sched | rasp.CUDA_GRAPH) as b:
+                load = rasp.rasp_load_programs_i32 if i32 else rasp.rasp_load_programs
+                load(b.h, wl.programs, wl.prog_off, wl.prog_of_vm)
+                b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+                assert not b.describe()["entries"]
+                if how != "pinned":
+                    b.run(33)
+                    assert_same_state(b.read_state(), part, wl.ell, wl.s, what=how)
+                    assert not b.describe()["entries"]
+                if how == "autotuned":
+                    b.autotune(max_steps=1000, reps=1)
+                    assert b.describe()["entries"]
+                else:
+                    for k in b.describe()["buckets"]:
+                        b.plan_bucket(k["index"], rasp.SCHED_PERSIST_GL)
+                for _ in range(2):
+                    b.run(1000)
+                    assert b.describe()["entries"]
+                    assert_same_state(b.read_state(), full, wl.ell, wl.s, what=how)
+                    b.reset()
