@@ -119,13 +119,17 @@ typedef struct rasp_config {
     uint32_t epoch;      /* steps (fused entries, where programs have them)
                             between warp scheduling points; 0 = default       */
     uint32_t warps_per_cta; /* persistent kernels: warps per CTA (SMEM-staged
-                            up to 8, HBM-slab up to 4); 0 = default           */
+                            up to 8, HBM-slab up to 4); 0 = default (HBM-slab:
+                            4, and one where few VMs spread over the GPU)      */
     uint32_t refill_min; /* persistent kernels: idle lanes that trigger a
-                            refill (SMEM-staged), or stopped lanes that end
-                            an epoch early (HBM-slab); 0 = default            */
+                            refill (SMEM-staged), or lanes that have stopped
+                            (with fused entries: or wait for a step that
+                            no entry holds) and end an epoch early (HBM-slab);
+                            0 = default                                       */
     uint32_t ctas_per_sm;/* persistent kernels: resident CTAs per SM (fewer
                             resident VMs keep their memory in L1/L2);
-                            0 = as many as fit                                */
+                            0 = as many as fit (and where few VMs spread,
+                            up to 16 CTAs of one warp)                        */
     uint32_t reserved;   /* must be 0                                         */
     void*    stream;     /* cudaStream_t for all work of the batch; NULL = the
                             legacy default stream                              */

@@ -304,6 +304,7 @@ void plan_buckets(rasp_batch* b) {
     } else {
       sh.staged = false;
       sh.warps = 4;
+      sh.spread = !cfg_warps && !cfg_ctas;
       sh.refill_min = 1;
       sh.epoch = cfg_epoch ? cfg_epoch : 128u;
       sh.idle_exit = std::min<uint32_t>(b->cfg.refill_min, 32u);   // epoch loop: end an epoch after this many stops
@@ -376,7 +377,7 @@ void build_groups(rasp_batch* b) {
     const PersistShape& gs = b->groups.empty() ? k.shape : b->groups.back().shape;
     const bool same_shape = gs.warps == k.shape.warps && gs.epoch == k.shape.epoch && gs.grid == k.shape.grid &&
                             gs.ctas_per_sm == k.shape.ctas_per_sm && gs.idle_exit == k.shape.idle_exit &&
-                            gs.block == k.shape.block;
+                            gs.block == k.shape.block && gs.spread == k.shape.spread;
     if (!b->groups.empty() && k.sched == RASP_SCHED_PERSIST_GL && b->groups.back().sched == RASP_SCHED_PERSIST_GL &&
         same_shape && b->groups.back().first + b->groups.back().count == k.first) {
       b->groups.back().count += k.count;
@@ -1379,9 +1380,9 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
   // a time (fastest when a few thousand short runs leave the loop often).
   struct Cand { const char* name; uint32_t sched, epoch, warps, ctas; bool block; };
   static const Cand cands[] = {
-      {"persist_gl e128 w4", RASP_SCHED_PERSIST_GL, 128, 4, 0, false},
-      {"persist_gl e64 w4", RASP_SCHED_PERSIST_GL, 64, 4, 0, false},
-      {"persist_gl e256 w4", RASP_SCHED_PERSIST_GL, 256, 4, 0, false},
+      {"persist_gl e128 w4", RASP_SCHED_PERSIST_GL, 128, 0, 0, false},   // (the default 4 warps; few VMs may spread)
+      {"persist_gl e64 w4", RASP_SCHED_PERSIST_GL, 64, 0, 0, false},
+      {"persist_gl e256 w4", RASP_SCHED_PERSIST_GL, 256, 0, 0, false},
       {"persist_gl e128 w2", RASP_SCHED_PERSIST_GL, 128, 2, 0, false},
       {"persist_gl e128 w4 c3", RASP_SCHED_PERSIST_GL, 128, 4, 3, false},
       {"persist_gl e128 w4 c5", RASP_SCHED_PERSIST_GL, 128, 4, 5, false},

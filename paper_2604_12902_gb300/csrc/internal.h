@@ -37,6 +37,7 @@ struct PersistShape {
   uint32_t grid;        // CTAs
   uint32_t ctas_per_sm; // resident CTAs per SM (occupancy)
   uint32_t fuse_ctas;   // HBM-slab: the same for programs with fused entries
+  bool spread;          // HBM-slab: few VMs may run on one-warp CTAs (no launch setting asks otherwise)
   size_t smem;          // dynamic shared memory per CTA
 };
 
@@ -88,7 +89,8 @@ inline bool shared_fuses(uint32_t max_plen) { return 16ull * ((max_plen + 1u) & 
 
 // What a persistent launch over `count` VMs is: the resident CTAs of the kernel
 // that runs (with fused entries fewer fit an SM), at most as many as the VMs
-// fill; few VMs in the HBM-slab form spread over one-warp CTAs. dense: a
+// fill; few VMs in the HBM-slab form spread over one-warp CTAs unless warps or
+// CTAs were set. dense: a
 // compacted queue, of at most `count` VMs.
 struct PersistLaunch {
   uint32_t grid, warps, lanes;   // CTAs, warps per CTA, lanes of a warp that take VMs

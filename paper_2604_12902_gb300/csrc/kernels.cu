@@ -1625,7 +1625,7 @@ PersistLaunch persist_launch(const StepVariant& var, bool entries, uint32_t coun
   const uint32_t warps_needed = (count + 31u) / 32u;   // of a dense queue, count is an upper bound
   const uint32_t max_useful = (warps_needed + sh.warps - 1u) / sh.warps;
   const uint32_t spread = 8u * (uint32_t)num_sms();
-  if (!sh.staged && !dense && warps_needed < spread && resident * sh.warps >= 2u * spread) {
+  if (sh.spread && !dense && warps_needed < spread && resident * sh.warps >= 2u * spread) {
     // Few VMs (under 38,912 on 152 SMs): 8 warps per SM, each with as few lanes
     // as that takes, and four where that would be five to eight: the lanes of a
     // warp wait for one another's misses and general steps. Run kernel, 32

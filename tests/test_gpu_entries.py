@@ -354,3 +354,25 @@ def test_entries_only_where_a_plan_runs_from_them(rasp, sched, i32):
                     assert b.describe()["entries"]
                     assert_same_state(b.read_state(), full, wl.ell, wl.s, what=how)
                     b.reset()
+
+
+def test_launch_settings_hold_for_few_machines(rasp):
+    """Few VMs spread over one-warp CTAs only where neither warps_per_cta nor
+    ctas_per_sm is set, in the configuration or for a bucket."""
+    wl = W.template_programs(num_vms=2048, seed=5)
+    st, _ = oracle_state(wl, threads=8)
+    for kw, want in (({}, None), (dict(warps_per_cta=4), (16, 4, 32)), (dict(warps_per_cta=2), (32, 2, 32)),
+                     (dict(ctas_per_sm=5), (16, 4, 32))):
+        for pin in (False, True):
+            with rasp.Batch(wl.mem_words, wl.ell, wl.s, **({} if pin else kw)) as b:
+                b.load_workload(wl)
+                if pin:
+                    b.plan_bucket(b.describe()["buckets"][0]["index"], rasp.SCHED_PERSIST_GL, **kw)
+                got = b.describe()["launches"][0]
+                got = got["grid"], got["warps_per_cta"], got["lanes_per_warp"]
+                if want is None:
+                    assert got[1] == 1 and got[2] < 32 and got[0] * got[2] >= 2048, got
+                else:
+                    assert got == want
+                b.run()
+                assert_same_state(b.read_state(), st, wl.ell, wl.s, what=str(kw))
