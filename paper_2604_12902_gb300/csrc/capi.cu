@@ -137,6 +137,7 @@ struct rasp_batch {
   uint32_t num_programs = 0;
   uint32_t max_plen = 0;
   uint4* fuse_at = nullptr;    // the place of the programs' fused entries (NULL: they get none); S.fops once decoded
+  bool self_writing = false;   // most of the loaded programs write into themselves (look_at)
   bool fuse_own = false;       // the entries may read program words as data (owns_code at the load)
   bool dirty_valid = false;    // codedirty is up to date for the VMs of the schedules that keep it
   bool ran_untracked = false;  // since the last pack a schedule ran that does not keep codedirty
@@ -258,6 +259,7 @@ StepVariant variant_of(const rasp_batch* b) {
   v.classic = (b->cfg.flags & RASP_ISA_CLASSIC) != 0;
   v.block = (b->cfg.flags & RASP_STEP_BLOCK) != 0;
   v.narrow = b->narrow;
+  v.self_writing = b->self_writing;
   return v;
 }
 
@@ -683,33 +685,38 @@ bool owns_code(const rasp_batch* b) {
   return !b->shared_programs && (b->cfg.flags & RASP_SCHED_MASK) != RASP_SCHED_SHARED;
 }
 
-// Whether most of the programs are better run one instruction at a time, by a
-// look at up to 64 of them: an eighth of their instructions or more write into
-// the program (their VMs would leave the entries at once: 65,536 random programs
-// with n = 256 212 us a run without entries, 275 with), or do not fit an entry
-// though the one-instruction loop takes them in its stride -- operands behind
-// word 65,535, and constants beyond 16 bits where the entries may not read the
-// program words (4,096 machines in a loop of 10 steps with two such operands,
-// n = 70,000: 2.37 ms a run, from entries that they leave 2.52, and 4.4 before
-// few machines were spread over many warps; 131,072 with two wide constants in
-// 12 instructions 8.86 and 10.4 ms).
+// A look at up to 64 of the programs. writing: an eighth or more of the
+// instructions of most of them write into the program. unfit: that, or operands
+// that no entry holds though the one-instruction loop takes them in its stride
+// (behind word 65,535, and constants beyond 16 bits where the entries may not
+// read the program words). Most machines of such programs would leave their
+// entries, and the kernel without them is faster: 65,536 random programs with
+// n = 256 212 us a run, with entries 275; 4,096 machines in a loop of 10 steps
+// with two such operands, n = 70,000: 2.37 and 2.52 ms (4.4 before few machines
+// were spread over many warps); 131,072 with two wide constants in 12
+// instructions 8.86 and 10.4 ms.
+struct ProgramLook {
+  bool unfit, writing;
+};
 template <class W>
-bool poor_entries(const W* words, const uint64_t* offsets, uint64_t num_programs, uint64_t wmask, bool own) {
+ProgramLook look_at(const W* words, const uint64_t* offsets, uint64_t num_programs, uint64_t wmask, bool own) {
   const uint64_t looks = std::min<uint64_t>(num_programs, 64);
-  uint64_t poor = 0;
+  uint64_t unfit = 0, writing = 0;
   for (uint64_t q = 0; q < looks; ++q) {
     const uint64_t p = q * (num_programs / looks | 1ull) % num_programs;   // an odd stride: batches may be periodic
     const uint64_t len = offsets[p + 1] - offsets[p], seen = std::min<uint64_t>(len, 1024);
     const W* w = words + offsets[p];
-    uint64_t unfit = 0;
+    uint64_t writes = 0, other = 0;
     for (uint64_t k = 0; k + 1 < seen; k += 2) {
       const uint64_t o = (uint64_t)(int64_t)w[k] & wmask, j = (uint64_t)(int64_t)w[k + 1] & wmask;
-      if (o == 1) unfit += !own && ((uint64_t)(int64_t)(int16_t)(uint16_t)j & wmask) != j ? 1 : 0;
-      else if (o != 5 && o - 1 < 7) unfit += ((o == 4 || o == 6) && j < len) || (j > 0xFFFF) ? 1 : 0;
+      if (o == 1) other += !own && ((uint64_t)(int64_t)(int16_t)(uint16_t)j & wmask) != j ? 1 : 0;
+      else if ((o == 4 || o == 6) && j < len) ++writes;
+      else if (o != 5 && o - 1 < 7) other += j > 0xFFFF ? 1 : 0;
     }
-    poor += unfit && 16 * unfit >= seen ? 1 : 0;
+    writing += writes && 16 * writes >= seen ? 1 : 0;
+    unfit += writes + other && 16 * (writes + other) >= seen ? 1 : 0;
   }
-  return 2 * poor > looks;
+  return {2 * unfit > looks, 2 * writing > looks};
 }
 
 // The place of the fused entries (at most 16 bytes per instruction, 8 per
@@ -841,6 +848,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
     cudaStreamSynchronize(st);   // the caller's buffers are read before the call returns
     return bad;
   }
+  const bool writing_before = b->self_writing;
   const bool same_args = b->shared_programs == (prog_of_vm != nullptr) && b->max_plen == max_plen &&
                          b->num_programs == (uint32_t)num_programs;
   const uint4* fops_before = b->S.fops;
@@ -864,11 +872,13 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
     CK(cudaStreamSynchronize(st));
   }
   CK(cudaStreamSynchronize(st));   // the caller's buffers are read before the call returns
-  const bool from_memory =
-      total && (word_size == 8 ? poor_entries((const int64_t*)words, offsets, num_programs, b->wmask, owns_code(b))
-                               : poor_entries((const int32_t*)words, offsets, num_programs, b->wmask, owns_code(b)));
-  b->fuse_at = from_memory ? nullptr : place_fused(b, total, keep32);
+  ProgramLook look{false, false};
+  if (total)
+    look = word_size == 8 ? look_at((const int64_t*)words, offsets, num_programs, b->wmask, owns_code(b))
+                          : look_at((const int32_t*)words, offsets, num_programs, b->wmask, owns_code(b));
+  b->fuse_at = look.unfit ? nullptr : place_fused(b, total, keep32);
   b->fuse_own = owns_code(b);
+  b->self_writing = look.writing;
   b->S.fops = nullptr;
   b->S.frec = (const uint4*)(b->base + b->L.off_frec);
   b->S.prog_off = b->d_progoff;
@@ -881,7 +891,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   b->prog64_valid = !b->prog32;
   if (word_size == 4 && total && !keep32) CK(launch_widen(staged, b->d_prog, total, st));
   if (uses_entries(b)) CK(decode_entries(b, reinterpret_cast<uint4*>(b->S.mem), st));
-  if (!same_args || b->S.fops != fops_before) drop_graphs(b);   // captured runs hold the old launch arguments
+  if (!same_args || b->S.fops != fops_before || b->self_writing != writing_before) drop_graphs(b);   // captured runs hold the old launch arguments
   CK(fill_bytes(b->d_hist, 0, 8 * 10, st));
   b->code_lazy = pack_lazy(b);
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,

@@ -22,6 +22,7 @@ struct StepVariant {
                  // shared-program schedule: one step at a time per lane instead of the epoch loop
   bool narrow;   // M in 4-byte words (w <= 32): plain and HBM-slab persistent schedules
   bool fuse;     // HBM-slab epoch loop: the programs have fused entries
+  bool self_writing; // most of the loaded programs write into themselves
 };
 
 // Persistent-kernel launch shape for one bucket of VMs.

@@ -1627,15 +1627,19 @@ PersistLaunch persist_launch(const StepVariant& var, bool entries, uint32_t coun
   const uint32_t spread = 8u * (uint32_t)num_sms();
   if (sh.spread && !dense && warps_needed < spread && resident * sh.warps >= 2u * spread) {
     // Few VMs (under 38,912 on 152 SMs): 8 warps per SM, each with as few lanes
-    // as that takes, and four where that would be five to eight: the lanes of a
-    // warp wait for one another's misses and general steps. Run kernel, 32
-    // lanes a warp -> this: 1,024 random programs 225 -> 128 us, 8,192 262 ->
-    // 178, 2,048 templates 143 -> 101, 16,384 153 -> 133, 32,768 193 -> 187,
-    // 32,768 search programs 8.2 -> 7.3 ms. With 16 warps per SM 2,048
-    // templates take 134 us and 16,384 181.
+    // as that takes: the lanes of a warp wait for one another's misses and
+    // general steps. Run kernel, 32 lanes a warp -> this: 1,024 random programs
+    // 225 -> 128 us, 2,048 templates 143 -> 101, 8,192 149 -> 109, 16,384 153 ->
+    // 133, 32,768 193 -> 187, 32,768 search programs 8.2 -> 7.3 ms. With 16
+    // warps per SM 2,048 templates take 134 us and 16,384 181.
+    // Where that would be five to eight lanes, programs that write into
+    // themselves take twice the warps of four (general steps at nearly every
+    // step: 8,192 random programs 287 -> 189 us, 7,300 286 -> 189, 9,700 266 ->
+    // 229); others lose by it (8,192 templates 109 -> 146 us, CHECKED 0.41 ->
+    // 0.54 ms, uneven 2.75 -> 2.89 ms).
     l.warps = 1u;
     l.lanes = (count + spread - 1u) / spread;
-    if (l.lanes > 4u && l.lanes <= 8u) l.lanes = 4u;
+    if (var.self_writing && l.lanes > 4u && l.lanes <= 8u) l.lanes = 4u;
     l.grid = (count + l.lanes - 1u) / l.lanes;
   } else if (l.grid > max_useful) {
     l.grid = max_useful;

@@ -376,3 +376,21 @@ def test_launch_settings_hold_for_few_machines(rasp):
                     assert got == want
                 b.run()
                 assert_same_state(b.read_state(), st, wl.ell, wl.s, what=str(kw))
+
+
+@pytest.mark.parametrize("V", [1, 33, 6100, 8192, 9800])
+def test_lanes_of_few_machines(rasp, V):
+    """One-warp CTAs of as many lanes as eight warps per SM take, at their
+    edges; programs that write into themselves run on four lanes in place of
+    five to eight."""
+    import torch
+    spread = 8 * torch.cuda.get_device_properties(0).multi_processor_count
+    lanes = -(-V // spread)
+    for wl, own in ((W.template_programs(num_vms=V, seed=6), False), (W.random_programs(num_vms=V, seed=6), True)):
+        st, _ = oracle_state(wl, threads=8)
+        with rasp.Batch(wl.mem_words, wl.ell, wl.s) as b:
+            b.load_workload(wl)
+            got, want = b.describe()["launches"][0], 4 if own and 4 < lanes <= 8 else lanes
+            assert (got["warps_per_cta"], got["lanes_per_warp"], got["grid"]) == (1, want, -(-V // want))
+            b.run()
+            assert_same_state(b.read_state(), st, wl.ell, wl.s, what="%s %d" % (wl.name, V))
