@@ -94,7 +94,9 @@ enum rasp_semantics {
                                           with the still-running VMs compacted
                                           between rounds; by default only
                                           batches larger than half of the
-                                          resident lanes do                    */
+                                          resident lanes do (larger than all
+                                          of them where most programs write
+                                          into themselves)                     */
 #define RASP_STEP_BLOCK        0x20000u /* HBM-slab persistent schedule: evaluate
                                           every step as one predicated block
                                           (the earlier form) instead of the

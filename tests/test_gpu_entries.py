@@ -394,3 +394,18 @@ def test_lanes_of_few_machines(rasp, V):
             assert (got["warps_per_cta"], got["lanes_per_warp"], got["grid"]) == (1, want, -(-V // want))
             b.run()
             assert_same_state(b.read_state(), st, wl.ell, wl.s, what="%s %d" % (wl.name, V))
+
+
+def test_budget_rounds_by_kind(rasp):
+    """Between half and all of the resident lanes, batches run in budget rounds
+    unless their programs write into themselves."""
+    import torch
+    V = 152 * 7 * 128 * 3 // 4 if torch.cuda.get_device_properties(0).multi_processor_count == 152 else 100_000
+    for wl, rounds in ((W.template_programs(num_vms=V, seed=8, cap=5000), True),
+                       (W.random_programs(num_vms=V, seed=8, cap=5000), False)):
+        st, _ = oracle_state(wl, threads=8)
+        with rasp.Batch(wl.mem_words, wl.ell, wl.s) as b:
+            b.load_workload(wl)
+            b.run()
+            assert (b.stats()["launches"] > 1) is rounds, wl.name
+            assert_same_state(b.read_state(), st, wl.ell, wl.s, what=wl.name)
