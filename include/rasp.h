@@ -421,7 +421,8 @@ int rasp_run_static(const rasp_static_run* run);
  * nothing on the device waits on the host without a limit. The pool's calls
  * are serialised by an internal mutex; errors are reported by
  * rasp_pool_last_error (thread-local). cfg's schedule, dispatch and stats
- * flags do not apply to pools. */
+ * flags do not apply to pools, whose requests hold M in 8-byte words at every
+ * w (as many bytes as rasp_batch_bytes gives for RASP_SCHED_SHARED). */
 typedef struct rasp_pool rasp_pool;
 
 enum rasp_request_state { RASP_REQ_QUEUED = 0, RASP_REQ_RUNNING = 1, RASP_REQ_DONE = 2 };

@@ -483,6 +483,14 @@ Params rasp::batch_params(const rasp_batch* b) {
 
 const uint32_t* rasp::batch_queue(const rasp_batch* b) { return b->d_ids; }
 
+uint64_t rasp::batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan) {
+  uint64_t mw = 0;
+  for (uint64_t v = 0; v < num_vms; ++v) mw += even(mem_words[v]);
+  mw += pad_words(num_vms);
+  return make_layout(num_vms, mw, even(cfg->in_cap), even(cfg->out_cap), narrow_layout(cfg, plan) ? 4u : 8u).total +
+         ALIGN;
+}
+
 extern "C" {
 
 const char* rasp_last_error(void) { return g_err.c_str(); }
@@ -493,11 +501,7 @@ int rasp_batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* m
   int rc = validate_config(cfg, num_vms, mem_words);
   if (rc) return rc;
   if (!out_bytes) return fail(RASP_EINVAL, "out_bytes is NULL");
-  uint64_t mw = 0;
-  for (uint64_t v = 0; v < num_vms; ++v) mw += even(mem_words[v]);
-  mw += pad_words(num_vms);
-  *out_bytes = make_layout(num_vms, mw, even(cfg->in_cap), even(cfg->out_cap), narrow_layout(cfg, true) ? 4u : 8u).total +
-               ALIGN;
+  *out_bytes = rasp::batch_bytes(cfg, num_vms, mem_words, true);
   return RASP_OK;
 }
 

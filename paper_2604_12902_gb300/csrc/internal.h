@@ -203,6 +203,9 @@ cudaError_t launch_widen(const int32_t* src, uint64_t* dst, uint64_t count, cuda
 int create_batch(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan,
                  rasp_batch** out);
 
+// The device memory of such a batch (rasp_batch_bytes; arguments checked).
+uint64_t batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan);
+
 // The state store and step parameters of a batch (for the serving pool).
 const RunState& batch_run_state(const rasp_batch* b);
 Params batch_params(const rasp_batch* b);

@@ -409,3 +409,15 @@ def test_budget_rounds_by_kind(rasp):
             b.run()
             assert (b.stats()["launches"] > 1) is rounds, wl.name
             assert_same_state(b.read_state(), st, wl.ell, wl.s, what=wl.name)
+
+
+@pytest.mark.parametrize("w", [32, 20])
+def test_pools_of_small_words(rasp, w):
+    """A pool's requests hold 8-byte words at every w: their size is asked for so."""
+    from paper_2604_12902_gb300 import serving
+    wl = machines(900, 40, w, seed=180 + w, extra=100)
+    st, _ = oracle_state(wl, threads=8)
+    with serving.Pool(1 << 26, wl.ell, wl.s, word_bits=w) as pool:
+        tickets = [pool.submit(wl) for _ in range(3)]
+        for t in tickets:
+            assert_same_state(pool.read(t), st, wl.ell, wl.s, what="pool, w = %d" % w)
