@@ -168,7 +168,11 @@ typedef struct rasp_stats {
     uint64_t launches;      /* kernel launches of the last rasp_run            */
 } rasp_stats;
 
-/* Bytes of device memory a batch needs (for sizing rasp_config.arena).
+/* Bytes of device memory a batch needs (for sizing rasp_config.arena). About
+ * 16 bytes per 128 words of M and 32 per VM of them are room for the records of
+ * entries (see rasp_load_programs) and between the slabs of the shared-program
+ * schedule: rasp_batch_create takes an arena, or device memory, that lacks only
+ * these, and such a batch runs without entries.
  * Same argument rules as rasp_batch_create. */
 int rasp_batch_bytes(const rasp_config* cfg, uint64_t num_vms,
                      const uint32_t* mem_words, uint64_t* out_bytes);

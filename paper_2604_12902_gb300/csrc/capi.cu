@@ -197,7 +197,8 @@ bool narrow_layout(const rasp_config* cfg, bool plan) {
   return plan && cfg->word_bits <= 32 && sched != RASP_SCHED_SHARED && sched != RASP_SCHED_PERSIST;
 }
 
-Layout make_layout(uint64_t V, uint64_t mem_words, uint32_t ellp, uint32_t sp, uint32_t word_bytes) {
+// entries: room for the records of fused entries (else off_frec is 0).
+Layout make_layout(uint64_t V, uint64_t mem_words, uint32_t ellp, uint32_t sp, uint32_t word_bytes, bool entries) {
   Layout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -232,7 +233,7 @@ Layout make_layout(uint64_t V, uint64_t mem_words, uint32_t ellp, uint32_t sp, u
   L.off_ids2 = take(4 * V);                             // compacted queue between budget rounds
   L.off_rcount = take(4 * kNumBuckets);                 // its length, per launch group
   L.off_topk = take(sizeof(TopCand) * (topk_blocks(V) + 1) * kMaxTopK);  // top-k candidates, result
-  L.off_frec = take(16 * fuse_records(mem_words, V));  // records of the fused entries
+  L.off_frec = entries ? take(16 * fuse_records(mem_words, V)) : 0;      // records of the fused entries
   L.total = o;
   return L;
 }
@@ -245,7 +246,8 @@ uint32_t even(uint32_t x) { return (x + 1u) & ~1u; }
 // the same L1 banks (32 cycles for such a load; k_shared_loop on 2^20 VMs
 // 1.2 ms, 0.81 ms so; after every fourth slab 0.84, every eighth 0.99). Whole
 // sectors: with 16 bytes the pack took 0.25 ms in place of 0.19. The room is
-// part of every batch, whose size does not depend on the schedule.
+// part of every batch, whose size does not depend on the schedule, unless it
+// has to do without (see create_batch).
 constexpr uint64_t kSlabGroup = 2, kGroupPad = 4;
 uint64_t pad_words(uint64_t num_vms) { return (num_vms - 1) / kSlabGroup * kGroupPad; }
 bool padded_slabs(const rasp_config* cfg) { return (cfg->flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED; }
@@ -483,11 +485,11 @@ Params rasp::batch_params(const rasp_batch* b) {
 
 const uint32_t* rasp::batch_queue(const rasp_batch* b) { return b->d_ids; }
 
-uint64_t rasp::batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan) {
+uint64_t rasp::batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan, bool room) {
   uint64_t mw = 0;
   for (uint64_t v = 0; v < num_vms; ++v) mw += even(mem_words[v]);
-  mw += pad_words(num_vms);
-  return make_layout(num_vms, mw, even(cfg->in_cap), even(cfg->out_cap), narrow_layout(cfg, plan) ? 4u : 8u).total +
+  if (room) mw += pad_words(num_vms);
+  return make_layout(num_vms, mw, even(cfg->in_cap), even(cfg->out_cap), narrow_layout(cfg, plan) ? 4u : 8u, room).total +
          ALIGN;
 }
 
@@ -501,7 +503,7 @@ int rasp_batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* m
   int rc = validate_config(cfg, num_vms, mem_words);
   if (rc) return rc;
   if (!out_bytes) return fail(RASP_EINVAL, "out_bytes is NULL");
-  *out_bytes = rasp::batch_bytes(cfg, num_vms, mem_words, true);
+  *out_bytes = rasp::batch_bytes(cfg, num_vms, mem_words, true, true);
   return RASP_OK;
 }
 
@@ -532,23 +534,31 @@ int rasp::create_batch(const rasp_config* cfg, uint64_t num_vms, const uint32_t*
   b->wmask = cfg->word_bits >= 64 ? ~0ull : ((1ull << cfg->word_bits) - 1ull);
   b->h_n.assign(mem_words, mem_words + num_vms);
   b->h_memoff.resize(num_vms);
-  uint64_t off = 0;
-  for (uint64_t v = 0; v < num_vms; ++v) {
-    if (v && v % kSlabGroup == 0 && padded_slabs(cfg)) off += kGroupPad;
-    b->h_memoff[v] = off;
-    off += even(mem_words[v]);
-  }
-  if (!padded_slabs(cfg)) off += pad_words(num_vms);
-  b->mem_words = off;
   b->narrow = narrow_layout(cfg, plan);
-  b->L = make_layout(num_vms, off, b->ellp, b->sp, b->narrow ? 4u : 8u);
+  // with the room for fused entries and between the slabs of the shared-program
+  // schedule; without it (and them) where the caller's arena or the device does
+  // not have it, so that a batch that fitted without entries still does
+  auto lay_out = [&](bool room) {
+    uint64_t off = 0;
+    for (uint64_t v = 0; v < num_vms; ++v) {
+      if (v && v % kSlabGroup == 0 && room && padded_slabs(cfg)) off += kGroupPad;
+      b->h_memoff[v] = off;
+      off += even(mem_words[v]);
+    }
+    if (room && !padded_slabs(cfg)) off += pad_words(num_vms);
+    b->mem_words = off;
+    b->L = make_layout(num_vms, off, b->ellp, b->sp, b->narrow ? 4u : 8u, room);
+  };
+  lay_out(true);
   if (cfg->arena) {
     const uintptr_t p = (uintptr_t)cfg->arena;
     const uintptr_t aligned = (p + ALIGN - 1) & ~(uintptr_t)(ALIGN - 1);
+    if (aligned - p + b->L.total > cfg->arena_bytes) lay_out(false);
     if (aligned - p + b->L.total > cfg->arena_bytes) {
+      const unsigned long long need = b->L.total + ALIGN;
       delete b;
       return fail(RASP_ENOMEM, "arena of %llu bytes is smaller than the %llu the batch needs",
-                  (unsigned long long)cfg->arena_bytes, (unsigned long long)(b->L.total + ALIGN));
+                  (unsigned long long)cfg->arena_bytes, need);
     }
     b->base = (char*)aligned;
     b->owns = false;
@@ -559,10 +569,16 @@ int rasp::create_batch(const rasp_config* cfg, uint64_t num_vms, const uint32_t*
       return fail(RASP_ENOMEM, "injected allocation failure (RASP_FAULT_INJECT=alloc)");
     }
     cudaError_t e = cudaMalloc(&p, b->L.total);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      lay_out(false);
+      e = cudaMalloc(&p, b->L.total);
+    }
     if (e != cudaSuccess) {
+      const unsigned long long total = b->L.total;
       cudaGetLastError();
       delete b;
-      return fail(RASP_ENOMEM, "cudaMalloc(%llu) failed: %s", (unsigned long long)b->L.total, cudaGetErrorString(e));
+      return fail(RASP_ENOMEM, "cudaMalloc(%llu) failed: %s", total, cudaGetErrorString(e));
     }
     b->base = (char*)p;
     b->owns = true;
@@ -728,10 +744,11 @@ ProgramLook look_at(const W* words, const uint64_t* offsets, uint64_t num_progra
 // the pack) in the part of the program area that the programs leave free: behind
 // the 8-byte words, or behind where they would be widened to -- from the start
 // when nothing widens them. NULL where there is no room (programs that fill
-// more than half of the memories), where no kernel of the batch's options runs
+// more than half of the memories; a batch laid out without room for their
+// records), where no kernel of the batch's options runs
 // from them, or where a program has more instructions than an entry can name.
 uint4* place_fused(const rasp_batch* b, uint64_t total, bool keep32) {
-  if (!total || !runs_entries(variant_of(b)) || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
+  if (!total || !b->L.off_frec || !runs_entries(variant_of(b)) || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
   const uint64_t lo = keep32 && owns_code(b) ? 0 : 8ull * total;
   const uint64_t end = keep32 ? 4ull * kept_words_at(b) : 8ull * b->mem_words;
   if (lo + 8ull * total > end || 8ull * total > (b->narrow ? 4ull : 8ull) * b->mem_words) return nullptr;

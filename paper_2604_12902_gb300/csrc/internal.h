@@ -203,8 +203,9 @@ cudaError_t launch_widen(const int32_t* src, uint64_t* dst, uint64_t count, cuda
 int create_batch(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan,
                  rasp_batch** out);
 
-// The device memory of such a batch (rasp_batch_bytes; arguments checked).
-uint64_t batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan);
+// The device memory of such a batch (rasp_batch_bytes; arguments checked);
+// without `room` the least that create_batch takes: no fused entries.
+uint64_t batch_bytes(const rasp_config* cfg, uint64_t num_vms, const uint32_t* mem_words, bool plan, bool room);
 
 // The state store and step parameters of a batch (for the serving pool).
 const RunState& batch_run_state(const rasp_batch* b);

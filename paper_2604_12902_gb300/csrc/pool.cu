@@ -477,7 +477,8 @@ int rasp_pool_submit(rasp_pool* p, const rasp_request* q, uint64_t* ticket) {
   uint64_t need = 0;
   int rc = rasp_batch_bytes(&p->cfg, q->num_vms, q->mem_words, &need);
   if (rc) return pfail(rc, std::string("request rejected: ") + rasp_last_error());
-  need = batch_bytes(&p->cfg, q->num_vms, q->mem_words, false);   // as create_batch lays it out without a plan
+  need = batch_bytes(&p->cfg, q->num_vms, q->mem_words, false, true);   // as create_batch lays it out without a plan
+  if (need > p->bytes) need = batch_bytes(&p->cfg, q->num_vms, q->mem_words, false, false);
   need = (need + kAlign - 1) & ~(kAlign - 1);
   if (need > p->bytes) return pfail(RASP_ENOMEM, "request needs more device memory than the whole pool");
   std::lock_guard<std::mutex> lock(p->mu);

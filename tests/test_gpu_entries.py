@@ -421,3 +421,48 @@ def test_pools_of_small_words(rasp, w):
         tickets = [pool.submit(wl) for _ in range(3)]
         for t in tickets:
             assert_same_state(pool.read(t), st, wl.ell, wl.s, what="pool, w = %d" % w)
+
+
+@pytest.mark.parametrize("sched,w", [(0x00, 64), (0x00, 32), (0x40, 64), (0x20, 64)])
+def test_arenas_without_room_for_entries(rasp, sched, w):
+    """A caller's arena that lacks only the room for entries and between slabs
+    (16 bytes per 128 words and per VM, 32 bytes after every second slab) holds
+    the batch without them; a smaller one is refused."""
+    import ctypes
+    import torch
+    V = 999
+    wl = machines(V, 30, w, seed=190 + w + sched, extra=90, shared=40 if sched == 0x40 else 0)
+    st, _ = oracle_state(wl, threads=8)
+    cfg = rasp.rasp_config(w, 0, wl.ell, wl.s, sched, 0, 0, 0, 0, 0, None, None, 0)
+    pad = (V - 1) // 2 * 4
+    words = int((wl.mem_words.astype(np.int64) + 1 & ~1).sum()) + pad
+    lean = rasp.rasp_batch_bytes(cfg, wl.mem_words) - 16 * (words // 128 + V + 1) - (8 + (4 if w == 32 else 8)) * pad
+    arena = torch.empty(lean + 1024, dtype=torch.uint8, device="cuda")
+    cfg.arena = ctypes.c_void_p(arena.data_ptr())
+    for size, ok in ((lean + 1024, True), (lean - 2048, False)):
+        cfg.arena_bytes = size
+        if not ok:
+            with pytest.raises(rasp.RaspError):
+                rasp.rasp_batch_create(cfg, wl.mem_words)
+            continue
+        b = rasp.Batch.__new__(rasp.Batch)
+        b.mem_words, b.V, b.ell, b.s, b.w, b.cfg, b._arena = wl.mem_words, V, wl.ell, wl.s, w, cfg, arena
+        b.h, b.n_total = rasp.rasp_batch_create(cfg, wl.mem_words), int(wl.mem_words.sum())
+        with b:
+            b.load_workload(wl)
+            assert not b.describe()["entries"]
+            for _ in range(2):
+                b.run()
+                assert_same_state(b.read_state(), st, wl.ell, wl.s, what="lean arena")
+                b.reset()
+
+
+def test_pools_without_room_for_entries(rasp):
+    from paper_2604_12902_gb300 import serving
+    V = 20_000
+    wl = W.template_programs(num_vms=V, seed=12)
+    st, _ = oracle_state(wl, threads=8)
+    cfg = rasp.rasp_config(64, 0, wl.ell, wl.s, 0, 0, 0, 0, 0, 0, None, None, 0)
+    with serving.Pool(rasp.rasp_batch_bytes(cfg, wl.mem_words) - 32 * V, wl.ell, wl.s) as pool:
+        for _ in range(2):
+            assert_same_state(pool.read(pool.submit(wl)), st, wl.ell, wl.s, what="lean pool")
