@@ -198,9 +198,19 @@ int rasp_batch_create(const rasp_config* cfg, uint64_t num_vms,
  * WRAP programs are also decoded on the device, into entries of several
  * instructions that the schedules AUTO, PERSIST_GL and SHARED and the pools run
  * from while a VM has not written into its program (results do not depend on
- * it; rasp_describe says whether there are any): not with RASP_COLLECT_STATS,
- * RASP_DISPATCH_VOTE or RASP_STEP_BLOCK, nor where the programs fill more than
- * half of the memories.
+ * it; rasp_describe says whether there are any). This call decodes where the
+ * plan runs from entries, unless the inputs' caps are known and too small for
+ * a first run to gain by it; otherwise the first run or tuning that gains by
+ * them does. There are no entries
+ * - with RASP_COLLECT_STATS, RASP_DISPATCH_VOTE, RASP_STEP_BLOCK or CHECKED;
+ * - where the programs fill more than half of the memories; for programs
+ *   given as int32 that VMs share, or on RASP_SCHED_SHARED, a quarter;
+ * - where one program has more than 65,535 instructions (on RASP_SCHED_SHARED
+ *   6,144 words);
+ * - where an eighth of the instructions of most programs (up to 64 are looked
+ *   at) write into the program or have operands that no entry holds: words
+ *   behind 65,535, and in shared programs constants beyond 16 bits;
+ * - in an arena without room for their records (see rasp_batch_bytes).
  * EINVAL: odd program length, 2m > n of a VM using it, bad index. The copy
  * to the device is issued before the per-program checks run (so that they
  * overlap it); after a failed check the batch holds no programs and

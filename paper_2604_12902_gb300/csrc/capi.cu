@@ -138,6 +138,7 @@ struct rasp_batch {
   uint32_t max_plen = 0;
   uint4* fuse_at = nullptr;    // the place of the programs' fused entries (NULL: they get none); S.fops once decoded
   bool self_writing = false;   // most of the loaded programs write into themselves (look_at)
+  bool ran = false;            // rasp_run since the programs were loaded
   bool fuse_own = false;       // the entries may read program words as data (owns_code at the load)
   bool dirty_valid = false;    // codedirty is up to date for the VMs of the schedules that keep it
   bool ran_untracked = false;  // since the last pack a schedule ran that does not keep codedirty
@@ -765,6 +766,20 @@ bool uses_entries(const rasp_batch* b) {
   return uses;
 }
 
+// Whether a first run to at most `steps` steps makes up for decoding: not below
+// 16 steps for each instruction that a VM has on average, for few VMs (whose
+// decoding takes less of the GPU) down to five. Load and run from page-locked
+// memory, without entries and with: 262,144 templates of 64 instructions to 200
+// steps 1.50 and 1.87 ms, to 1,000 2.26 and 2.16; 32,768 uneven programs of 121
+// to 400 0.54 and 0.75, to 2,500 1.04 and 1.01; 65,536 halting programs of 44
+// to 300 1.02 and 1.13, to 1,000 1.19 and 1.16; 2,048 templates to 200 0.101
+// and 0.119, to 450 0.138 and 0.137; 8,192 uneven to 400 0.26 and 0.29, to
+// 1,000 0.37 and 0.37.
+bool entries_pay(const rasp_batch* b, uint64_t steps) {
+  const uint64_t factor = std::min<uint64_t>(std::max<uint64_t>(b->V / 1024u, 5u), 16u);
+  return steps >= factor * (b->prog_words / 2u) / b->V;
+}
+
 // The smallest memory that runs each program, for the decoder: S.n where VM v
 // runs program v, else into d_ids2. pvm: the program of each VM (NULL: read back).
 cudaError_t program_bounds(rasp_batch* b, const uint32_t* pvm, cudaStream_t st) {
@@ -793,11 +808,13 @@ cudaError_t decode_entries(rasp_batch* b, uint4* tmp, cudaStream_t st) {
   return e;
 }
 
-// The plan has come to run from entries after a load that did not make them
-// (eagerly, outside any captured graph).
+// Entries after a load that did not make them: the plan has come to run from
+// them, or a load for a short run is run again (eagerly, outside any captured
+// graph).
 cudaError_t late_entries(rasp_batch* b, cudaStream_t st) {
   if (b->S.fops || !b->fuse_at) return cudaSuccess;
   drop_graphs(b);                              // captured runs hold the old launch arguments
+  if (b->ran_untracked) b->dirty_valid = false;   // VMs may have written program words since the pack
   const cudaError_t e = program_bounds(b, nullptr, st);
   return e == cudaSuccess ? decode_entries(b, nullptr, st) : e;
 }
@@ -904,14 +921,17 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   b->S.frec = (const uint4*)(b->base + b->L.off_frec);
   b->S.prog_off = b->d_progoff;
   b->S.prog_of_vm = b->shared_programs ? b->d_progvm : nullptr;
-  if (uses_entries(b)) CK(program_bounds(b, prog_of_vm, st));
+  b->prog_words = total;
+  b->ran = false;
+  // (inputs not loaded: their caps are not known; a second run decodes)
+  const bool decode = uses_entries(b) && (!b->inputs_loaded || entries_pay(b, b->max_cap));
+  if (decode) CK(program_bounds(b, prog_of_vm, st));
   // widening, like the pack, is left queued on the stream: it may have to
   // wait for SMs that another batch's run holds, and the host need not
   b->prog32 = keep32 && total ? staged : nullptr;
-  b->prog_words = total;
   b->prog64_valid = !b->prog32;
   if (word_size == 4 && total && !keep32) CK(launch_widen(staged, b->d_prog, total, st));
-  if (uses_entries(b)) CK(decode_entries(b, reinterpret_cast<uint4*>(b->S.mem), st));
+  if (decode) CK(decode_entries(b, reinterpret_cast<uint4*>(b->S.mem), st));
   if (!same_args || b->S.fops != fops_before || b->self_writing != writing_before) drop_graphs(b);   // captured runs hold the old launch arguments
   CK(fill_bytes(b->d_hist, 0, 8 * 10, st));
   b->code_lazy = pack_lazy(b);
@@ -1104,7 +1124,8 @@ int rasp_run(rasp_batch* b, uint64_t max_steps) {
     const int rc = replan(b);
     if (rc) return rc;
   }
-  if (uses_entries(b)) CK(late_entries(b, b->stream));
+  if (uses_entries(b) && (b->ran || entries_pay(b, std::min(max_steps, b->max_cap)))) CK(late_entries(b, b->stream));
+  b->ran = true;
   // 8-byte program words for the kernels that read them, eagerly (outside any captured graph)
   if (b->code_lazy || (b->cfg.flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED) CK(ensure_prog64(b, b->stream));
   CK(settle_dirty(b, b->stream));

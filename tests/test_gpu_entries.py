@@ -466,3 +466,44 @@ def test_pools_without_room_for_entries(rasp):
     with serving.Pool(rasp.rasp_batch_bytes(cfg, wl.mem_words) - 32 * V, wl.ell, wl.s) as pool:
         for _ in range(2):
             assert_same_state(pool.read(pool.submit(wl)), st, wl.ell, wl.s, what="lean pool")
+
+
+@pytest.mark.parametrize("flags", [0x0, 0x4000], ids=["eager", "cuda-graph"])
+@pytest.mark.parametrize("w", [64, 32])
+def test_short_runs_of_new_programs(rasp, w, flags):
+    """Programs loaded after inputs with small caps are decoded by the second
+    run, whether it starts from c_0 or goes on from memories that the first
+    has written code into; with larger caps or steps by the load or the run."""
+    wl = machines(700, 60, w, seed=200 + w, extra=130, p_code=0.2)
+    short = np.minimum(wl.caps, 250)
+    with rasp.Batch(wl.mem_words, wl.ell, wl.s, word_bits=w, flags=flags) as b:
+        def load(caps):
+            wl.caps = caps
+            b.load_inputs(wl.tapes, wl.tape_off, caps)
+            b.load_programs(wl.programs, wl.prog_off)
+
+        def run(t, entries):
+            b.run(t)
+            assert b.describe()["entries"] is entries
+            assert_same_state(b.read_state(), oracle_state(wl, budget=t, threads=8)[0], wl.ell, wl.s, what="%d" % t)
+
+        long = wl.caps.copy()
+        for _ in range(2):
+            load(short)
+            run(1000, False)
+            b.reset()
+            run(30, True)
+            run(1000, True)
+            load(short)
+            run(40, False)
+            run(90, True)                     # from memories without marks
+            run(1000, True)
+            b.reset()
+            run(1000, True)
+            load(long)
+            run(30, True)
+            run(1000, True)
+            load(short)
+            wl.caps = long
+            b.load_inputs(wl.tapes, wl.tape_off, long)
+            run(1000, True)
