@@ -1380,6 +1380,7 @@ int rasp_read_stats(rasp_batch* b, rasp_stats* out) {
 namespace {
 
 void drop_graphs(rasp_batch* b) {
+  if (!b->graphs.empty()) cudaStreamSynchronize(b->stream);   // their launches have ended
   for (auto& e : b->graphs) cudaGraphExecDestroy(e.second);
   b->graphs.clear();
 }
