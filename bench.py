@@ -181,8 +181,10 @@ def outcomes(stats) -> dict:
 
 def algorithmic_bytes(stats, fetch_from_smem: bool = False, word_bytes: int = 8) -> float:
     """Opcode-weighted bytes of VM state touched by the executed steps; with
-    fetch_from_smem the 16-byte instruction fetch is left out (the
-    shared-program kernel reads the program words from shared memory). The
+    fetch_from_smem the 16-byte instruction fetch is left out: the shared-program
+    kernel reads the program words from shared memory, and a VM that runs from
+    fused entries fetches 16 bytes for several steps, which are not counted
+    here either (so the fraction is of the data alone). The
     table is in 8-byte words; a batch held in 4-byte words (w <= 32) touches
     half as many bytes per access."""
     ops = stats["op_steps"]
@@ -195,6 +197,11 @@ def algorithmic_bytes(stats, fetch_from_smem: bool = False, word_bytes: int = 8)
 
 KERNEL_OF = {"persist_gl": "k_persist_gl", "plain": "k_plain", "persist_smem": "k_persist", "shared": "k_shared_loop"}
 SCHED_NAME = {0x10: "plain", 0x20: "persist_smem", 0x30: "persist_gl", 0x40: "shared"}
+
+
+def fetch_free(kernel: str, batch) -> bool:
+    """Whether the run kernel makes no 16-byte fetch of its own for each VM-step."""
+    return kernel.startswith("k_shared") or (kernel == "k_persist_gl" and bool(batch.describe().get("entries")))
 
 
 def run_kernel_name(chosen: str, flags: int) -> str:
@@ -244,7 +251,8 @@ def time_config(R, torch, wl, desc, flags, steps, warmup, flush_l2=False):
         chosen = tuned["chosen"] if tuned else "flags %#x" % flags
         kernel = run_kernel_name(chosen if tuned else SCHED_NAME.get(flags & 0xF0, "persist_gl"), flags)
         word_bytes = b.describe().get("word_bytes", 8)
-        alg = algorithmic_bytes(stats, fetch_from_smem=kernel.startswith("k_shared"), word_bytes=word_bytes)
+        no_fetch = fetch_free(kernel, b)
+        alg = algorithmic_bytes(stats, fetch_from_smem=no_fetch, word_bytes=word_bytes)
         for _ in range(warmup):
             b.reset()
             b.run()
@@ -279,7 +287,8 @@ def time_config(R, torch, wl, desc, flags, steps, warmup, flush_l2=False):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                          "traffic": None, "kernel": kernel, "peak_kind": peak_kind,
                          "bytes_per_step": alg / max(stats["vm_steps"], 1),
-                         "fetch_from_smem_excluded": kernel.startswith("k_shared"), "word_bytes": word_bytes,
+                         "fetch_from_smem_excluded": kernel.startswith("k_shared"), "fetch_excluded": no_fetch,
+                         "word_bytes": word_bytes,
                          "kernel_ms": run_avg, "pack_ms": float(np.mean(pack_ms))},
             "outcomes": outcomes(st)}
 
@@ -536,9 +545,9 @@ def main():
         stats = bs.stats()
     total_steps = stats["vm_steps"]
     kernel = run_kernel_name(tuned["chosen"] if tuned else SCHED_NAME.get(args.flags & 0xF0, "persist_gl"), args.flags)
-    # the shared-program kernel reads instruction pairs from shared memory
     word_bytes = b.describe().get("word_bytes", 8)
-    alg_bytes = algorithmic_bytes(stats, fetch_from_smem=kernel.startswith("k_shared"), word_bytes=word_bytes)
+    no_fetch = fetch_free(kernel, b)
+    alg_bytes = algorithmic_bytes(stats, fetch_from_smem=no_fetch, word_bytes=word_bytes)
 
     # halting workload: the tau_h histogram is computed on the device in every step
     hist_edges = np.concatenate([np.arange(0, 101), [10 ** 6, 1 << 62]]).astype(np.uint64)
@@ -593,7 +602,7 @@ def main():
     run_avg = float(np.mean(run_ms))
     achieved = alg_bytes / (run_avg * 1e-3) / 1e9
     # the summary was taken on the default launch shape (HBM-slab persistent,
-    # 4 warps x 7 CTAs per SM, epoch 128); a tuned shape that differs only in
+    # 4 warps x 6 CTAs per SM, epoch 128); a tuned shape that differs only in
     # its epoch runs the same kernel at the same occupancy
     chosen = tuned.get("chosen", "") if tuned else "persist_gl e128 w4"
     same_shape = args.workload == "templates" and args.flags == 0 and not args.epoch and \
@@ -604,7 +613,8 @@ def main():
                 "traffic_source": "profiles/traffic.json (ncu, 262,144-VM case, epoch 128, scaled by VM-steps)"
                 if traffic is not None else None,
                 "kernel": kernel, "peak_kind": peak_kind,
-                "fetch_from_smem_excluded": kernel.startswith("k_shared"), "word_bytes": word_bytes,
+                "fetch_from_smem_excluded": kernel.startswith("k_shared"), "fetch_excluded": no_fetch,
+                "word_bytes": word_bytes,
                 "bytes_per_step": alg_bytes / max(total_steps, 1),
                 "kernel_ms": run_avg, "pack_ms": float(np.mean(pack_ms))}
 
