@@ -745,8 +745,8 @@ ProgramLook look_at(const W* words, const uint64_t* offsets, uint64_t num_progra
 // the pack) in the part of the program area that the programs leave free: behind
 // the 8-byte words, or behind where they would be widened to -- from the start
 // when nothing widens them. NULL where there is no room (programs that fill
-// more than half of the memories; a batch laid out without room for their
-// records), where no kernel of the batch's options runs
+// more than half of the memories, or a quarter where they are kept as 4-byte
+// words and may be widened; a batch laid out without room for their records), where no kernel of the batch's options runs
 // from them, or where a program has more instructions than an entry can name.
 uint4* place_fused(const rasp_batch* b, uint64_t total, bool keep32) {
   if (!total || !b->L.off_frec || !runs_entries(variant_of(b)) || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
