@@ -746,8 +746,9 @@ ProgramLook look_at(const W* words, const uint64_t* offsets, uint64_t num_progra
 // the 8-byte words, or behind where they would be widened to -- from the start
 // when nothing widens them. NULL where there is no room (programs that fill
 // more than half of the memories, or a quarter where they are kept as 4-byte
-// words and may be widened; a batch laid out without room for their records), where no kernel of the batch's options runs
-// from them, or where a program has more instructions than an entry can name.
+// words and may be widened; a batch laid out without room for their records),
+// where no kernel of the batch's options runs from them, or where a program has
+// more instructions than an entry can name.
 uint4* place_fused(const rasp_batch* b, uint64_t total, bool keep32) {
   if (!total || !b->L.off_frec || !runs_entries(variant_of(b)) || b->max_plen / 2u > kFuseMaxInstr) return nullptr;
   const uint64_t lo = keep32 && owns_code(b) ? 0 : 8ull * total;
@@ -810,9 +811,19 @@ cudaError_t decode_entries(rasp_batch* b, uint4* tmp, cudaStream_t st) {
 
 // Entries after a load that did not make them: the plan has come to run from
 // them, or a load for a short run is run again (eagerly, outside any captured
-// graph).
-cudaError_t late_entries(rasp_batch* b, cudaStream_t st) {
+// graph). While the caller captures the stream nothing can be decoded, and a
+// run captured without entries does not keep codedirty whenever it is replayed:
+// the programs then stay without entries until the next load. pay: they are
+// worth making.
+cudaError_t late_entries(rasp_batch* b, cudaStream_t st, bool pay) {
   if (b->S.fops || !b->fuse_at) return cudaSuccess;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    b->fuse_at = nullptr;
+    return cudaSuccess;
+  }
+  if (!pay) return cudaSuccess;
   drop_graphs(b);                              // captured runs hold the old launch arguments
   if (b->ran_untracked) b->dirty_valid = false;   // VMs may have written program words since the pack
   const cudaError_t e = program_bounds(b, nullptr, st);
@@ -932,7 +943,8 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   b->prog64_valid = !b->prog32;
   if (word_size == 4 && total && !keep32) CK(launch_widen(staged, b->d_prog, total, st));
   if (decode) CK(decode_entries(b, reinterpret_cast<uint4*>(b->S.mem), st));
-  if (!same_args || b->S.fops != fops_before || b->self_writing != writing_before) drop_graphs(b);   // captured runs hold the old launch arguments
+  // captured runs hold the old launch arguments
+  if (!same_args || b->S.fops != fops_before || b->self_writing != writing_before) drop_graphs(b);
   CK(fill_bytes(b->d_hist, 0, 8 * 10, st));
   b->code_lazy = pack_lazy(b);
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,
@@ -1124,7 +1136,7 @@ int rasp_run(rasp_batch* b, uint64_t max_steps) {
     const int rc = replan(b);
     if (rc) return rc;
   }
-  if (uses_entries(b) && (b->ran || entries_pay(b, std::min(max_steps, b->max_cap)))) CK(late_entries(b, b->stream));
+  if (uses_entries(b)) CK(late_entries(b, b->stream, b->ran || entries_pay(b, std::min(max_steps, b->max_cap))));
   b->ran = true;
   // 8-byte program words for the kernels that read them, eagerly (outside any captured graph)
   if (b->code_lazy || (b->cfg.flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED) CK(ensure_prog64(b, b->stream));
@@ -1403,7 +1415,7 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
   if (reps == 0) reps = 1;
   CK(apply_uhead_reset(b, b->stream));
   if (b->shared_programs || b->code_lazy) CK(ensure_prog64(b, b->stream));   // the shared-program trials
-  CK(late_entries(b, b->stream));              // the HBM-slab trials run from them
+  CK(late_entries(b, b->stream, true));        // the HBM-slab trials run from them
   int rc = check_device_error(b);
   if (rc) return rc;
   cudaStream_t st = b->stream;

@@ -91,8 +91,7 @@ inline bool shared_fuses(uint32_t max_plen) { return 16ull * ((max_plen + 1u) & 
 // What a persistent launch over `count` VMs is: the resident CTAs of the kernel
 // that runs (with fused entries fewer fit an SM), at most as many as the VMs
 // fill; few VMs in the HBM-slab form spread over one-warp CTAs unless warps or
-// CTAs were set. dense: a
-// compacted queue, of at most `count` VMs.
+// CTAs were set. dense: a compacted queue, of at most `count` VMs.
 struct PersistLaunch {
   uint32_t grid, warps, lanes;   // CTAs, warps per CTA, lanes of a warp that take VMs
   bool fuse;

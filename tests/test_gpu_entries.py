@@ -507,3 +507,34 @@ def test_short_runs_of_new_programs(rasp, w, flags):
             wl.caps = long
             b.load_inputs(wl.tapes, wl.tape_off, long)
             run(1000, True)
+
+
+@pytest.mark.parametrize("shared", [0, 40])
+@pytest.mark.parametrize("warm", [False, True])
+def test_short_runs_in_the_callers_graph(rasp, shared, warm):
+    """A run that the caller captures decodes nothing; its replays, which keep
+    no marks, mix with later runs."""
+    import torch
+    wl = machines(600, 60, 64, seed=210 + shared, extra=130, p_code=0.2, shared=shared)
+    wl.caps = np.minimum(wl.caps, 250)
+    part, full = (oracle_state(wl, budget=t, threads=8)[0] for t in (60, 1000))
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side), rasp.Batch(wl.mem_words, wl.ell, wl.s) as b:
+        b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+        for _ in range(2):
+            b.load_programs(wl.programs, wl.prog_off, wl.prog_of_vm)
+            assert b.describe()["entries"] is bool(shared)   # (shared: few instructions for each machine)
+            if warm:
+                b.run(60)
+                b.reset()
+            side.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                b.run(60)
+            for _ in range(2):
+                g.replay()
+                assert_same_state(b.read_state(), part, wl.ell, wl.s, what="replay")
+                b.run(1000)
+                assert_same_state(b.read_state(), full, wl.ell, wl.s, what="run on")
+                b.reset()
+            assert b.describe()["entries"] is bool(shared)
