@@ -142,6 +142,7 @@ struct rasp_batch {
   bool fuse_own = false;       // the entries may read program words as data (owns_code at the load)
   bool dirty_valid = false;    // codedirty is up to date for the VMs of the schedules that keep it
   bool ran_untracked = false;  // since the last pack a schedule ran that does not keep codedirty
+  bool replays = false;        // a caller's graph may run VMs without keeping codedirty
   bool code_lazy = false;      // slabs of VMs with codedirty = 0 lack their program words (lazy pack)
   bool tuned_block = false;    // autotuned: the SMEM-staged schedule one step at a time
   bool narrow = false;         // M in 4-byte words (w <= 32)
@@ -419,16 +420,30 @@ bool tracks_code(const rasp_batch* b, const Group& g) {
   return g.sched == RASP_SCHED_PERSIST_GL && b->S.fops && runs_entries(variant_of(b));
 }
 
-// Before a run (eagerly, outside any captured graph): where codedirty is not
-// up to date -- another schedule may have written program words, and the plan
-// has changed since -- every VM runs from its memory until the next pack.
+// Whether the caller captures the stream into a graph of its own.
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &c) == cudaSuccess && c == cudaStreamCaptureStatusNone) return false;
+  cudaGetLastError();
+  return true;
+}
+
+// Before a run (eagerly, outside the batch's own graphs): where codedirty is
+// not up to date -- another schedule may have written program words, and the
+// plan has changed since -- every VM runs from its memory until the next pack.
+// In a caller's graph the marks are set when it is replayed, so they stay out
+// of date for the runs before that; and a run that keeps no marks may be
+// replayed at any time, so that from then on they are out of date before every
+// run.
 cudaError_t settle_dirty(rasp_batch* b, cudaStream_t st) {
   bool tracked = false, untracked = false;
   for (const Group& g : b->groups) (tracks_code(b, g) ? tracked : untracked) = true;
   cudaError_t e = cudaSuccess;
-  if (tracked && !b->dirty_valid) {
+  const bool captured = capturing(st);
+  b->replays = b->replays || (captured && untracked);
+  if (tracked && (!b->dirty_valid || b->replays)) {
     e = cudaMemsetAsync(b->S.codedirty, 1, b->V, st);
-    b->dirty_valid = true;
+    b->dirty_valid = !captured;
   }
   b->ran_untracked = b->ran_untracked || untracked;
   return e;
@@ -811,15 +826,12 @@ cudaError_t decode_entries(rasp_batch* b, uint4* tmp, cudaStream_t st) {
 
 // Entries after a load that did not make them: the plan has come to run from
 // them, or a load for a short run is run again (eagerly, outside any captured
-// graph). While the caller captures the stream nothing can be decoded, and a
-// run captured without entries does not keep codedirty whenever it is replayed:
-// the programs then stay without entries until the next load. pay: they are
-// worth making.
+// graph). While the caller captures the stream nothing can be decoded, and the
+// run captured without entries keeps no marks (see settle_dirty): the batch
+// then stays without them. pay: they are worth making.
 cudaError_t late_entries(rasp_batch* b, cudaStream_t st, bool pay) {
   if (b->S.fops || !b->fuse_at) return cudaSuccess;
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
+  if (capturing(st)) {
     b->fuse_at = nullptr;
     return cudaSuccess;
   }
@@ -925,7 +937,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   if (total)
     look = word_size == 8 ? look_at((const int64_t*)words, offsets, num_programs, b->wmask, owns_code(b))
                           : look_at((const int32_t*)words, offsets, num_programs, b->wmask, owns_code(b));
-  b->fuse_at = look.unfit ? nullptr : place_fused(b, total, keep32);
+  b->fuse_at = look.unfit || b->replays ? nullptr : place_fused(b, total, keep32);
   b->fuse_own = owns_code(b);
   b->self_writing = look.writing;
   b->S.fops = nullptr;

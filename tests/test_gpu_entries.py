@@ -538,3 +538,54 @@ def test_short_runs_in_the_callers_graph(rasp, shared, warm):
                 assert_same_state(b.read_state(), full, wl.ell, wl.s, what="run on")
                 b.reset()
             assert b.describe()["entries"] is bool(shared)
+
+
+@pytest.mark.parametrize("w", [64, 32])
+def test_callers_graphs_and_the_marks(rasp, w):
+    """Replays of a run captured on the plain schedule write program words
+    without marks; marks set inside a capture are not there before its replay."""
+    import torch
+    wl = machines(600, 60, w, seed=220 + w, extra=130, p_code=0.2)
+    full = oracle_state(wl, threads=8)[0]
+    side = torch.cuda.Stream()
+
+    def batch():
+        b = rasp.Batch(wl.mem_words, wl.ell, wl.s, word_bits=w)
+        b.load_workload(wl)
+        assert b.describe()["entries"]
+        return b, b.describe()["buckets"][0]["index"]
+
+    def capture(b, t):
+        side.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            b.run(t)
+        return g
+
+    with torch.cuda.stream(side):
+        b, k = batch()
+        b.plan_bucket(k, rasp.SCHED_PLAIN)
+        g = capture(b, 60)
+        b.plan_bucket(k, rasp.SCHED_PERSIST_GL)
+        for rep in range(3):
+            if rep == 2:
+                b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+                b.load_programs(wl.programs, wl.prog_off)
+            g.replay()
+            b.run()
+            assert_same_state(b.read_state(), full, wl.ell, wl.s, what="replayed on the plain schedule, %d" % rep)
+            b.reset()
+        b.close()
+
+        b, k = batch()
+        b.plan_bucket(k, rasp.SCHED_PLAIN)
+        b.run(60)
+        b.plan_bucket(k, rasp.SCHED_PERSIST_GL)
+        g = capture(b, 200)
+        b.run()
+        assert_same_state(b.read_state(), full, wl.ell, wl.s, what="marks captured, not replayed")
+        b.reset()
+        g.replay()
+        b.run()
+        assert_same_state(b.read_state(), full, wl.ell, wl.s, what="replayed after a reset")
+        b.close()
