@@ -142,7 +142,8 @@ struct rasp_batch {
   bool fuse_own = false;       // the entries may read program words as data (owns_code at the load)
   bool dirty_valid = false;    // codedirty is up to date for the VMs of the schedules that keep it
   bool ran_untracked = false;  // since the last pack a schedule ran that does not keep codedirty
-  bool replays = false;        // a caller's graph may run VMs without keeping codedirty
+  bool captured = false;       // the caller has captured a run into a graph of its own
+  bool replays = false;        // such a graph may run VMs without keeping codedirty
   bool code_lazy = false;      // slabs of VMs with codedirty = 0 lack their program words (lazy pack)
   bool tuned_block = false;    // autotuned: the SMEM-staged schedule one step at a time
   bool narrow = false;         // M in 4-byte words (w <= 32)
@@ -440,6 +441,7 @@ cudaError_t settle_dirty(rasp_batch* b, cudaStream_t st) {
   for (const Group& g : b->groups) (tracks_code(b, g) ? tracked : untracked) = true;
   cudaError_t e = cudaSuccess;
   const bool captured = capturing(st);
+  b->captured = b->captured || captured;
   b->replays = b->replays || (captured && untracked);
   if (tracked && (!b->dirty_valid || b->replays)) {
     e = cudaMemsetAsync(b->S.codedirty, 1, b->V, st);
@@ -1027,6 +1029,7 @@ int rasp_load_inputs(rasp_batch* b, const int64_t* tape, const uint64_t* offsets
     if (rc) return rc;
   }
   b->uhead_pending = true;         // u_0 = 0: by the next pack, or before u_0 is next read
+  if (b->captured) CK(apply_uhead_reset(b, st));   // which a replay of a caller's graph would not see
   b->inputs_loaded = true;
   g_err.clear();
   return RASP_OK;

@@ -589,3 +589,21 @@ def test_callers_graphs_and_the_marks(rasp, w):
         b.run()
         assert_same_state(b.read_state(), full, wl.ell, wl.s, what="replayed after a reset")
         b.close()
+
+
+def test_new_inputs_of_a_callers_graph(rasp):
+    """u_0 = 0 of new inputs is not owed until after the replay that reads them."""
+    import torch
+    side = torch.cuda.Stream()
+    a, c = (machines(600, 60, 64, seed=seed, extra=130) for seed in (230, 231))
+    with torch.cuda.stream(side), rasp.Batch(a.mem_words, a.ell, a.s) as b:
+        b.load_workload(a)
+        b.run()
+        side.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            b.run()
+        for wl in (c, a):
+            b.load_workload(wl)
+            g.replay()
+            assert_same_state(b.read_state(), oracle_state(wl, threads=8)[0], wl.ell, wl.s, what="new inputs")
