@@ -142,6 +142,11 @@ struct rasp_batch {
   bool fuse_own = false;       // the entries may read program words as data (owns_code at the load)
   bool dirty_valid = false;    // codedirty is up to date for the VMs of the schedules that keep it
   bool ran_untracked = false;  // since the last pack a schedule ran that does not keep codedirty
+  // a caller's graph runs from entries at this place, of programs shared so; once
+  // these are gone, every VM is marked after every pack
+  const uint4* graph_fops = nullptr;
+  const uint32_t* graph_pvm = nullptr;
+  bool marked = false;
   bool captured = false;       // the caller has captured a run into a graph of its own
   bool replays = false;        // such a graph may run VMs without keeping codedirty
   bool code_lazy = false;      // slabs of VMs with codedirty = 0 lack their program words (lazy pack)
@@ -402,7 +407,7 @@ void build_groups(rasp_batch* b) {
 // The shared-program schedule reads program words from the program itself
 // until a VM writes one of them, so its c_0 writes only the data words.
 bool pack_lazy(const rasp_batch* b) {
-  return b->planned && (b->cfg.flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED;
+  return b->planned && !b->marked && (b->cfg.flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED;
 }
 
 // The 8-byte program words of programs kept as 4-byte words, before a
@@ -435,13 +440,22 @@ bool capturing(cudaStream_t st) {
 // In a caller's graph the marks are set when it is replayed, so they stay out
 // of date for the runs before that; and a run that keeps no marks may be
 // replayed at any time, so that from then on they are out of date before every
-// run.
-cudaError_t settle_dirty(rasp_batch* b, cudaStream_t st) {
-  bool tracked = false, untracked = false;
-  for (const Group& g : b->groups) (tracks_code(b, g) ? tracked : untracked) = true;
+// run. A graph that runs from entries keeps their place, where a later load may
+// put something else: such a load marks every VM, and so does every pack after
+// it, since a marked VM does not look at its entries.
+cudaError_t settle_dirty(rasp_batch* b, cudaStream_t st, bool captured) {
+  bool tracked = false, untracked = false, entries = false;
+  for (const Group& g : b->groups) {
+    (tracks_code(b, g) ? tracked : untracked) = true;
+    entries = entries || (g.sched == RASP_SCHED_PERSIST_GL && tracks_code(b, g));
+  }
   cudaError_t e = cudaSuccess;
-  const bool captured = capturing(st);
   b->captured = b->captured || captured;
+  if (captured && entries) {
+    b->marked = b->marked || (b->graph_fops && (b->graph_fops != b->S.fops || b->graph_pvm != b->S.prog_of_vm));
+    b->graph_fops = b->S.fops;
+    b->graph_pvm = b->S.prog_of_vm;
+  }
   b->replays = b->replays || (captured && untracked);
   if (tracked && (!b->dirty_valid || b->replays)) {
     e = cudaMemsetAsync(b->S.codedirty, 1, b->V, st);
@@ -469,6 +483,11 @@ cudaError_t apply_uhead_reset(rasp_batch* b, cudaStream_t st) {
   if (!b->uhead_pending) return cudaSuccess;
   b->uhead_pending = false;
   return fill_bytes(b->S.uhead, 0, 4ull * b->V, st);
+}
+
+// After a pack: see settle_dirty.
+cudaError_t mark_all(rasp_batch* b, cudaStream_t st) {
+  return b->marked ? cudaMemsetAsync(b->S.codedirty, 1, b->V, st) : cudaSuccess;
 }
 
 int replan(rasp_batch* b);
@@ -908,6 +927,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
                  (unsigned long long)(offsets[p + 1] - offsets[p]), b->h_n[v]);
   }
   if (bad) {
+    if (b->graph_fops) cudaMemsetAsync(b->S.codedirty, 1, b->V, st);   // the copy may lie where its entries were
     cudaStreamSynchronize(st);   // the caller's buffers are read before the call returns
     return bad;
   }
@@ -949,7 +969,12 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   b->prog_words = total;
   b->ran = false;
   // (inputs not loaded: their caps are not known; a second run decodes)
-  const bool decode = uses_entries(b) && (!b->inputs_loaded || entries_pay(b, b->max_cap));
+  bool decode = uses_entries(b) && (!b->inputs_loaded || b->graph_fops || entries_pay(b, b->max_cap));
+  if (b->graph_fops && !(decode && b->fuse_at == b->graph_fops && b->S.prog_of_vm == b->graph_pvm)) b->marked = true;
+  if (b->marked) {
+    b->fuse_at = nullptr;
+    decode = false;
+  }
   if (decode) CK(program_bounds(b, prog_of_vm, st));
   // widening, like the pack, is left queued on the stream: it may have to
   // wait for SMs that another batch's run holds, and the host need not
@@ -963,6 +988,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   b->code_lazy = pack_lazy(b);
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,
                  b->wmask, b->sp, b->code_lazy, st));
+  CK(mark_all(b, st));
   b->uhead_pending = false;        // the pack resets u_0
   b->programs_loaded = true;
   b->dirty_valid = true;
@@ -1042,6 +1068,7 @@ int rasp_reset(rasp_batch* b) {
   b->code_lazy = pack_lazy(b);
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,
                  b->wmask, b->sp, b->code_lazy, b->stream));
+  CK(mark_all(b, b->stream));
   b->uhead_pending = false;
   b->dirty_valid = true;
   b->ran_untracked = false;
@@ -1073,8 +1100,10 @@ constexpr uint64_t kRoundGrowth = 8;
 constexpr int kMaxRounds = 6;
 
 // Enqueue one rasp_run on `st`: reset the queue counters, one launch per group
-// (per budget round for the HBM-slab persistent schedule).
-int enqueue_run(rasp_batch* b, cudaStream_t st, uint64_t max_steps) {
+// (per budget round for the HBM-slab persistent schedule). In a caller's graph
+// (captured) the shared-program schedule goes without entries, which it copies
+// into shared memory from wherever they were.
+int enqueue_run(rasp_batch* b, cudaStream_t st, uint64_t max_steps, bool captured) {
   const StepVariant var = variant_of(b);
   Params P{};
   P.wmask = b->wmask;
@@ -1096,7 +1125,9 @@ int enqueue_run(rasp_batch* b, cudaStream_t st, uint64_t max_steps) {
     }
     if (g.sched == RASP_SCHED_SHARED) {
       CK(ensure_prog64(b, st));
-      CK(launch_shared(var, b->S, P, b->d_prog, b->d_progoff, b->d_pvoff, b->d_pvids, b->num_programs,
+      RunState S = b->S;
+      if (captured) S.fops = nullptr;
+      CK(launch_shared(var, S, P, b->d_prog, b->d_progoff, b->d_pvoff, b->d_pvids, b->num_programs,
                        b->max_plen, b->cfg.epoch, st));
     } else if (g.sched == RASP_SCHED_PLAIN) {
       CK(launch_plain(var, b->S, P, ids, g.count, st));
@@ -1155,15 +1186,16 @@ int rasp_run(rasp_batch* b, uint64_t max_steps) {
   b->ran = true;
   // 8-byte program words for the kernels that read them, eagerly (outside any captured graph)
   if (b->code_lazy || (b->cfg.flags & RASP_SCHED_MASK) == RASP_SCHED_SHARED) CK(ensure_prog64(b, b->stream));
-  CK(settle_dirty(b, b->stream));
-  if (!b->cap_stream) return enqueue_run(b, b->stream, max_steps);
+  const bool captured = capturing(b->stream);
+  CK(settle_dirty(b, b->stream, captured));
+  if (!b->cap_stream || captured) return enqueue_run(b, b->stream, max_steps, captured);
   // CUDA graph: capture the run once per budget on a private stream, replay it on the batch stream
   cudaGraphExec_t exec = nullptr;
   for (auto& e : b->graphs)
     if (e.first == max_steps) exec = e.second;
   if (!exec) {
     CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = enqueue_run(b, b->cap_stream, max_steps);
+    const int rc = enqueue_run(b, b->cap_stream, max_steps, false);
     cudaGraph_t graph = nullptr;
     const cudaError_t e = cudaStreamEndCapture(b->cap_stream, &graph);
     if (rc != RASP_OK) {
@@ -1496,10 +1528,10 @@ int rasp_autotune(rasp_batch* b, uint64_t max_steps, uint32_t reps) {
       b->dirty_valid = dirty_valid0 && !untracked0;
       b->code_lazy = code_lazy0;
       b->ran_untracked = untracked0;
-      if (ce == cudaSuccess) ce = settle_dirty(b, st);
+      if (ce == cudaSuccess) ce = settle_dirty(b, st, false);
       if (ce != cudaSuccess) break;
       cudaEventRecord(e0, st);
-      r2 = enqueue_run(b, st, max_steps);
+      r2 = enqueue_run(b, st, max_steps, false);
       if (r2) return r2;
       cudaEventRecord(e1, st);
       ce = cudaEventSynchronize(e1);

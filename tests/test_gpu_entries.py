@@ -607,3 +607,91 @@ def test_new_inputs_of_a_callers_graph(rasp):
             b.load_workload(wl)
             g.replay()
             assert_same_state(b.read_state(), oracle_state(wl, threads=8)[0], wl.ell, wl.s, what="new inputs")
+
+
+def test_new_programs_under_a_callers_graph(rasp):
+    """A graph that the caller has captured holds the place of the entries:
+    loads that move them, have none or fail leave its replays right."""
+    import torch
+    side = torch.cuda.Stream()
+    n = 250
+    kinds = [machines(500, m, 64, seed=240 + m, extra=n - 2 * m, p_code=0.05) for m in (60, 20, 41)]
+    kinds.append(W.random_programs(num_vms=500, seed=244, mem_words=n, tape_len=5, s=3, cap=600))
+    kinds.append(kinds[0])
+    full = [oracle_state(wl, threads=8)[0] for wl in kinds]
+    for i32 in (False, True):
+        with torch.cuda.stream(side), rasp.Batch(kinds[0].mem_words, 5, 3) as b:
+            def load(wl):
+                b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+                (rasp.rasp_load_programs_i32 if i32 else rasp.rasp_load_programs)(b.h, wl.programs, wl.prog_off)
+
+            load(kinds[0])
+            assert b.describe()["entries"]
+            b.run()
+            side.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                b.run()
+            for k, (wl, st) in enumerate(zip(kinds, full)):
+                load(wl)
+                assert b.describe()["entries"] is (k < 3 if i32 else k == 0)   # int32 words: one place for all
+                g.replay()
+                assert_same_state(b.read_state(), st, wl.ell, wl.s, what="kind %d" % k)
+                b.reset()
+                b.run(40)
+                g.replay()
+                assert_same_state(b.read_state(), st, wl.ell, wl.s, what="kind %d, after a run" % k)
+
+
+def test_a_failed_load_under_a_callers_graph(rasp):
+    import torch
+    side = torch.cuda.Stream()
+    wl = machines(500, 60, 64, seed=250, extra=130)
+    full = oracle_state(wl, threads=8)[0]
+    bad = np.arange(501, dtype=np.uint64) * np.uint64(220)       # words over the entries of those before
+    bad[7] += 1                                                  # an odd length
+    with torch.cuda.stream(side), rasp.Batch(wl.mem_words, wl.ell, wl.s) as b:
+        b.load_workload(wl)
+        b.run()
+        side.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            b.run()
+        b.reset()
+        b.run(25)
+        junk = np.full(500 * 220, 0x4444444444444444, np.int64)
+        with pytest.raises(rasp.RaspError):
+            b.load_programs(junk, bad)
+        g.replay()
+        assert_same_state(b.read_state(), full, wl.ell, wl.s, what="after a failed load")
+        b.load_workload(wl)
+        g.replay()
+        assert_same_state(b.read_state(), full, wl.ell, wl.s, what="loaded again")
+
+
+@pytest.mark.parametrize("flags", [0x40, 0x4040], ids=["shared", "shared, own graph too"])
+def test_shared_programs_under_a_callers_graph(rasp, flags):
+    import torch
+    side = torch.cuda.Stream()
+    kinds = [machines(700, m, 64, seed=260 + m, extra=240 - 2 * m, shared=30, p_code=0.05) for m in (60, 25)]
+    for wl in kinds:
+        wl.mem_words[:] = 240
+    full = [oracle_state(wl, threads=8)[0] for wl in kinds]
+    with torch.cuda.stream(side), rasp.Batch(kinds[0].mem_words, 5, 3, flags=flags) as b:
+        b.load_workload(kinds[0])
+        b.run()
+        side.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            b.run()
+        for k in (0, 1, 0):
+            wl = kinds[k]
+            b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+            b.load_programs(wl.programs, wl.prog_off, wl.prog_of_vm)
+            for _ in range(2):
+                g.replay()
+                assert_same_state(b.read_state(), full[k], wl.ell, wl.s, what="kind %d" % k)
+                b.reset()
+                b.run()
+                assert_same_state(b.read_state(), full[k], wl.ell, wl.s, what="kind %d, run" % k)
+                b.reset()
