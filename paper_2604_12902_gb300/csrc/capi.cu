@@ -152,6 +152,7 @@ struct rasp_batch {
   bool code_lazy = false;      // slabs of VMs with codedirty = 0 lack their program words (lazy pack)
   bool tuned_block = false;    // autotuned: the SMEM-staged schedule one step at a time
   bool narrow = false;         // M in 4-byte words (w <= 32)
+  bool uhead_moved = true;     // u_0 may differ from 0: no pack yet, or a run or a restored state since
   bool uhead_pending = false;  // u_0 = 0 owed since rasp_load_inputs (done by the pack or before the next use)
   bool ids_uploaded = false;   // d_ids holds h_ids
   bool ids_base = true;        // h_ids is h_ids_base (bucket order, no cap-class sort)
@@ -989,7 +990,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,
                  b->wmask, b->sp, b->code_lazy, st));
   CK(mark_all(b, st));
-  b->uhead_pending = false;        // the pack resets u_0
+  b->uhead_pending = b->uhead_moved = false;   // the pack resets u_0
   b->programs_loaded = true;
   b->dirty_valid = true;
   b->ran_untracked = false;
@@ -1054,7 +1055,7 @@ int rasp_load_inputs(rasp_batch* b, const int64_t* tape, const uint64_t* offsets
     const int rc = order_ids(b);
     if (rc) return rc;
   }
-  b->uhead_pending = true;         // u_0 = 0: by the next pack, or before u_0 is next read
+  b->uhead_pending = b->uhead_moved;   // u_0 = 0: by the next pack, or before u_0 is next read
   if (b->captured) CK(apply_uhead_reset(b, st));   // which a replay of a caller's graph would not see
   b->inputs_loaded = true;
   g_err.clear();
@@ -1069,7 +1070,7 @@ int rasp_reset(rasp_batch* b) {
   CK(launch_pack(b->S, b->d_prog, b->prog32, b->d_progoff, b->shared_programs ? b->d_progvm : nullptr, b->V,
                  b->wmask, b->sp, b->code_lazy, b->stream));
   CK(mark_all(b, b->stream));
-  b->uhead_pending = false;
+  b->uhead_pending = b->uhead_moved = false;
   b->dirty_valid = true;
   b->ran_untracked = false;
   return RASP_OK;
@@ -1177,6 +1178,7 @@ int rasp_run(rasp_batch* b, uint64_t max_steps) {
   if (!b) return fail(RASP_EINVAL, "batch is NULL");
   if (!b->programs_loaded || !b->inputs_loaded) return fail(RASP_ESTATE, "load programs and inputs before rasp_run");
   CK(apply_uhead_reset(b, b->stream));   // eagerly, outside any captured graph
+  b->uhead_moved = true;
   if (!b->planned) {
     b->planned = true;
     const int rc = replan(b);
@@ -1332,6 +1334,7 @@ int rasp_load_state(rasp_batch* b, uint64_t first, uint64_t count, const rasp_st
   cudaStream_t st = b->stream;
   const DevState& S = b->S;
   CK(apply_uhead_reset(b, st));
+  b->uhead_moved = true;
   if (in->i) CK(cudaMemcpyAsync(S.i + first, in->i, 8 * count, cudaMemcpyHostToDevice, st));
   if (in->a) CK(cudaMemcpyAsync(S.a + first, in->a, 8 * count, cudaMemcpyHostToDevice, st));
   if (in->steps) CK(cudaMemcpyAsync(S.steps + first, in->steps, 8 * count, cudaMemcpyHostToDevice, st));

@@ -609,6 +609,27 @@ def test_new_inputs_of_a_callers_graph(rasp):
             assert_same_state(b.read_state(), oracle_state(wl, threads=8)[0], wl.ell, wl.s, what="new inputs")
 
 
+def test_a_first_run_in_a_callers_graph(rasp):
+    """A graph captured right after the loads does not reset u_0: nothing has
+    moved it since the pack."""
+    import torch
+    side = torch.cuda.Stream()
+    wl = machines(600, 60, 64, seed=232, extra=130)
+    full = oracle_state(wl, threads=8)[0]
+    with torch.cuda.stream(side), rasp.Batch(wl.mem_words, wl.ell, wl.s) as b:
+        b.load_workload(wl)
+        side.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            b.run()
+        for t in (0, 40, 90):
+            if t:
+                b.run(t)
+            g.replay()
+            assert_same_state(b.read_state(), full, wl.ell, wl.s, what="after %d steps" % t)
+            b.reset()
+
+
 def test_new_programs_under_a_callers_graph(rasp):
     """A graph that the caller has captured holds the place of the entries:
     loads that move them, have none or fail leave its replays right."""
