@@ -1055,7 +1055,7 @@ int rasp_load_inputs(rasp_batch* b, const int64_t* tape, const uint64_t* offsets
     const int rc = order_ids(b);
     if (rc) return rc;
   }
-  b->uhead_pending = b->uhead_moved;   // u_0 = 0: by the next pack, or before u_0 is next read
+  b->uhead_pending = b->uhead_moved || b->captured;   // u_0 = 0: by the next pack, or before u_0 is next read
   if (b->captured) CK(apply_uhead_reset(b, st));   // which a replay of a caller's graph would not see
   b->inputs_loaded = true;
   g_err.clear();

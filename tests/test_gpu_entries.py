@@ -628,6 +628,9 @@ def test_a_first_run_in_a_callers_graph(rasp):
             g.replay()
             assert_same_state(b.read_state(), full, wl.ell, wl.s, what="after %d steps" % t)
             b.reset()
+        g.replay()
+        b.load_inputs(wl.tapes, wl.tape_off, wl.caps)
+        assert not b.read_state()["uhead"].any()
 
 
 def test_new_programs_under_a_callers_graph(rasp):
