@@ -148,7 +148,6 @@ struct rasp_batch {
   const uint32_t* graph_pvm = nullptr;
   bool marked = false;
   bool captured = false;       // the caller has captured a run into a graph of its own
-  bool replays = false;        // such a graph may run VMs without keeping codedirty
   bool code_lazy = false;      // slabs of VMs with codedirty = 0 lack their program words (lazy pack)
   bool tuned_block = false;    // autotuned: the SMEM-staged schedule one step at a time
   bool narrow = false;         // M in 4-byte words (w <= 32)
@@ -439,11 +438,12 @@ bool capturing(cudaStream_t st) {
 // not up to date -- another schedule may have written program words, and the
 // plan has changed since -- every VM runs from its memory until the next pack.
 // In a caller's graph the marks are set when it is replayed, so they stay out
-// of date for the runs before that; and a run that keeps no marks may be
-// replayed at any time, so that from then on they are out of date before every
-// run. A graph that runs from entries keeps their place, where a later load may
-// put something else: such a load marks every VM, and so does every pack after
-// it, since a marked VM does not look at its entries.
+// of date for the runs before that. A captured run that keeps no marks sets all
+// of them itself, and so does an eager one where a captured run reads them, for
+// either may be replayed at any time. A graph that runs from entries keeps
+// their place, where a later load may put something else: such a load marks
+// every VM, and so does every pack after it, since a marked VM does not look at
+// its entries.
 cudaError_t settle_dirty(rasp_batch* b, cudaStream_t st, bool captured) {
   bool tracked = false, untracked = false, entries = false;
   for (const Group& g : b->groups) {
@@ -457,11 +457,9 @@ cudaError_t settle_dirty(rasp_batch* b, cudaStream_t st, bool captured) {
     b->graph_fops = b->S.fops;
     b->graph_pvm = b->S.prog_of_vm;
   }
-  b->replays = b->replays || (captured && untracked);
-  if (tracked && (!b->dirty_valid || b->replays)) {
+  if ((tracked && !b->dirty_valid) || (untracked && (captured || b->graph_fops)))
     e = cudaMemsetAsync(b->S.codedirty, 1, b->V, st);
-    b->dirty_valid = !captured;
-  }
+  if (tracked && !captured) b->dirty_valid = true;
   b->ran_untracked = b->ran_untracked || untracked;
   return e;
 }
@@ -848,16 +846,10 @@ cudaError_t decode_entries(rasp_batch* b, uint4* tmp, cudaStream_t st) {
 
 // Entries after a load that did not make them: the plan has come to run from
 // them, or a load for a short run is run again (eagerly, outside any captured
-// graph). While the caller captures the stream nothing can be decoded, and the
-// run captured without entries keeps no marks (see settle_dirty): the batch
-// then stays without them. pay: they are worth making.
+// graph, the caller's included). pay: they are worth making.
 cudaError_t late_entries(rasp_batch* b, cudaStream_t st, bool pay) {
   if (b->S.fops || !b->fuse_at) return cudaSuccess;
-  if (capturing(st)) {
-    b->fuse_at = nullptr;
-    return cudaSuccess;
-  }
-  if (!pay) return cudaSuccess;
+  if (!pay || capturing(st)) return cudaSuccess;
   drop_graphs(b);                              // captured runs hold the old launch arguments
   if (b->ran_untracked) b->dirty_valid = false;   // VMs may have written program words since the pack
   const cudaError_t e = program_bounds(b, nullptr, st);
@@ -960,7 +952,7 @@ int rasp::load_programs(rasp_batch* b, const void* words, int word_size, const u
   if (total)
     look = word_size == 8 ? look_at((const int64_t*)words, offsets, num_programs, b->wmask, owns_code(b))
                           : look_at((const int32_t*)words, offsets, num_programs, b->wmask, owns_code(b));
-  b->fuse_at = look.unfit || b->replays ? nullptr : place_fused(b, total, keep32);
+  b->fuse_at = look.unfit ? nullptr : place_fused(b, total, keep32);
   b->fuse_own = owns_code(b);
   b->self_writing = look.writing;
   b->S.fops = nullptr;

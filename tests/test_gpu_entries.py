@@ -537,7 +537,7 @@ def test_short_runs_in_the_callers_graph(rasp, shared, warm):
                 b.run(1000)
                 assert_same_state(b.read_state(), full, wl.ell, wl.s, what="run on")
                 b.reset()
-            assert b.describe()["entries"] is bool(shared)
+            assert b.describe()["entries"]
 
 
 @pytest.mark.parametrize("w", [64, 32])
@@ -574,6 +574,20 @@ def test_callers_graphs_and_the_marks(rasp, w):
             g.replay()
             b.run()
             assert_same_state(b.read_state(), full, wl.ell, wl.s, what="replayed on the plain schedule, %d" % rep)
+            b.reset()
+        b.close()
+
+        b, k = batch()
+        h = capture(b, 1 << 62)
+        for rep in range(2):
+            b.plan_bucket(k, rasp.SCHED_PLAIN)
+            if rep == 0:
+                b.run(60)
+                g = capture(b, 60)
+            else:
+                g.replay()
+            h.replay()
+            assert_same_state(b.read_state(), full, wl.ell, wl.s, what="entries replayed after the plain schedule")
             b.reset()
         b.close()
 
