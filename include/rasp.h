@@ -255,7 +255,11 @@ int rasp_reset(rasp_batch* b);
  * resumable epochs as in the persistent workers of App. A (Alg. 1). steps is cumulative, so
  * rasp_run(T1) followed by rasp_run(T2) equals rasp_run(T2). A VM that stops
  * on the budget (max_steps < cap) stays RUNNING unless it is a fixed point.
- * Asynchronous on the batch stream. ESTATE before both loads. */
+ * Asynchronous on the batch stream. ESTATE before both loads.
+ * A caller that captures the batch stream may capture this call (its loads
+ * made, a first run done before) and replay it after further loads, resets and
+ * runs; on RASP_SCHED_SHARED such a graph holds the number of programs and the
+ * longest of them, which later loads before a replay must not exceed. */
 int rasp_run(rasp_batch* b, uint64_t max_steps);
 
 /* Wait for the batch stream; EDEVICE if a kernel flagged an internal error. */
